@@ -48,8 +48,9 @@ def listed():
         named("me_ggttggg_fp64_8192", "me", "ggttggg", "fp64", 8192),
         named("me_ggttggg_tc_2049", "me", "ggttggg", "tc", 2049),
         named("me_ggttggg_mixed_65536", "me", "ggttggg", "mixed", 65536),
-        # a generator with its momenta in host memory: copies in and out inside the call
-        named("host_ggttg_mixed_131073", "host", "ggttg", "mixed", 131073),
+        # a generator with its momenta in host memory: copies in and out inside the call (the benchmark's
+        # end-to-end form)
+        named("host_ggttg_fp64_131073", "host", "ggttg", "fp64", 131073),
         # event-level epilogues: helicity and colour choices with the running coupling; channel weights
         named("lhe_ggttgg_32768", "lhe", "ggttgg", "fp64", 32768),
         named("sde_ggttg_65536", "sde", "ggttg", "fp64", 65536),
