@@ -48,7 +48,9 @@ mg_status grow(double** buf, int64_t* cap, int64_t need) {
 // complex multiply-add as 8): mirrors the kernel operation by operation.  One thread per gluon-
 // helicity combination with a good helicity; per thread the gluon currents once, (gamma.J) v per
 // antitop helicity, a depth-first walk of the quark-line prefixes per top helicity, the jamps and
-// the colour sum per good helicity.  mask == NULL means every helicity is good.
+// the colour sum per good helicity.  mask == NULL means every helicity is good.  This counts the
+// algorithm with every good helicity evaluated; the FP64 kernels evaluate one of each pair of flipped
+// helicities (hel_weight) and execute about half of it.
 // warp_simt: the FP32 lane-group kernel's SIMT colour epilogue, which multiplies the full ncol x ncol matrix
 // into the jamps of all four helicities of a slot (4 ncol^2 + 4 ncol each, good or not) instead of the
 // packed triangle per good helicity.  warp: the FP32 lane-group kernel (any epilogue), which for 5 gluons
@@ -191,7 +193,8 @@ mg_status ctx_reserve(mg_ctx* ctx, int64_t nevt, mg_precision precision) {
   const bool tc = (precision == MG_FP64_TCCOLOR || precision == MG_MIXED) && !mixed_in_kernel(ctx, precision);
   int64_t chunk = stride;
   if (tc) {
-    const int64_t per_event = static_cast<int64_t>(ctx->nhel) * ctx->ncol;
+    // (FP64 amplitudes: the jamps of one of each pair of flipped helicities)
+    const int64_t per_event = static_cast<int64_t>(fp32 ? ctx->nhel : ctx->nhel / 2) * ctx->ncol;
     chunk = (int64_t(1) << 29) / per_event / kPage * kPage;
     if (chunk < kPage) chunk = kPage;
     if (chunk > stride) chunk = stride;
@@ -224,7 +227,8 @@ mg_status ctx_copy_mask(mg_ctx* dst, const mg_ctx* src, cudaStream_t st) {
   const bool ok = cp(dst->d_mask, src->d_mask, 4 * sizeof(uint32_t)) && cp(dst->d_good, src->d_good, 128 * sizeof(int)) &&
                   cp(dst->d_ngood, src->d_ngood, sizeof(int)) && cp(dst->d_maxr, src->d_maxr, 128 * sizeof(double)) &&
                   cp(dst->d_gslots, src->d_gslots, 32 * sizeof(int)) && cp(dst->d_ngslots, src->d_ngslots, sizeof(int)) &&
-                  cp(dst->d_nrows, src->d_nrows, sizeof(int));
+                  cp(dst->d_nrows, src->d_nrows, sizeof(int)) && cp(dst->d_hslots, src->d_hslots, 16 * sizeof(int)) &&
+                  cp(dst->d_nhslots, src->d_nhslots, sizeof(int)) && cp(dst->d_nhrows, src->d_nhrows, sizeof(int));
   if (!ok) { cudaGetLastError(); return MG_ECUDA; }
   dst->mask_ready = true;
   return MG_OK;
@@ -351,6 +355,9 @@ void mg_destroy(mg_ctx* ctx) {
   mg::dev_free(ctx->d_ngslots);
   mg::dev_free(ctx->d_allg);
   mg::dev_free(ctx->d_nrows);
+  mg::dev_free(ctx->d_hslots);
+  mg::dev_free(ctx->d_nhslots);
+  mg::dev_free(ctx->d_nhrows);
   mg::dev_free(ctx->d_cmat);
   mg::dev_free(ctx->d_cumma);
   mg::dev_free(ctx->d_tcerr);
@@ -457,13 +464,16 @@ mg_status mg_create(mg_process proc, const mg_params* params, mg_ctx** out) {
       }
     }
     if (mg::dev_alloc(&c->d_gslots, 32 * sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_ngslots, sizeof(int)) != cudaSuccess ||
+        mg::dev_alloc(&c->d_hslots, 16 * sizeof(int)) != cudaSuccess ||
+        mg::dev_alloc(&c->d_nhslots, sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_nhrows, sizeof(int)) != cudaSuccess ||
         mg::dev_alloc(&c->d_allg, 32 * sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_nallg, sizeof(int)) != cudaSuccess) {
       st = MG_ENOMEM;
       break;
     }
     if (cudaMemcpy(c->d_allg, all.data(), ng2 * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->d_nallg, &ng2, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemset(c->d_ngslots, 0, sizeof(int)) != cudaSuccess) {
+        cudaMemset(c->d_ngslots, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->d_nhslots, 0, sizeof(int)) != cudaSuccess ||
+        cudaMemset(c->d_nhrows, 0, sizeof(int)) != cudaSuccess) {
       st = MG_ECUDA;
       break;
     }
@@ -577,7 +587,8 @@ mg_status mg_hel_filter(mg_ctx* ctx, const double* mom_dev, int64_t nevt, void* 
   MG_CUDA(mg::launch_hel_sum(ctx->d_part, ctx->d_nhel, w, stride, 1.0, ctx->d_tot, st));
   MG_CUDA(mg::launch_hel_mask(ctx->d_part, ctx->d_tot, ctx->nhel, w, stride, ctx->prm.hel_tau, ctx->d_maxr,
                               ctx->d_mask, ctx->d_good, ctx->d_ngood, st));
-  MG_CUDA(mg::launch_gluon_slots(ctx->d_mask, ctx->K, ctx->d_gslots, ctx->d_ngslots, ctx->d_nrows, st));
+  MG_CUDA(mg::launch_gluon_slots(ctx->d_mask, ctx->K, ctx->d_gslots, ctx->d_ngslots, ctx->d_nrows, ctx->d_hslots,
+                                 ctx->d_nhslots, ctx->d_nhrows, st));
   ctx->mask_ready = true;
   return MG_OK;
 }
@@ -622,8 +633,14 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
   mg_status s = grow(&ctx->d_part, &ctx->part_cap, stride * ctx->nhel);
   if (s != MG_OK) return s;
   ctx->last = st;
-  const mg::MeConst cst = me_const(ctx);
+  mg::MeConst cst = me_const(ctx);
   const double norm = 1.0 / (256.0 * mg::factorial(ctx->ng));
+  // FP64 amplitudes: one of each pair of flipped helicities (hel_weight)
+  const bool half = (precision == MG_FP64 || precision == MG_FP64_TCCOLOR) && ctx->prm.wt == 0.0;
+  cst.conj = half ? 1 : 0;
+  const int* slots = half ? ctx->d_hslots : ctx->d_gslots;
+  const int* nslots = half ? ctx->d_nhslots : ctx->d_ngslots;
+  const int maxslot = half ? 1 << (ctx->K - 1) : 1 << ctx->K;
   if (tc && !mixed_in_kernel) {
     // amplitudes -> FP32 jamps -> tensor-core colour sums, in chunks of whole pages that keep the jamp
     // buffer within 4 GiB
@@ -631,7 +648,8 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
     const bool warp = fp32 && ctx->shape[precision].warp && mg::me_warp_available(ctx->K, true);
     const bool fused = fp32 && !warp && ctx->shape[precision].fused && ctx->shape[precision].unrolled &&
                        mg::me_static_available(ctx->K, true);
-    const int64_t per_event = static_cast<int64_t>(ctx->nhel) * ctx->ncol;   // float2 per event
+    const int rows = half ? ctx->nhel / 2 : ctx->nhel;                       // jamp rows per event
+    const int64_t per_event = static_cast<int64_t>(rows) * ctx->ncol;        // float2 per event
     int64_t chunk = (int64_t(1) << 29) / per_event;                          // 2^29 float2 = 4 GiB
     chunk = chunk / mg::kPage * mg::kPage;
     if (chunk < mg::kPage) chunk = mg::kPage;
@@ -678,24 +696,27 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
                                    ctx->d_flag, st));
       else if (shared) {
         MG_CUDA(mg::launch_share(ctx->K, ctx->d_prep, n, ctx->d_tab, cst, ctx->d_share, st));
-        MG_CUDA(mg::launch_me_gluonhel(ctx->K, false, false, mom_c, ctx->d_prep, n, ctx->d_tab, ctx->d_gslots, 1 << ctx->K,
-                                       ctx->d_ngslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part,
+        MG_CUDA(mg::launch_me_gluonhel(ctx->K, false, false, mom_c, ctx->d_prep, n, ctx->d_tab, slots, maxslot,
+                                       nslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part,
                                        cst_stride, st, ctx->d_jamps, ctx->shape[precision], nullptr, nullptr, nullptr, 0,
                                        ctx->d_share));
       }
       else
-        MG_CUDA(mg::launch_me_gluonhel(ctx->K, fp32, false, mom_c, ctx->d_prep, n, ctx->d_tab, ctx->d_gslots, 1 << ctx->K,
-                                       ctx->d_ngslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part, cst_stride,
+        MG_CUDA(mg::launch_me_gluonhel(ctx->K, fp32, false, mom_c, ctx->d_prep, n, ctx->d_tab, slots, maxslot,
+                                       nslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part, cst_stride,
                                        st, ctx->d_jamps, ctx->shape[precision], fp32 ? ctx->d_flag : nullptr));
       if (ctx->shape[precision].tc_sync)
-        MG_CUDA(mg::launch_colour_tc(ctx->ncol, ctx->d_jamps, n, ctx->nhel, ctx->d_nrows, ctx->d_cmat, cst.colour_scale,
+        MG_CUDA(mg::launch_colour_tc(ctx->ncol, ctx->d_jamps, n, rows, half ? ctx->d_nhrows : ctx->d_nrows, ctx->d_cmat, cst.colour_scale,
                                      ctx->d_part, cst_stride, st, fp32 ? ctx->d_flag : nullptr));
       else
-        MG_CUDA(mg::launch_colour_umma(ctx->ncol, ctx->d_jamps, n, ctx->nhel, ctx->d_nrows, ctx->d_cumma, cst.colour_scale,
+        MG_CUDA(mg::launch_colour_umma(ctx->ncol, ctx->d_jamps, n, rows, half ? ctx->d_nhrows : ctx->d_nrows, ctx->d_cumma, cst.colour_scale,
                                        ctx->d_part, cst_stride, st, fp32 ? ctx->d_flag : nullptr, ctx->d_tcerr,
                                        ctx->tc_stall));
       if (fp32) MG_CUDA(join_repair(ctx, st));
-      MG_CUDA(mg::launch_hel_sum(ctx->d_part, ctx->d_nrows, n, cst_stride, norm, me_dev + e0, st));
+      if (half)
+        MG_CUDA(mg::launch_hel_sum_rows(ctx->K, ctx->d_part, slots, nslots, ctx->d_mask, n, cst_stride, norm, me_dev + e0, st));
+      else
+        MG_CUDA(mg::launch_hel_sum(ctx->d_part, ctx->d_nrows, n, cst_stride, norm, me_dev + e0, st));
     }
   } else if (ctx->prm.wt == 0.0) {
     const bool fp32 = precision == MG_FP32_AMP || mixed_in_kernel;
@@ -727,7 +748,7 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
         const double* mom_c = mom_dev + (e0 / mg::kPage) * ctx->npar * 4 * mg::kPage;
         MG_CUDA(mg::launch_share(ctx->K, rec_c, n, ctx->d_tab, cst, ctx->d_share, st));
         MG_CUDA(mg::launch_me_gluonhel(ctx->K, false, false, mom_c, const_cast<double*>(rec_c), n, ctx->d_tab,
-                                       ctx->d_gslots, 1 << ctx->K, ctx->d_ngslots, ctx->d_mask, ctx->d_ctri,
+                                       slots, maxslot, nslots, ctx->d_mask, ctx->d_ctri,
                                        ctx->d_ctri_f, cst, ctx->d_part + e0, stride, st, nullptr, ctx->shape[precision],
                                        nullptr, nullptr, nullptr, 0, ctx->d_share));
       }
@@ -739,11 +760,11 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
                                  ctx->d_mask, ctx->d_cfull, ctx->d_cmat, mixed_in_kernel ? 2 : 0, cst, ctx->d_part,
                                  stride, nullptr, ctx->d_flag, st));
     else
-      MG_CUDA(mg::launch_me_gluonhel(ctx->K, fp32, false, mom_dev, ctx->d_prep, nevt, ctx->d_tab, ctx->d_gslots,
-                                     1 << ctx->K, ctx->d_ngslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part,
+      MG_CUDA(mg::launch_me_gluonhel(ctx->K, fp32, false, mom_dev, ctx->d_prep, nevt, ctx->d_tab, slots,
+                                     maxslot, nslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part,
                                      stride, st, nullptr, ctx->shape[precision], fp32 ? ctx->d_flag : nullptr));
     if (fp32) MG_CUDA(join_repair(ctx, st));
-    MG_CUDA(mg::launch_hel_sum(ctx->d_part, ctx->d_ngslots, nevt, stride, norm, me_dev, st));
+    MG_CUDA(mg::launch_hel_sum(ctx->d_part, nslots, nevt, stride, norm, me_dev, st));
   } else {
     MG_CUDA(mg::launch_me_helicity(ctx->K, precision == MG_FP32_AMP, mom_dev, nevt, ctx->d_tab, ctx->d_good, ctx->nhel,
                                    ctx->d_ngood, ctx->d_ctri, cst, ctx->d_part, stride, st));

@@ -14,7 +14,20 @@ struct MeConst {
   double mt, wt;        // top mass and width
   double colour_scale;  // g_s^2 / colour-matrix denominator
   double fp32_tau = 3e-4;  // FP32 modes: events with an internal invariant below fp32_tau * s are redone in FP64
+  // 1: the slots are one of each pair of flipped gluon-helicity combinations (launch_gluon_slots' hslots) and every
+  // helicity h stands for itself and for ~h, |M_h|^2 = |M_~h|^2 (hel_weight); 0: every combination has its own slot
+  int conj = 0;
 };
+
+// How often |M_h|^2 enters the helicity sum.  With zero widths a tree amplitude with every helicity flipped is the
+// complex conjugate (up to a sign common to all colour orderings) of the unflipped one: polarisation vectors and
+// helicity spinors of opposite helicity are conjugates of each other and the vertices and propagators are real.  So
+// |M_h|^2 = |M_~h|^2, colour sum and single diagrams included, and the FP64 kernels evaluate one of the two.
+__host__ __device__ inline int hel_weight(const uint32_t* mask, int h, int npar, int conj) {
+  const int f = (1 << npar) - 1 - h;
+  const int w = static_cast<int>((mask[h >> 5] >> (h & 31)) & 1u);
+  return conj ? w + static_cast<int>((mask[f >> 5] >> (f & 31)) & 1u) : w;
+}
 
 // Launch shape of the matrix-element kernel: a block of kMeThreads threads covers tile_ev events x
 // (kMeThreads / tile_ev) gluon-helicity slots (tile_ev in {32, 64, 128}); slot_major orders the grid so
@@ -128,7 +141,13 @@ void colour_tc_pack(int ncol, const int64_t* num, uint16_t* out_halves);
 cudaError_t launch_colour_tc(int ncol, const float2* jamps, int64_t nevt, int rows_alloc, const int* nrows,
                              const void* cmat, double scale, double* out, int64_t stride, cudaStream_t st,
                              const uint8_t* skip = nullptr);
-cudaError_t launch_gluon_slots(const uint32_t* mask, int K, int* gslots, int* n, int* nrows, cudaStream_t st);
+// gslots: the gluon-helicity combinations with a good helicity (*n of them, *nrows = 4 *n); hslots: those with
+// gluon K-1 of helicity -1 for which the combination or its flip has a good helicity (*nh, *nhrows = 4 *nh).
+cudaError_t launch_gluon_slots(const uint32_t* mask, int K, int* gslots, int* n, int* nrows, int* hslots, int* nh,
+                               int* nhrows, cudaStream_t st);
+// me[e] = norm * sum over the rows of hslots (slot * 4 + 2 top + antitop) of hel_weight * part[row * stride + e]
+cudaError_t launch_hel_sum_rows(int K, const double* part, const int* hslots, const int* nh, const uint32_t* mask,
+                                int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st);
 cudaError_t launch_hel_sum(const double* part, const int* nslot, int64_t nevt, int64_t stride, double norm,
                            double* me, cudaStream_t st);
 cudaError_t launch_hel_mask(const double* part, const double* tot, int nhel, int64_t nevt, int64_t stride, double tau,

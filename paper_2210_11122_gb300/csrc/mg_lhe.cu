@@ -75,15 +75,17 @@ k_lhe_epilogue(const double* __restrict__ part, const double* __restrict__ j2, c
   const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= nevt) return;
   const int nslot = *nslot_dev;
-  int slot_of[1 << K];
+  int slot_of[1 << (K - 1)];
 #pragma unroll
-  for (int g = 0; g < (1 << K); ++g) slot_of[g] = -1;
+  for (int g = 0; g < (1 << (K - 1)); ++g) slot_of[g] = -1;
   for (int s = 0; s < nslot; ++s) slot_of[gslots[s]] = s;
   auto row_of = [&](int h) -> int {
     int gc = 0;
 #pragma unroll
     for (int g = 0; g < K; ++g) gc |= ((h >> (npar - 1 - (g < 2 ? g : g + 2))) & 1) << g;
     const int a = (h >> (npar - 3)) & 1, b = (h >> (npar - 4)) & 1;
+    // the flipped helicity has the same |M_h|^2, in the slot of the flipped combination
+    if (gc >> (K - 1)) return slot_of[(1 << K) - 1 - gc] * 4 + 2 * (1 - a) + (1 - b);
     return slot_of[gc] * 4 + 2 * a + b;
   };
   auto good = [&](int h) -> bool { return (mask[h >> 5] >> (h & 31)) & 1u; };
@@ -214,12 +216,12 @@ mg_status grow_buf(double** buf, int64_t* cap, int64_t need) {
 
 cudaError_t lhe_me(int K, const double* rec, int64_t nevt, const mg_ctx* c, const mg::MeConst& cst, double* part,
                    double* j2, int64_t stride, const double* share, cudaStream_t st) {
-  const int ms = 1 << K;
+  const int ms = 1 << (K - 1);
   switch (K) {
-    case 2: return mg::lhe::launch_lhe_me<2>(rec, nevt, c->d_tab, c->d_gslots, ms, c->d_ngslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
-    case 3: return mg::lhe::launch_lhe_me<3>(rec, nevt, c->d_tab, c->d_gslots, ms, c->d_ngslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
-    case 4: return mg::lhe::launch_lhe_me<4>(rec, nevt, c->d_tab, c->d_gslots, ms, c->d_ngslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
-    case 5: return mg::lhe::launch_lhe_me<5>(rec, nevt, c->d_tab, c->d_gslots, ms, c->d_ngslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
+    case 2: return mg::lhe::launch_lhe_me<2>(rec, nevt, c->d_tab, c->d_hslots, ms, c->d_nhslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
+    case 3: return mg::lhe::launch_lhe_me<3>(rec, nevt, c->d_tab, c->d_hslots, ms, c->d_nhslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
+    case 4: return mg::lhe::launch_lhe_me<4>(rec, nevt, c->d_tab, c->d_hslots, ms, c->d_nhslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
+    case 5: return mg::lhe::launch_lhe_me<5>(rec, nevt, c->d_tab, c->d_hslots, ms, c->d_nhslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -229,10 +231,10 @@ cudaError_t lhe_epilogue(int K, const double* j2, const mg_ctx* c, const double*
                          double* as, cudaStream_t st) {
   const double a0 = c->prm.alphas, mt = c->prm.mt;
   switch (K) {
-    case 2: return mg::lhe::launch_epilogue<2>(c->d_part, j2, c->d_gslots, c->d_ngslots, c->d_mask, mom, nevt, stride, norm, running, a0, mt, rh, rc, me, hel, col, as, st);
-    case 3: return mg::lhe::launch_epilogue<3>(c->d_part, j2, c->d_gslots, c->d_ngslots, c->d_mask, mom, nevt, stride, norm, running, a0, mt, rh, rc, me, hel, col, as, st);
-    case 4: return mg::lhe::launch_epilogue<4>(c->d_part, j2, c->d_gslots, c->d_ngslots, c->d_mask, mom, nevt, stride, norm, running, a0, mt, rh, rc, me, hel, col, as, st);
-    case 5: return mg::lhe::launch_epilogue<5>(c->d_part, j2, c->d_gslots, c->d_ngslots, c->d_mask, mom, nevt, stride, norm, running, a0, mt, rh, rc, me, hel, col, as, st);
+    case 2: return mg::lhe::launch_epilogue<2>(c->d_part, j2, c->d_hslots, c->d_nhslots, c->d_mask, mom, nevt, stride, norm, running, a0, mt, rh, rc, me, hel, col, as, st);
+    case 3: return mg::lhe::launch_epilogue<3>(c->d_part, j2, c->d_hslots, c->d_nhslots, c->d_mask, mom, nevt, stride, norm, running, a0, mt, rh, rc, me, hel, col, as, st);
+    case 4: return mg::lhe::launch_epilogue<4>(c->d_part, j2, c->d_hslots, c->d_nhslots, c->d_mask, mom, nevt, stride, norm, running, a0, mt, rh, rc, me, hel, col, as, st);
+    case 5: return mg::lhe::launch_epilogue<5>(c->d_part, j2, c->d_hslots, c->d_nhslots, c->d_mask, mom, nevt, stride, norm, running, a0, mt, rh, rc, me, hel, col, as, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -257,7 +259,7 @@ mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, cons
   ctx->last = st;
   const int K = ctx->K;
   // chunks of whole pages that keep the per-slot jamp-square sums within 2^27 doubles (1 GiB)
-  const int64_t per_event = static_cast<int64_t>(1 << K) * ctx->ncol;
+  const int64_t per_event = static_cast<int64_t>(1 << (K - 1)) * ctx->ncol;
   int64_t chunk = (int64_t(1) << 27) / per_event / mg::kPage * mg::kPage;
   const int64_t stride_all = pad_page(nevt);
   if (chunk < mg::kPage) chunk = mg::kPage;
@@ -277,6 +279,7 @@ mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, cons
   cst.gs = std::sqrt(4.0 * 3.14159265358979323846 * ctx->prm.alphas);
   cst.mt = ctx->prm.mt;
   cst.wt = ctx->prm.wt;
+  cst.conj = 1;   // one of each pair of flipped helicities
   cst.colour_scale = cst.gs * cst.gs / static_cast<double>(ctx->colour_den);
   const double norm = 1.0 / (256.0 * mg::factorial(ctx->ng));
   for (int64_t e0 = 0; e0 < nevt; e0 += chunk) {

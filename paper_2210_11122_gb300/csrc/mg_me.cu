@@ -387,6 +387,27 @@ __global__ void k_hel_sum(const double* __restrict__ part, const int* __restrict
   me[e] = s * norm;
 }
 
+// me[e] = norm * sum over the rows (slot * 4 + 2 top + antitop) of one of each pair of flipped helicities
+__global__ void k_hel_sum_rows(int K, const double* __restrict__ part, const int* __restrict__ hslots,
+                               const int* __restrict__ nh_dev, const uint32_t* __restrict__ mask, int64_t nevt,
+                               int64_t stride, double norm, double* __restrict__ me) {
+  const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (e >= nevt) return;
+  const int nh = *nh_dev, npar = K + 2;
+  double s = 0.0;
+  for (int k = 0; k < nh; ++k) {
+    const int gc = hslots[k];
+    int hb = 0;
+    for (int g = 0; g < K; ++g)
+      if ((gc >> g) & 1) hb |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
+    for (int t = 0; t < 4; ++t) {
+      const int h = hb | ((t >> 1) << (npar - 3)) | ((t & 1) << (npar - 4));
+      s = fma(static_cast<double>(hel_weight(mask, h, npar, 1)), part[(4 * k + t) * stride + e], s);
+    }
+  }
+  me[e] = s * norm;
+}
+
 // helicity filter, step 1: maxr[h] = max over the warm-up events of part[h][e] / tot[e]
 // (one block per helicity, fixed-shape tree reduction: order-independent maximum).
 __global__ void k_hel_ratio_max(const double* __restrict__ part, const double* __restrict__ tot, int64_t nevt,
@@ -455,6 +476,15 @@ cudaError_t launch_hel_sum(const double* part, const int* nslot, int64_t nevt, i
   const unsigned blocks = static_cast<unsigned>((nevt + threads - 1) / threads);
   if (blocks == 0) return cudaSuccess;
   { k_hel_sum<<<blocks, threads, 0, st>>>(part, nslot, nevt, stride, norm, me); mg::note_launch(); }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_hel_sum_rows(int K, const double* part, const int* hslots, const int* nh, const uint32_t* mask,
+                                int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st) {
+  const int threads = 256;
+  const unsigned blocks = static_cast<unsigned>((nevt + threads - 1) / threads);
+  if (blocks == 0) return cudaSuccess;
+  { k_hel_sum_rows<<<blocks, threads, 0, st>>>(K, part, hslots, nh, mask, nevt, stride, norm, me); mg::note_launch(); }
   return cudaGetLastError();
 }
 

@@ -22,16 +22,16 @@ __device__ __forceinline__ P* share_event(P* share, int64_t e, int stride) {
 }
 
 // JOUT: instead of colour sums, write the jamps of every helicity of the slot as FP32 complex
-// numbers to jout[((e * 4 * 2^K) + slot * 4 + 2 * top + antitop) * ncol + sigma] (zeros for helicities
-// outside the mask), for the tensor-core colour sum.
+// numbers to jout[(e * rows + slot * 4 + 2 * top + antitop) * ncol + sigma] (zeros for helicities of weight 0),
+// for the tensor-core colour sum; rows = 4 * 2^K jamp rows per event, half of them with cst.conj.
 // SHARED (FP64 with a per-event record): the gluon currents of fewer than all gluons and their (gamma.J) v
 // are not computed here but read from share where they are used (not copied into the thread's local
 // memory), where k_share_level left them once per helicity assignment of their own gluons (item
 // tab->share_base[s] + helicity bits of s's gluons, 24 doubles: J, then (gamma.J) v for both antitop
 // helicities; page-interleaved, share_event); likewise the quark-line prefixes of k_prefix_level.
 // LHE (FP64 with a per-event record, for the event-level epilogues): the colour sum of every helicity of
-// the slot in its own row, out[(slot * 4 + 2 top + antitop) * stride + e] (zero for helicities outside
-// the mask), and the slot's sum over its good helicities of every |jamp|^2,
+// the slot in its own row, out[(slot * 4 + 2 top + antitop) * stride + e] (unweighted; zero for helicities of
+// weight 0), and the slot's weighted sum over its helicities of every |jamp|^2,
 // j2[(slot * ncol + sigma) * stride + e].
 // The work of one thread: event e, gluon-helicity slot `slot` with gluon helicities gc (bit g = helicity +1
 // of gluon g).  Called by k_me_gluonhel below and by the persistent multi-process kernel (mg_persist.cu).
@@ -206,17 +206,19 @@ __device__ __forceinline__ void me_slot(const double* __restrict__ mom, const T*
     if ((gc >> g) & 1) hbase |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
   const int bit_t = 1 << (npar - 3), bit_tb = 1 << (npar - 4);
 
+  const int nrow = (4 << K) >> cst.conj;   // jamp rows per event
   double total = 0.0;
   double jsum[LHE ? NCOL : 1];
   if constexpr (LHE)
     for (int c = 0; c < NCOL; ++c) jsum[c] = 0.0;
   for (int a = 0; a < 2; ++a) {
     const int h0 = hbase | (a ? bit_t : 0), h1 = h0 | bit_tb;
-    const bool good0 = PER_HEL || ((mask[h0 >> 5] >> (h0 & 31)) & 1u);
-    const bool good1 = PER_HEL || ((mask[h1 >> 5] >> (h1 & 31)) & 1u);
+    // cst.conj: the number of good helicities h0 (h1) stands for, 0, 1 or 2
+    const int w0 = PER_HEL ? 1 : hel_weight(mask, h0, npar, cst.conj), w1 = PER_HEL ? 1 : hel_weight(mask, h1, npar, cst.conj);
+    const bool good0 = w0 > 0, good1 = w1 > 0;
     if (!good0 && !good1) {
       if (JOUT) {
-        float2* row = jout + (e * (4 << K) + slot * 4 + 2 * a) * NCOL;
+        float2* row = jout + (e * nrow + slot * 4 + 2 * a) * NCOL;
         for (int c = 0; c < 2 * NCOL; ++c) row[c] = make_float2(0.f, 0.f);
       }
       if (LHE) {
@@ -303,7 +305,7 @@ __device__ __forceinline__ void me_slot(const double* __restrict__ mom, const T*
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
         const bool good = b ? good1 : good0;
-        float2* row = jout + (e * (4 << K) + slot * 4 + 2 * a + b) * NCOL;
+        float2* row = jout + (e * nrow + slot * 4 + 2 * a + b) * NCOL;
         for (int c = 0; c < NCOL; ++c)
           row[c] = good ? make_float2(static_cast<float>(A[b][c].r), static_cast<float>(A[b][c].i)) : make_float2(0.f, 0.f);
       }
@@ -324,9 +326,11 @@ __device__ __forceinline__ void me_slot(const double* __restrict__ mom, const T*
           v = static_cast<double>(colour_sum<NCOL, T>(A[b], ctri)) * cst.colour_scale;
         if (PER_HEL) out[h * stride + e] = v;
         else if (LHE) out[(slot * 4 + 2 * a + b) * stride + e] = v;
-        else total += v;
-        if constexpr (LHE)
-          for (int c = 0; c < NCOL; ++c) jsum[c] = fma(A[b][c].r, A[b][c].r, fma(A[b][c].i, A[b][c].i, jsum[c]));
+        else total += (b ? w1 : w0) > 1 ? v + v : v;
+        if constexpr (LHE) {
+          const double w = static_cast<double>(b ? w1 : w0);
+          for (int c = 0; c < NCOL; ++c) jsum[c] = fma(w, fma(A[b][c].r, A[b][c].r, A[b][c].i * A[b][c].i), jsum[c]);
+        }
       }
     }
   }
@@ -425,6 +429,7 @@ k_share_level(const double* __restrict__ rec, int64_t nevt, const Tables* __rest
   const int s = s0 + (j >> level), h = j & ((1 << level) - 1);
   const int msk = tab->seq_mask[s];
   const int gc = pdep_bits(h, msk);
+  if (gc >> (K - 1)) return;   // the slots have gluon K-1 of helicity -1 (launch_gluon_slots' hslots)
   const double* in = rec + (e / kPage) * L::NITEM * kPage + (e % kPage);
   auto ld = [&](int item) -> double { return __ldg(in + item * kPage); };
   double* sh = share_event(share, e, tab->share_stride);
@@ -519,6 +524,7 @@ k_prefix_level(const double* __restrict__ rec, int64_t nevt, const Tables* __res
   int gcp = 0;   // the prefix gluons' helicity bits, by gluon
 #pragma unroll
   for (int j = 0; j < m; ++j) gcp |= ((h >> j) & 1) << tab->perm[c0][j];
+  if (gcp >> (K - 1)) return;   // (as k_share_level)
   Slash<double> g[m];
 #pragma unroll
   for (int j = 0; j < m; ++j) {

@@ -71,10 +71,11 @@ extern "C" mg_status mg_sigmakin_noalloc(mg_ctx* ctx, const double* mom_dev, int
   const double norm = 1.0 / (256.0 * mg::factorial(ctx->ng));
   // every element the sum kernel reads (good slots x events) is written first: nothing to clear
   if (ctx->prm.wt == 0.0) {
-    if (mg::launch_me_gluonhel(ctx->K, false, false, mom_dev, nullptr, nevt, ctx->d_tab, ctx->d_gslots, 1 << ctx->K,
-                               ctx->d_ngslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, scratch, stride, st) != cudaSuccess)
+    cst.conj = 1;   // one of each pair of flipped helicities
+    if (mg::launch_me_gluonhel(ctx->K, false, false, mom_dev, nullptr, nevt, ctx->d_tab, ctx->d_hslots,
+                               1 << (ctx->K - 1), ctx->d_nhslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, scratch, stride, st) != cudaSuccess)
       return MG_ECUDA;
-    if (mg::launch_hel_sum(scratch, ctx->d_ngslots, nevt, stride, norm, me_dev, st) != cudaSuccess) return MG_ECUDA;
+    if (mg::launch_hel_sum(scratch, ctx->d_nhslots, nevt, stride, norm, me_dev, st) != cudaSuccess) return MG_ECUDA;
   } else {
     if (mg::launch_me_helicity(ctx->K, false, mom_dev, nevt, ctx->d_tab, ctx->d_good, ctx->nhel, ctx->d_ngood,
                                ctx->d_ctri, cst, scratch, stride, st) != cudaSuccess)

@@ -32,7 +32,7 @@ constexpr int kTileEv = 128;
 struct PJob {
   const double* rec;        // per-event FP64 record
   const Tables* tab;
-  const int* gslots;        // gluon-helicity combinations with a good helicity
+  const int* gslots;        // gluon-helicity combinations (one of each flipped pair) with a good helicity
   const int* nslot;
   const uint32_t* mask;
   const double* ctri;
@@ -167,6 +167,7 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     cst.gs = std::sqrt(4.0 * 3.14159265358979323846 * c->prm.alphas);
     cst.mt = c->prm.mt;
     cst.wt = c->prm.wt;
+    cst.conj = 1;   // one of each pair of flipped helicities
     cst.colour_scale = cst.gs * cst.gs / static_cast<double>(c->colour_den);
     if (mg::launch_event_prep(c->K, false, j.mom_dev, j.nevt, cst, c->d_prep, st) != cudaSuccess) { s = MG_ECUDA; break; }
     // the job's currents and quark-line prefixes shared between its gluon-helicity combinations, where its
@@ -183,8 +184,8 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     p.share = share;
     p.rec = c->d_prep;
     p.tab = c->d_tab;
-    p.gslots = c->d_gslots;
-    p.nslot = c->d_ngslots;
+    p.gslots = c->d_hslots;
+    p.nslot = c->d_nhslots;
     p.mask = c->d_mask;
     p.ctri = c->d_ctri;
     p.part = c->d_part;
@@ -194,7 +195,7 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     p.ntile_ev = static_cast<int>((j.nevt + mg::pers::kTileEv - 1) / mg::pers::kTileEv);
     p.tile0 = batch->ntiles;
     p.cst = cst;
-    batch->ntiles += static_cast<int64_t>(p.ntile_ev) << c->K;   // every possible slot; absent ones exit at once
+    batch->ntiles += static_cast<int64_t>(p.ntile_ev) << (c->K - 1);   // every possible slot; absent ones exit at once
   }
   if (s == MG_OK && batch->njobs > 0) {
     // the tile counter of the costliest job's context (a context's work is ordered on one stream at a time)
@@ -217,7 +218,7 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
       const mg_batch_job& j = jobs[i];
       if (j.nevt == 0) continue;
       const double norm = 1.0 / (256.0 * mg::factorial(j.ctx->ng));
-      if (mg::launch_hel_sum(j.ctx->d_part, j.ctx->d_ngslots, j.nevt, pad_pg(j.nevt), norm, j.me_dev, st) != cudaSuccess)
+      if (mg::launch_hel_sum(j.ctx->d_part, j.ctx->d_nhslots, j.nevt, pad_pg(j.nevt), norm, j.me_dev, st) != cudaSuccess)
         s = MG_ECUDA;
     }
   }

@@ -12,7 +12,7 @@
 //     before parents) and a depth-first walk over the ordered lists of trees that partition the gluons
 //     (a "push" attaches a tree and propagates the spinor, a "leaf" closes a diagram with the antitop):
 //     3 / 15 / 105 / 945 channels;
-//   * device: one thread per (event, gluon-helicity combination) builds every tree current once (the
+//   * device: one thread per (event, gluon-helicity combination; one of each flipped pair) builds every tree current once (the
 //     gluon helicities fixed) and walks the list for each top helicity, the spinor prefixes on a stack,
 //     adding |A_d|^2 of each good helicity into per-channel sums; a second kernel adds the combinations
 //     and normalises per event.
@@ -196,8 +196,9 @@ __global__ void __launch_bounds__(128) k_sde(const double* __restrict__ rec, int
   for (int d = 0; d < NCH; ++d) acc[d] = 0.0;
   for (int a = 0; a < 2; ++a) {
     const int h0 = hbase | (a << (npar - 3)), h1 = h0 | (1 << (npar - 4));
-    const bool good0 = (mask[h0 >> 5] >> (h0 & 31)) & 1u, good1 = (mask[h1 >> 5] >> (h1 & 31)) & 1u;
-    if (!good0 && !good1) continue;
+    // a single diagram's |A_d|^2 is the same with every helicity flipped too (hel_weight)
+    const double w0 = hel_weight(mask, h0, npar, 1), w1 = hel_weight(mask, h1, npar, 1);
+    if (w0 == 0.0 && w1 == 0.0) continue;
     cx<double> stk[K][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) stk[0][q] = ub[a][q];
@@ -209,10 +210,7 @@ __global__ void __launch_bounds__(128) k_sde(const double* __restrict__ rec, int
         cx<double> a0 = {0.0, 0.0}, a1 = {0.0, 0.0};
         v2::sdot_acc(a0, t, vv[0], false);
         v2::sdot_acc(a1, t, vv[1], false);
-        double s = 0.0;
-        if (good0) s = fma(a0.r, a0.r, fma(a0.i, a0.i, s));
-        if (good1) s = fma(a1.r, a1.r, fma(a1.i, a1.i, s));
-        acc[ch] += s;
+        acc[ch] += fma(w0, fma(a0.r, a0.r, a0.i * a0.i), w1 * fma(a1.r, a1.r, a1.i * a1.i));
       } else {
         v2::row_prop(t, qc[tab->op_mask[i]], stk[dep + 1]);
       }
@@ -262,8 +260,8 @@ mg_status growb(double** buf, int64_t* cap, int64_t need) {
 template <int K>
 cudaError_t launch_sde(const double* rec, int64_t n, const mg::sde::Tab* tab, const mg_ctx* c, double* part, int64_t stride,
                        cudaStream_t st) {
-  const dim3 grid(static_cast<unsigned>((n + 127) / 128), static_cast<unsigned>(1 << K));
-  mg::sde::k_sde<K><<<grid, 128, 0, st>>>(rec, n, tab, c->d_gslots, c->d_ngslots, c->d_mask, part, stride);
+  const dim3 grid(static_cast<unsigned>((n + 127) / 128), static_cast<unsigned>(1 << (K - 1)));
+  mg::sde::k_sde<K><<<grid, 128, 0, st>>>(rec, n, tab, c->d_hslots, c->d_nhslots, c->d_mask, part, stride);
   mg::note_launch();
   return cudaGetLastError();
 }
@@ -308,7 +306,7 @@ mg_status mg_sde_weights(mg_ctx* ctx, const double* mom_dev, int64_t nevt, doubl
   }
   ctx->last = st;
   // chunks of whole pages that keep the per-slot channel sums within 2^28 doubles (2 GiB)
-  const int64_t per_event = static_cast<int64_t>(1 << K) * b.tab.nch;
+  const int64_t per_event = static_cast<int64_t>(1 << (K - 1)) * b.tab.nch;
   int64_t chunk = (int64_t(1) << 28) / per_event / mg::kPage * mg::kPage;
   if (chunk < mg::kPage) chunk = mg::kPage;
   if (chunk > padp(nevt)) chunk = padp(nevt);
@@ -335,7 +333,7 @@ mg_status mg_sde_weights(mg_ctx* ctx, const double* mom_dev, int64_t nevt, doubl
     }
     if (e != cudaSuccess) return MG_ECUDA;
     mg::sde::k_sde_norm<<<static_cast<unsigned>((n + 127) / 128), 128, 0, st>>>(ctx->d_sde, n, stride, b.tab.nch,
-                                                                               ctx->d_ngslots, w_dev + e0, nevt);
+                                                                               ctx->d_nhslots, w_dev + e0, nevt);
     mg::note_launch();
     if (cudaGetLastError() != cudaSuccess) return MG_ECUDA;
   }
