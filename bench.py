@@ -423,9 +423,9 @@ class Leg:
             traffic = profiled_traffic([os.path.join(csrc, f) for f in ME_SOURCES], prof, nev) if prof else None
             shared = self.shapes[name]["shared"]
             K = self.ng + 2
-            slot_kernel = ("k_me_gluonhel_occ<%d>" % K) if (K >= 4 or (K == 3 and shared)) else ("k_me_gluonhel<%d,double>" % K)
+            slot_kernel = "k_me_gluonhel2" if K == 2 else "k_me64<%d>" % K
             kernel = ("k_event_prep + %s%s + k_hel_sum (one mg_sigmakin call)"
-                      % ("k_share_level (per sequence length) + k_prefix_level (per prefix length) + " if shared else "", slot_kernel))
+                      % ("k_pass64 (per pass) + " if shared and K >= 3 else "", slot_kernel))
             return fp64_roofline(amp + col, oracle_flops, nev, me_ms, p64, traffic, kernel)
         if precision == mg.MG_FP64_TCCOLOR:
             return time_roofline([("fp64", amp * nev, p64, src64),

@@ -299,10 +299,11 @@ mg_status mg_colour_flow(mg_process proc, int flow, int* order);
  *                       the tensor cores itself, unless
  *   MG_LAUNCH_TC_APART  MG_MIXED with MG_LAUNCH_WARP: write the jamps out for the separate tensor-core
  *                       colour kernel instead;
- *   MG_LAUNCH_SHARED    MG_FP64: the gluon currents of fewer than all gluons (and their products with the
- *                       antitop spinors) are computed once per helicity assignment of their own gluons, by
- *                       a pass before the matrix-element kernel, instead of once per gluon-helicity
- *                       combination;
+ *   MG_LAUNCH_SHARED    MG_FP64, from gg -> t tbar g on: everything that depends on fewer than all gluons
+ *                       (their currents, the quark line's row and column spinors and their products) is
+ *                       computed once per helicity assignment of those gluons, by a few passes before the
+ *                       matrix-element kernel, instead of once per gluon-helicity combination (the same
+ *                       bits);
  *   MG_LAUNCH_TC_SYNC   the separate tensor-core colour pass (MG_FP64_TCCOLOR, and MG_MIXED where the jamps
  *                       are written out) on warp-level mma.sync instead of the default fifth-generation
  *                       tensor-core kernel (tcgen05.mma with the accumulators in tensor memory). */

@@ -81,9 +81,9 @@ void flop_model(const mg::Tables& t, const uint32_t* mask, bool fp32, bool share
       per_slot += 2.0 * gamma_col * t.nseq;
   }
   // shared (FP64): the quark-line prefixes of lengths 1 .. pref_levels once per helicity assignment of
-  // their gluons and top helicity per event (k_prefix_level: both top helicities share each current's
+  // their gluons and top helicity per event (both top helicities share each current's
   // gamma.J entries, the 8 additions of row_gamma), the longer ones in the slot's walk
-  const int plev = shared ? t.pref_levels : 0;
+  const int plev = shared ? (K - 1 < 3 ? K - 1 : 3) : 0;
   for (int m = 1; m <= plev; ++m) {
     int orderings = 1;
     for (int i = 0; i < m; ++i) orderings *= K - i;
@@ -169,11 +169,27 @@ cudaError_t free_raw(void* p, bool host) {
   return host ? cudaFreeHost(p) : cudaFree(p);
 }
 
+int64_t share_doubles(int K) { return K >= 3 ? tab64_host(K).stride : 0; }
+
 int64_t share_chunk(int K, int64_t stride) {
   const int64_t per_event = share_doubles(K);   // doubles
+  if (per_event == 0) return stride;
   int64_t chunk = (int64_t(1) << 28) / per_event / kPage * kPage;       // 2^28 doubles = 2 GiB
   if (chunk < kPage) chunk = kPage;
   return chunk < stride ? chunk : stride;
+}
+
+cudaError_t fp64_slots(mg_ctx* ctx, const double* mom, const double* rec, int64_t n, bool shared, const MeConst& cst,
+                       double* out, int64_t stride, float2* jout, MeShape shape, cudaStream_t st) {
+  if (ctx->K == 2)
+    return launch_me_gluonhel(2, false, false, mom, const_cast<double*>(rec), n, ctx->d_tab, ctx->d_hslots, 2,
+                              ctx->d_nhslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, out, stride, st, jout, shape);
+  if (shared) {
+    const cudaError_t e = launch_pass64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, cst, ctx->d_share, st);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_me64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, ctx->d_hslots, ctx->d_nhslots, ctx->d_mask, ctx->d_ctri, cst,
+                     out, stride, jout, shape, shared ? ctx->d_share : nullptr, nullptr, st);
 }
 
 bool mixed_in_kernel(const mg_ctx* ctx, mg_precision precision) {
@@ -342,6 +358,7 @@ void mg_destroy(mg_ctx* ctx) {
   if (!ctx) return;
   cudaDeviceSynchronize();
   mg::dev_free(ctx->d_tab);
+  mg::dev_free(ctx->d_tab64);
   mg::dev_free(ctx->d_ctri);
   mg::dev_free(ctx->d_ctri_f);
   mg::dev_free(ctx->d_cfull);
@@ -417,6 +434,10 @@ mg_status mg_create(mg_process proc, const mg_params* params, mg_ctx** out) {
     cudaError_t e = mg::dev_alloc(&c->d_tab, sizeof(mg::Tables));
     if (e == cudaSuccess) e = cudaMemcpy(c->d_tab, t, sizeof(mg::Tables), cudaMemcpyHostToDevice);
     delete t;
+    if (e == cudaSuccess && c->K >= 3) {
+      e = mg::dev_alloc(&c->d_tab64, sizeof(mg::Tab64));
+      if (e == cudaSuccess) e = cudaMemcpy(c->d_tab64, &mg::tab64_host(c->K), sizeof(mg::Tab64), cudaMemcpyHostToDevice);
+    }
     if (e != cudaSuccess) { st = e == cudaErrorMemoryAllocation ? MG_ENOMEM : MG_ECUDA; break; }
     std::vector<int64_t> num;
     mg::colour_matrix_exact(c->K, num, c->colour_den);
@@ -655,7 +676,7 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
     if (chunk < mg::kPage) chunk = mg::kPage;
     if (chunk > stride) chunk = stride;
     // FP64 amplitudes: optionally the currents shared between gluon-helicity combinations (as MG_FP64)
-    const bool shared = !fp32 && ctx->shape[precision].shared;
+    const bool shared = !fp32 && ctx->shape[precision].shared && ctx->K >= 3;
     if (shared) {
       const int64_t sc = mg::share_chunk(ctx->K, stride);
       if (sc < chunk) chunk = sc;
@@ -694,17 +715,13 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
         MG_CUDA(mg::launch_me_warp(ctx->K, ctx->d_prep, n, ctx->d_tab, ctx->d_gslots, 1 << ctx->K, ctx->d_ngslots,
                                    ctx->d_mask, ctx->d_cfull, ctx->d_cmat, 1, cst, ctx->d_part, cst_stride, ctx->d_jamps,
                                    ctx->d_flag, st));
-      else if (shared) {
-        MG_CUDA(mg::launch_share(ctx->K, ctx->d_prep, n, ctx->d_tab, cst, ctx->d_share, st));
-        MG_CUDA(mg::launch_me_gluonhel(ctx->K, false, false, mom_c, ctx->d_prep, n, ctx->d_tab, slots, maxslot,
-                                       nslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part,
-                                       cst_stride, st, ctx->d_jamps, ctx->shape[precision], nullptr, nullptr, nullptr, 0,
-                                       ctx->d_share));
-      }
+      else if (!fp32)
+        MG_CUDA(mg::fp64_slots(ctx, mom_c, ctx->d_prep, n, shared, cst, ctx->d_part, cst_stride, ctx->d_jamps,
+                               ctx->shape[precision], st));
       else
-        MG_CUDA(mg::launch_me_gluonhel(ctx->K, fp32, false, mom_c, ctx->d_prep, n, ctx->d_tab, slots, maxslot,
-                                       nslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part, cst_stride,
-                                       st, ctx->d_jamps, ctx->shape[precision], fp32 ? ctx->d_flag : nullptr));
+        MG_CUDA(mg::launch_me_gluonhel(ctx->K, true, false, mom_c, ctx->d_prep, n, ctx->d_tab, slots, maxslot, nslots,
+                                       ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part, cst_stride, st,
+                                       ctx->d_jamps, ctx->shape[precision], ctx->d_flag));
       if (ctx->shape[precision].tc_sync)
         MG_CUDA(mg::launch_colour_tc(ctx->ncol, ctx->d_jamps, n, rows, half ? ctx->d_nhrows : ctx->d_nrows, ctx->d_cmat, cst.colour_scale,
                                      ctx->d_part, cst_stride, st, fp32 ? ctx->d_flag : nullptr));
@@ -734,23 +751,18 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
     // events with a small internal invariant: recomputed with double-float or FP64 amplitudes (per-slot
     // layout) on the side stream
     if (fp32) MG_CUDA(fork_repair(ctx, mom_dev, nevt, cst, stride, 0, ctx->shape[precision].df_redo, st));
-    const bool shared = !fp32 && ctx->shape[precision].shared;
-    if (shared) {
-      // FP64: the currents of fewer than all gluons once per helicity assignment of their gluons, then
-      // the matrix elements reading them; in chunks of events that bound the scratch
-      const int64_t chunk = mg::share_chunk(ctx->K, stride);
-      s = grow(&ctx->d_share, &ctx->share_cap, chunk * mg::share_doubles(ctx->K));
+    const bool shared = !fp32 && ctx->shape[precision].shared && ctx->K >= 3;
+    if (!fp32) {
+      // with shared items, in chunks of events that bound their buffer
+      const int64_t chunk = shared ? mg::share_chunk(ctx->K, stride) : stride;
+      if (shared) s = grow(&ctx->d_share, &ctx->share_cap, chunk * mg::share_doubles(ctx->K));
       if (s != MG_OK) return s;
       const int64_t nitem = mg::event_record_bytes(ctx->K, false) / 8;
       for (int64_t e0 = 0; e0 < nevt; e0 += chunk) {
         const int64_t n = nevt - e0 < chunk ? nevt - e0 : chunk;
-        const double* rec_c = ctx->d_prep + (e0 / mg::kPage) * nitem * mg::kPage;
-        const double* mom_c = mom_dev + (e0 / mg::kPage) * ctx->npar * 4 * mg::kPage;
-        MG_CUDA(mg::launch_share(ctx->K, rec_c, n, ctx->d_tab, cst, ctx->d_share, st));
-        MG_CUDA(mg::launch_me_gluonhel(ctx->K, false, false, mom_c, const_cast<double*>(rec_c), n, ctx->d_tab,
-                                       slots, maxslot, nslots, ctx->d_mask, ctx->d_ctri,
-                                       ctx->d_ctri_f, cst, ctx->d_part + e0, stride, st, nullptr, ctx->shape[precision],
-                                       nullptr, nullptr, nullptr, 0, ctx->d_share));
+        MG_CUDA(mg::fp64_slots(ctx, mom_dev + (e0 / mg::kPage) * ctx->npar * 4 * mg::kPage,
+                               ctx->d_prep + (e0 / mg::kPage) * nitem * mg::kPage, n, shared, cst, ctx->d_part + e0, stride,
+                               nullptr, ctx->shape[precision], st));
       }
     } else if (fused)
       MG_CUDA(mg::launch_me_fused(ctx->K, true, mom_dev, nevt, ctx->d_gslots, ctx->d_ngslots, ctx->d_mask, cst,
@@ -760,9 +772,9 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
                                  ctx->d_mask, ctx->d_cfull, ctx->d_cmat, mixed_in_kernel ? 2 : 0, cst, ctx->d_part,
                                  stride, nullptr, ctx->d_flag, st));
     else
-      MG_CUDA(mg::launch_me_gluonhel(ctx->K, fp32, false, mom_dev, ctx->d_prep, nevt, ctx->d_tab, slots,
+      MG_CUDA(mg::launch_me_gluonhel(ctx->K, true, false, mom_dev, ctx->d_prep, nevt, ctx->d_tab, slots,
                                      maxslot, nslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part,
-                                     stride, st, nullptr, ctx->shape[precision], fp32 ? ctx->d_flag : nullptr));
+                                     stride, st, nullptr, ctx->shape[precision], ctx->d_flag));
     if (fp32) MG_CUDA(join_repair(ctx, st));
     MG_CUDA(mg::launch_hel_sum(ctx->d_part, nslots, nevt, stride, norm, me_dev, st));
   } else {

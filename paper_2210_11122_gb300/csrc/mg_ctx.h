@@ -51,7 +51,8 @@ struct mg_ctx {
   void* d_sdetab = nullptr;    // mg_sde_weights: trees and walk of the channels (uploaded on first use)
   double* d_sde = nullptr;     // per-slot channel sums (one chunk of events)
   int64_t sde_cap = 0;         // in doubles
-  double* d_share = nullptr;   // FP64: currents shared between gluon-helicity combinations (one chunk of events)
+  mg::Tab64* d_tab64 = nullptr;   // FP64 matrix elements of 3 to 5 gluons: items, tasks and terms
+  double* d_share = nullptr;   // FP64: items shared between gluon-helicity combinations (one chunk of events)
   int64_t share_cap = 0;      // in doubles
   cudaStream_t side = nullptr;         // FP32 modes: the FP64 recomputation runs here, beside the FP32 launches
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -74,8 +75,15 @@ struct mg_ctx {
 
 
 namespace mg {
-// events per chunk of the FP64 shared-current path (its scratch stays within 2 GiB)
+// doubles per event of the items shared between FP64 gluon-helicity combinations (0 for 2 gluons: none are), and
+// events per chunk (the buffer stays within 2 GiB)
+int64_t share_doubles(int K);
 int64_t share_chunk(int K, int64_t stride);
+// FP64 amplitudes of n events (from a page boundary: momenta mom, FP64 records rec; zero top width) for the context's
+// half list of gluon-helicity combinations: colour sums or jamps as launch_me64.  shared: through the items buffer
+// (d_share, share_doubles(K) * pad(n) doubles, 3 to 5 gluons), else every combination on its own.
+cudaError_t fp64_slots(mg_ctx* ctx, const double* mom, const double* rec, int64_t n, bool shared, const MeConst& cst,
+                       double* out, int64_t stride, float2* jout, MeShape shape, cudaStream_t st);
 // MG_MIXED on the lane-group kernel: colour sums on the tensor cores inside it, per-slot outputs
 bool mixed_in_kernel(const mg_ctx* ctx, mg_precision precision);
 mg_status ctx_reserve(mg_ctx* ctx, int64_t nevt, mg_precision precision);

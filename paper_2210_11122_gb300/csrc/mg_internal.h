@@ -53,20 +53,6 @@ struct Tables {
   int16_t full_v4[kMaxNcol / 2][6][3];
   uint8_t full_nv3[kMaxNcol / 2], full_nv4[kMaxNcol / 2];
   uint8_t full_split_mask[kMaxNcol / 2][kMaxGluons - 1];   // mask of the left part of each V3 split
-  // currents shared between gluon-helicity combinations: canonical sequence s with the helicities of its
-  // own gluons h (2^len(s) of them) is item share_base[s] + h; share_n items per event
-  int16_t share_base[kMaxSeq];
-  int share_n;
-  // quark-line prefixes shared the same way: the row spinor after the first m gluons of a colour ordering
-  // (m = 1 .. pref_levels), for every helicity assignment of those gluons and both top helicities.
-  // Level m's node (p, h, a) -- p = ordering / (K - m)!, h = the prefix gluons' helicities in ordering
-  // order (bit j: gluon perm[.][j]), a = top helicity -- is item pref_off[m] + ((p << m | h) << 1 | a)
-  // (8 doubles) after the share_n current items (24 doubles each); share_stride doubles per event,
-  // interleaved by page of 32 events like the per-event record (double d of event e at
-  // (e / 32) * share_stride * 32 + d * 32 + e % 32).
-  int pref_levels;
-  int pref_off[kMaxGluons];
-  int share_stride;
 };
 
 // helicity bits of the gluons in mask, packed (bit g of gc -> the rank of g among mask's bits), and back
@@ -84,5 +70,43 @@ inline constexpr int pdep_bits(int h, int mask) {
 }
 
 void build_tables(int K, Tables& t);
+
+// ----------------------------------------------------------------------------------------
+// FP64 matrix elements of 3 to 5 gluons (mg_me64.cuh): the items shared between gluon-helicity combinations, the
+// tasks that compute them, and the terms of the colour-ordered amplitudes.  Offsets are in doubles per event; an item
+// of a gluon set holds one entry per helicity assignment of the set without gluon K-1 (which has helicity -1), in
+// pext_bits order; entries are 8 doubles (4 complex) times what the comment says.
+// ----------------------------------------------------------------------------------------
+struct Tab64 {
+  enum Type { kJ1, kJq0, kChi, kPsi, kSeq, kZ, kY, kQQ };
+  static constexpr int kMaxTask = 1500, kMaxLTask = 260, kMaxPass = 5;
+  struct Off {
+    int J[kMaxSeq];                        // current of a canonical sequence (1)
+    int X[kMaxSeq];                        // (gamma.J) v, three or more gluons (antitop helicity: 2); -1: none
+    int psi[kMaxGluons - 1][60];           // row spinor after m gluons, prefix = ordering / (K - m)! (top helicity: 2)
+    int chi[kMaxGluons];                   // column spinor before the last gluon (2)
+    int qg[kMaxGluons];                    // ubar gamma^mu chi(g) (2 top + antitop: 4)
+    int q0;                                // ubar gamma^mu v (4)
+    int z[kMaxGluons * kMaxGluons];        // last two gluons (2)
+    int y[kMaxSeq][kMaxGluons];            // (gamma.J_pair) chi(g) (2); -1: none
+    int qq[kMaxGluons * kMaxGluons];       // psi_1(g) gamma^mu chi(h), 5 gluons (4)
+  };
+  int K, stride, nloc;                     // doubles per event of the shared buffer, of one combination's own items
+  Off sh, loc;
+  int npass, pass0[kMaxPass + 1];
+  uint32_t task[kMaxTask];                 // type | a << 4 | b << 14 | gluon helicities << 20, by pass
+  int nltask;
+  uint32_t ltask[kMaxLTask];               // the same tasks without helicities, in an order that respects dependences
+  int16_t full_c[kMaxNcol / 2], full_cr[kMaxNcol / 2];   // orderings of a full current and of its reversal
+  int16_t t1[kMaxNcol / 2][4];             // sequence of K-1 gluons, last gluon, ordering, ordering reversed in the sequence
+  int16_t t2[kMaxNcol / 2][4];             // 5 gluons: sequence of the last 4, first gluon, ordering, reversed
+  int16_t t3[kMaxNcol / 2][4];             // 5 gluons: sequence of the middle 3, first * 5 + last gluon, ordering, reversed
+  int16_t g3[kMaxNcol / 6][3];             // six orderings with a common prefix of K-3: sequences xyz, xzy, yxz
+  int16_t gy[kMaxNcol / 6][3][2];          // (pair, last): (xy, z), (xz, y), (yz, x)
+  int16_t gz[kMaxNcol / 6][6];             // last two gluons, first * 5 + second, of the six orderings
+};
+
+void build_tab64(int K, const Tables& t, Tab64& o);
+const Tab64& tab64_host(int K);            // built once per process (K = 3..5)
 
 }  // namespace mg

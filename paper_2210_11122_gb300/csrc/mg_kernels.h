@@ -49,7 +49,7 @@ struct MeShape {
   bool fused = true;
   bool warp = false;
   bool tc_apart = false;
-  bool shared = true;   // FP64 amplitudes: currents of fewer than all gluons shared between slots
+  bool shared = true;   // FP64 amplitudes of 3 to 5 gluons: items shared between slots (launch_pass64)
   bool tc_sync = false;  // separate colour pass on mma.sync (k_colour_tc) instead of tcgen05 (k_colour_umma)
 };
 
@@ -80,16 +80,18 @@ cudaError_t launch_me_gluonhel(int K, bool fp32, bool per_hel, const double* mom
                                const uint32_t* mask, const double* ctri64, const float* ctri32, const MeConst& cst,
                                double* out, int64_t stride, cudaStream_t st, float2* jout = nullptr,
                                MeShape shape = MeShape(), const uint8_t* skip = nullptr,
-                               const int* evlist = nullptr, const int* nlist = nullptr, int rows_out = 0,
-                               const double* share = nullptr);
-// FP64 currents shared between gluon-helicity combinations: share_items(K) items of 24 doubles per event
-// (layout in mg_me_kernel.cuh), computed from the FP64 records of nevt events by K - 1 launches (one per
-// sequence length); launch_me_gluonhel(..., share) then reads them instead of computing them per slot.
-int share_items(int K);
-// doubles per event of the shared buffer: the current items, then the quark-line prefixes (mg_internal.h)
-int64_t share_doubles(int K);
-cudaError_t launch_share(int K, const void* rec, int64_t nevt, const Tables* tab, const MeConst& cst, double* share,
-                         cudaStream_t st);
+                               const int* evlist = nullptr, const int* nlist = nullptr, int rows_out = 0);
+// FP64 matrix elements of 3 to 5 gluons from the FP64 records of nevt events (mg_me64.cuh).  launch_pass64 fills the
+// items shared between gluon-helicity combinations (tab64_host(K).stride doubles per event, page-interleaved), a
+// few launches; launch_me64 runs one thread per (event, combination hslots[slot]), reading them, or with share = null
+// computing its own (the same bits).  Output: out[slot * stride + e] the weighted sum over the combination's
+// helicities (cst.conj = 1); or, with jout, FP32 jamps in rows of 2 * 2^K per event; or, with j2, the colour sum of
+// every helicity in rows slot * 4 + 2 top + antitop and the weighted jamp squares j2[(slot * ncol + sigma) * stride + e].
+cudaError_t launch_pass64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const MeConst& cst,
+                          double* share, cudaStream_t st);
+cudaError_t launch_me64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const int* hslots,
+                        const int* nslot, const uint32_t* mask, const double* ctri, const MeConst& cst, double* out,
+                        int64_t stride, float2* jout, MeShape shape, const double* share, double* j2, cudaStream_t st);
 int64_t event_record_bytes(int K, bool fp32);
 // The FP32 modes' recomputation of events evlist[0..*nlist) with double-float amplitudes (mg_me_dd.cu):
 // launch_me_gluonhel's contract for prep == NULL, per_hel false, FP32 colour table ctri32 (the per-thread

@@ -63,7 +63,7 @@ __device__ __forceinline__ double coupling_factor(double a0, double mu, double* 
 }
 
 // One thread per event: helicity sum (ascending helicity index), helicity and colour choices, coupling.
-// part rows: slot * 4 + 2 top + antitop (k_me_gluonhel<..., LHE>); j2: per-slot jamp-square sums.
+// part rows: slot * 4 + 2 top + antitop (launch_me64 with j2); j2: per-slot jamp-square sums.
 template <int K>
 __global__ void __launch_bounds__(128)
 k_lhe_epilogue(const double* __restrict__ part, const double* __restrict__ j2, const int* __restrict__ gslots,
@@ -144,45 +144,6 @@ k_alphas_running(const double* __restrict__ mom, int64_t nevt, double a0, double
   if (as_out) as_out[e] = as;
 }
 
-// The slot kernel's LHE rows with the currents and quark-line prefixes of launch_share, compiled for
-// MINB resident blocks per SM (the bound of the plain FP64 slot kernel)
-template <int K, int MINB>
-__global__ void __launch_bounds__(kMeThreads, MINB)
-k_lhe_slot(const double* __restrict__ rec, int64_t nevt, const Tables* __restrict__ tab, const int* __restrict__ gslots,
-           const int* __restrict__ nslot, const uint32_t* __restrict__ mask, const double* __restrict__ ctri, MeConst cst,
-           double* __restrict__ part, int64_t stride, int tile_ev, const double* __restrict__ share,
-           double* __restrict__ j2) {
-  v2::me_thread<K, double, false, true, false, true, true>(nullptr, rec, nevt, tab, gslots, nslot, mask, ctri, cst, part,
-                                                          stride, nullptr, tile_ev, 0, nullptr, nullptr, 0, nullptr,
-                                                          share, j2);
-}
-
-// share: the chunk's currents and quark-line prefixes from launch_share (the slot kernel reads them
-// instead of forming them; bit-identical), or null for the unshared walk
-template <int K>
-cudaError_t launch_lhe_me(const double* rec, int64_t nevt, const Tables* tab, const int* gslots, int maxslot,
-                          const int* nslot, const uint32_t* mask, const double* ctri, const MeConst& cst, double* part,
-                          double* j2, int64_t stride, const double* share, cudaStream_t st) {
-  const int tev = 128, tsl = kMeThreads / tev;
-  const dim3 grid(static_cast<unsigned>((nevt + tev - 1) / tev), static_cast<unsigned>((maxslot + tsl - 1) / tsl));
-  // bounded compile for 2, 3 and 5 gluons (measured 12-25 % faster than unbounded); with 4 its 24 per-flow
-  // sums spill at 168 registers and the unbounded kernel is 7 % faster
-  if (share) {
-    if constexpr (K == 4)
-      v2::k_me_gluonhel<K, double, false, true, false, true, true><<<grid, kMeThreads, 0, st>>>(
-          nullptr, rec, nevt, tab, gslots, nslot, mask, ctri, cst, part, stride, nullptr, tev, 0, nullptr, nullptr, 0,
-          nullptr, share, j2);
-    else
-      k_lhe_slot<K, K <= 3 ? 4 : 3><<<grid, kMeThreads, 0, st>>>(rec, nevt, tab, gslots, nslot, mask, ctri, cst, part,
-                                                                stride, tev, share, j2);
-  } else
-    v2::k_me_gluonhel<K, double, false, true, false, false, true><<<grid, kMeThreads, 0, st>>>(
-        nullptr, rec, nevt, tab, gslots, nslot, mask, ctri, cst, part, stride, nullptr, tev, 0, nullptr, nullptr, 0,
-        nullptr, nullptr, j2);
-  note_launch();
-  return cudaGetLastError();
-}
-
 template <int K>
 cudaError_t launch_epilogue(const double* part, const double* j2, const int* gslots, const int* nslot,
                             const uint32_t* mask, const double* mom, int64_t nevt, int64_t stride, double norm,
@@ -214,16 +175,20 @@ mg_status grow_buf(double** buf, int64_t* cap, int64_t need) {
   return MG_OK;
 }
 
+// The slots' colour sums per helicity and jamp squares; share: the chunk's items from launch_pass64 (3 to 5 gluons),
+// or null: every combination on its own (the same bits)
 cudaError_t lhe_me(int K, const double* rec, int64_t nevt, const mg_ctx* c, const mg::MeConst& cst, double* part,
                    double* j2, int64_t stride, const double* share, cudaStream_t st) {
-  const int ms = 1 << (K - 1);
-  switch (K) {
-    case 2: return mg::lhe::launch_lhe_me<2>(rec, nevt, c->d_tab, c->d_hslots, ms, c->d_nhslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
-    case 3: return mg::lhe::launch_lhe_me<3>(rec, nevt, c->d_tab, c->d_hslots, ms, c->d_nhslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
-    case 4: return mg::lhe::launch_lhe_me<4>(rec, nevt, c->d_tab, c->d_hslots, ms, c->d_nhslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
-    case 5: return mg::lhe::launch_lhe_me<5>(rec, nevt, c->d_tab, c->d_hslots, ms, c->d_nhslots, c->d_mask, c->d_ctri, cst, part, j2, stride, share, st);
-    default: return cudaErrorInvalidValue;
-  }
+  if (K >= 3)
+    return mg::launch_me64(K, rec, nevt, c->d_tab, c->d_tab64, c->d_hslots, c->d_nhslots, c->d_mask, c->d_ctri, cst, part,
+                           stride, nullptr, mg::MeShape(), share, j2, st);
+  constexpr int tev = mg::kMeThreads;
+  const dim3 grid(static_cast<unsigned>((nevt + tev - 1) / tev), 2);
+  mg::v2::k_me_gluonhel<2, double, false, true, false, true><<<grid, mg::kMeThreads, 0, st>>>(
+      nullptr, rec, nevt, c->d_tab, c->d_hslots, c->d_nhslots, c->d_mask, c->d_ctri, cst, part, stride, nullptr, tev, 0,
+      nullptr, nullptr, 0, nullptr, j2);
+  mg::note_launch();
+  return cudaGetLastError();
 }
 
 cudaError_t lhe_epilogue(int K, const double* j2, const mg_ctx* c, const double* mom, int64_t nevt, int64_t stride,
@@ -264,8 +229,8 @@ mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, cons
   const int64_t stride_all = pad_page(nevt);
   if (chunk < mg::kPage) chunk = mg::kPage;
   if (chunk > stride_all) chunk = stride_all;
-  // the FP64 launch shape's choice of shared currents and prefixes (chunks within their buffer)
-  const bool shared = ctx->shape[MG_FP64].shared;
+  // the FP64 launch shape's choice of shared items (chunks within their buffer)
+  const bool shared = ctx->shape[MG_FP64].shared && K >= 3;
   if (shared) {
     const int64_t sc = mg::share_chunk(K, stride_all);
     if (sc < chunk) chunk = sc;
@@ -287,7 +252,7 @@ mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, cons
     const int64_t stride = pad_page(n);
     const double* mom_c = mom_dev + (e0 / mg::kPage) * ctx->npar * 4 * mg::kPage;
     if (mg::launch_event_prep(K, false, mom_c, n, cst, ctx->d_prep, st) != cudaSuccess) return MG_ECUDA;
-    if (shared && mg::launch_share(K, ctx->d_prep, n, ctx->d_tab, cst, ctx->d_share, st) != cudaSuccess) return MG_ECUDA;
+    if (shared && mg::launch_pass64(K, ctx->d_prep, n, ctx->d_tab, ctx->d_tab64, cst, ctx->d_share, st) != cudaSuccess) return MG_ECUDA;
     if (lhe_me(K, ctx->d_prep, n, ctx, cst, ctx->d_part, ctx->d_j2, stride, shared ? ctx->d_share : nullptr, st) !=
         cudaSuccess)
       return MG_ECUDA;

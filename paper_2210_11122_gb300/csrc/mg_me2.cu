@@ -115,8 +115,7 @@ template <int K, class T, bool PER_HEL>
 static cudaError_t launch_v2(const double* mom, void* prep, int64_t nevt, const Tables* tab, const int* gslots,
                              int maxslot, const int* nslot, const uint32_t* mask, const void* ctri_any,
                              const MeConst& cst, double* out, int64_t stride, float2* jout, MeShape shape,
-                             const uint8_t* skip, const int* evlist, const int* nlist, int rows_out, cudaStream_t st,
-                             const double* share) {
+                             const uint8_t* skip, const int* evlist, const int* nlist, int rows_out, cudaStream_t st) {
   const T* ctri = static_cast<const T*>(ctri_any);
   int tev = shape.tile_ev;
   if (tev != 32 && tev != 64 && tev != 128) tev = 128;
@@ -141,38 +140,19 @@ static cudaError_t launch_v2(const double* mom, void* prep, int64_t nevt, const 
       return launch_me_static(K, sizeof(T) == 4, rec, nevt, gslots, maxslot, nslot, mask, cst, out, stride, jout, shape,
                               skip, st);
     if constexpr (std::is_same<T, double>::value) {
-      // the compile for more resident blocks (k_me_gluonhel_occ): 2, 4 and 5 gluons, and 3 with shared
-      // currents (without them its bounded compile spills ~0.5 KB per thread)
-      if constexpr (K >= 2) {
-        constexpr int MINB = K <= 3 ? 4 : 3;
-        if (K != 3 || share) {
-          if (jout && share)
-            { v2::k_me_gluonhel_occ<K, true, true, MINB><<<grid, threads, 0, st>>>(
-                rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride, jout, tev, sm, skip, share); mg::note_launch(); }
-          else if (share)
-            { v2::k_me_gluonhel_occ<K, false, true, MINB><<<grid, threads, 0, st>>>(
-                rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride, nullptr, tev, sm, skip, share); mg::note_launch(); }
-          else if (jout)
-            { v2::k_me_gluonhel_occ<K, true, false, MINB><<<grid, threads, 0, st>>>(
-                rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride, jout, tev, sm, skip, nullptr); mg::note_launch(); }
-          else
-            { v2::k_me_gluonhel_occ<K, false, false, MINB><<<grid, threads, 0, st>>>(
-                rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride, nullptr, tev, sm, skip, nullptr); mg::note_launch(); }
-          return cudaGetLastError();
-        }
-      }
-      if (share) {
+      // FP64 with a record: 2 gluons here (the compile for more resident blocks), 3 to 5 in launch_me64
+      if constexpr (K == 2) {
         if (jout)
-          { v2::k_me_gluonhel<K, T, false, true, true, true><<<grid, threads, 0, st>>>(
-              mom, rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride, jout, tev, sm, nullptr, nullptr, 0, skip,
-              share); mg::note_launch(); }
+          { v2::k_me_gluonhel2<true><<<grid, threads, 0, st>>>(rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride,
+                                                              jout, tev, sm); mg::note_launch(); }
         else
-          { v2::k_me_gluonhel<K, T, false, true, false, true><<<grid, threads, 0, st>>>(
-              mom, rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride, nullptr, tev, sm, nullptr, nullptr, 0,
-              skip, share); mg::note_launch(); }
+          { v2::k_me_gluonhel2<false><<<grid, threads, 0, st>>>(rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride,
+                                                               nullptr, tev, sm); mg::note_launch(); }
         return cudaGetLastError();
+      } else {
+        return cudaErrorInvalidValue;
       }
-    }
+    } else {
     if (jout)
       { v2::k_me_gluonhel<K, T, false, true, true><<<grid, threads, 0, st>>>(mom, rec, nevt, tab, gslots, nslot, mask,
                                                                              ctri, cst, out, stride, jout, tev, sm, nullptr,
@@ -181,6 +161,7 @@ static cudaError_t launch_v2(const double* mom, void* prep, int64_t nevt, const 
       { v2::k_me_gluonhel<K, T, false, true, false><<<grid, threads, 0, st>>>(mom, rec, nevt, tab, gslots, nslot,
                                                                               mask, ctri, cst, out, stride, nullptr, tev,
                                                                               sm, nullptr, nullptr, 0, skip); mg::note_launch(); }
+    }
   } else if (PER_HEL) {
     // the helicity filter: a few thousand threads, so blocks of one warp (32 events of one slot) spread
     // them evenly over every SM; 128-thread blocks left a third of the SMs with twice the work
@@ -211,75 +192,6 @@ cudaError_t launch_event_prep(int K, bool fp32, const double* mom, int64_t nevt,
     case 3: return fp32 ? launch_prep<3, float>(mom, nevt, cst, rec, st) : launch_prep<3, double>(mom, nevt, cst, rec, st);
     case 4: return fp32 ? launch_prep<4, float>(mom, nevt, cst, rec, st) : launch_prep<4, double>(mom, nevt, cst, rec, st);
     case 5: return fp32 ? launch_prep<5, float>(mom, nevt, cst, rec, st) : launch_prep<5, double>(mom, nevt, cst, rec, st);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-template <int K>
-static cudaError_t launch_share_k(const void* rec, int64_t nevt, const Tables* tab, const MeConst& cst, double* share,
-                                  cudaStream_t st) {
-  int s0 = 0;
-  for (int level = 1; level < K; ++level) {
-    int n = 1;   // canonical sequences of `level` gluons: K!/(K-level)!/2 (the K singles for level 1)
-    for (int i = 0; i < level; ++i) n *= K - i;
-    const int count = level == 1 ? K : n / 2;
-    const int64_t threads = (nevt + kPage - 1) / kPage * kPage * (static_cast<int64_t>(count) << level);
-    if (threads > 0)
-      { v2::k_share_level<K><<<static_cast<unsigned>((threads + 127) / 128), 128, 0, st>>>(
-          static_cast<const double*>(rec), nevt, tab, cst, level, s0, s0 + count, share); mg::note_launch(); }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    s0 += count;
-  }
-  // then the quark-line prefixes, level by level (each reads the currents and the lower levels)
-  const int levels = K - 1 < 3 ? K - 1 : 3;
-  for (int m = 1; m <= levels; ++m) {
-    int orderings = 1;
-    for (int i = 0; i < m; ++i) orderings *= K - i;
-    const int64_t threads = (nevt + kPage - 1) / kPage * kPage * (static_cast<int64_t>(orderings) << m);
-    const unsigned blocks = static_cast<unsigned>((threads + 127) / 128);
-    const double* r = static_cast<const double*>(rec);
-    if (threads > 0) {
-      if (m == 1) v2::k_prefix_level<K, 1><<<blocks, 128, 0, st>>>(r, nevt, tab, share);
-      if constexpr (K >= 3) if (m == 2) v2::k_prefix_level<K, 2><<<blocks, 128, 0, st>>>(r, nevt, tab, share);
-      if constexpr (K >= 4) if (m == 3) v2::k_prefix_level<K, 3><<<blocks, 128, 0, st>>>(r, nevt, tab, share);
-      mg::note_launch();
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-int64_t share_doubles(int K) {
-  int64_t nodes = 0;
-  const int levels = K - 1 < 3 ? K - 1 : 3;
-  for (int m = 1; m <= levels; ++m) {
-    int orderings = 1;
-    for (int i = 0; i < m; ++i) orderings *= K - i;
-    nodes += static_cast<int64_t>(orderings << m) * 2;
-  }
-  return static_cast<int64_t>(share_items(K)) * 24 + nodes * 8;
-}
-
-int share_items(int K) {
-  int n = 0, total = 0;
-  for (int level = 1; level < K; ++level) {
-    int f = 1;
-    for (int i = 0; i < level; ++i) f *= K - i;
-    n = level == 1 ? K : f / 2;
-    total += n << level;
-  }
-  return total;
-}
-
-cudaError_t launch_share(int K, const void* rec, int64_t nevt, const Tables* tab, const MeConst& cst, double* share,
-                         cudaStream_t st) {
-  switch (K) {
-    case 2: return launch_share_k<2>(rec, nevt, tab, cst, share, st);
-    case 3: return launch_share_k<3>(rec, nevt, tab, cst, share, st);
-    case 4: return launch_share_k<4>(rec, nevt, tab, cst, share, st);
-    case 5: return launch_share_k<5>(rec, nevt, tab, cst, share, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -320,18 +232,17 @@ cudaError_t launch_me_gluonhel(int K, bool fp32, bool per_hel, const double* mom
                                const Tables* tab, const int* gslots, int maxslot, const int* nslot,
                                const uint32_t* mask, const double* ctri64, const float* ctri32, const MeConst& cst,
                                double* out, int64_t stride, cudaStream_t st, float2* jout, MeShape shape,
-                               const uint8_t* skip, const int* evlist, const int* nlist, int rows_out,
-                               const double* share) {
+                               const uint8_t* skip, const int* evlist, const int* nlist, int rows_out) {
 #define MG_V2_CASE(KK)                                                                                              \
   case KK:                                                                                                          \
     if (per_hel) return fp32 ? launch_v2<KK, float, true>(mom, prep, nevt, tab, gslots, maxslot, nslot, mask, ctri32, cst,  \
-                                                          out, stride, jout, shape, skip, evlist, nlist, rows_out, st, share)                                          \
+                                                          out, stride, jout, shape, skip, evlist, nlist, rows_out, st)                                          \
                              : launch_v2<KK, double, true>(mom, prep, nevt, tab, gslots, maxslot, nslot, mask, ctri64, cst, \
-                                                           out, stride, jout, shape, skip, evlist, nlist, rows_out, st, share);                                        \
+                                                           out, stride, jout, shape, skip, evlist, nlist, rows_out, st);                                        \
     return fp32 ? launch_v2<KK, float, false>(mom, prep, nevt, tab, gslots, maxslot, nslot, mask, ctri32, cst, out, stride, \
-                                              jout, shape, skip, evlist, nlist, rows_out, st, share)                                                                   \
+                                              jout, shape, skip, evlist, nlist, rows_out, st)                                                                   \
                 : launch_v2<KK, double, false>(mom, prep, nevt, tab, gslots, maxslot, nslot, mask, ctri64, cst, out, stride,\
-                                               jout, shape, skip, evlist, nlist, rows_out, st, share);
+                                               jout, shape, skip, evlist, nlist, rows_out, st);
   switch (K) {
     MG_V2_CASE(2)
     MG_V2_CASE(3)

@@ -1,0 +1,525 @@
+// mg_me64.cuh -- the FP64 matrix elements of 3 to 5 gluons: colour-ordered amplitudes with the quark line cut
+// in front of its last two gluons, one thread per (event, gluon-helicity combination).
+//
+// GB300 issues one FP64 instruction per warp and SM sub-partition every 64 cycles, so the FP64 instruction count is
+// the cost and everything else (loads, integer work, local memory) hides behind it.  Two things keep it low:
+//   * everything that depends on fewer than all gluons is computed once per helicity assignment of those gluons and
+//     read by every combination that shares it (k_pass64, a few launches of independent tasks per event, into a
+//     page-interleaved buffer);
+//   * the amplitude of an ordering sigma of K gluons is not built by carrying the quark line up to the antitop but
+//     by cutting it.  With the row spinors psi_m (top and the first m gluons, propagator included), the column
+//     spinors chi(g) = S (gamma.J_g) v (antitop and the last gluon, propagator included) and the gluon currents J,
+//         A = psi_{K-2} . Z(s_{K-1}, s_K) + sum_{i < K-2} psi_i . [ X(i+1..K) + (gamma.J(i+1..K-1)) chi(s_K) ],
+//         Z(g, h) = (gamma.J_g) chi(h) + (gamma.J_gh) v,   X(i+1..K) = (gamma.J(i+1..K)) v:
+//     every term is one spinor or vector product (16 FP64 instructions per helicity), the factors are shared, and a
+//     term whose current holds two or more consecutive gluons serves two orderings (reflection, up to a sign).  No
+//     prefix of K-1 gluons is formed, which was most of the quark line's cost (5 gluons: 256 instead of 704
+//     instructions per ordering and combination).
+// A flipped combination's |M|^2 equals the combination's (hel_weight), so gluon K-1 has helicity -1 throughout and
+// an item's helicity index leaves its bit out.
+//
+// Measured against carrying the prefixes of up to K-1 gluons (both on half of the combinations): gg->ttg FP64 12.13 vs
+// 14.48 ms per 524,288 events, LHE choices of gg->ttgg 9.35 vs 11.63 ms per 32,768, gg->ttggg + TC colour 8.60 vs
+// 12.37 ms per 2,049.
+//
+// The combination may also build its own items in local memory (LOCAL, no buffer): the same functions, so the same
+// bits, at about three times the FP64 work.
+#pragma once
+
+#include "mg_me_algebra.cuh"
+
+namespace mg {
+namespace m64 {
+
+using v2::cx;
+
+__device__ constexpr int kFact[6] = {1, 1, 2, 6, 24, 120};
+
+// doubles of one combination's own items (LOCAL)
+template <int K> struct Loc;
+template <> struct Loc<3> { static constexpr int n = 368; };
+template <> struct Loc<4> { static constexpr int n = 1232; };
+template <> struct Loc<5> { static constexpr int n = 5352; };
+
+// (Qslash + m) f on a column spinor, coefficients as row_prop's
+__device__ __forceinline__ void col_prop(const cx<double>* s, const double* q, cx<double>* o) {
+  const double qa = q[0], qb = q[1], qm = q[4];
+  const cx<double> qp = {q[2], q[3]}, qn = {q[2], -q[3]};
+  o[0] = v2::cscale(qb, s[2]); v2::cmsub(o[0], qn, s[3]); v2::cmacr(o[0], qm, s[0]);
+  o[1] = v2::cscale(qa, s[3]); v2::cmsub(o[1], qp, s[2]); v2::cmacr(o[1], qm, s[1]);
+  o[2] = v2::cscale(qa, s[0]); v2::cmac(o[2], qn, s[1]); v2::cmacr(o[2], qm, s[2]);
+  o[3] = v2::cscale(qb, s[1]); v2::cmac(o[3], qp, s[0]); v2::cmacr(o[3], qm, s[3]);
+}
+
+// o += (gamma.J) v from the current's gamma.J entries
+__device__ __forceinline__ void col_slash_acc(cx<double>* o, const v2::Slash<double>& g, const cx<double>* v) {
+  v2::cmac(o[0], g.b, v[2]); v2::cmsub(o[0], g.jm, v[3]);
+  v2::cmac(o[1], g.a, v[3]); v2::cmsub(o[1], g.jp, v[2]);
+  v2::cmac(o[2], g.a, v[0]); v2::cmac(o[2], g.jm, v[1]);
+  v2::cmac(o[3], g.jp, v[0]); v2::cmac(o[3], g.b, v[1]);
+}
+
+// The items of one event for the helicities gc: in the shared buffer (double d of event e at
+// (e / 32) * stride * 32 + d * 32 + e % 32, so a warp's access is one 256-byte line) or in the thread's own array.
+template <int K, bool LOCAL>
+struct View {
+  using L = v2::EvLayout<K>;
+  static constexpr int ST = LOCAL ? 1 : kPage;
+  const double* in;   // the event's record
+  double* buf;
+  const Tables* tab;
+  const Tab64* t;
+  const Tab64::Off* o;
+  int gc;
+  double gs;
+
+  __device__ __forceinline__ int h(int mask) const { return LOCAL ? 0 : pext_bits(gc, mask & ((1 << (K - 1)) - 1)); }
+  __device__ __forceinline__ double rec(int item) const { return __ldg(in + item * kPage); }
+  __device__ __forceinline__ void ld(int off, cx<double>* v) const {
+    const double* p = buf + static_cast<int64_t>(off) * ST;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = {p[(2 * m) * ST], p[(2 * m + 1) * ST]};
+  }
+  __device__ __forceinline__ void st(int off, const cx<double>* v) const {
+    double* p = buf + static_cast<int64_t>(off) * ST;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      p[(2 * m) * ST] = v[m].r;
+      p[(2 * m + 1) * ST] = v[m].i;
+    }
+  }
+  __device__ __forceinline__ void top(int item, cx<double>* v) const {   // L::UB or L::VV + 8 * helicity
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = {rec(item + 2 * q), rec(item + 2 * q + 1)};
+  }
+  __device__ __forceinline__ void qc(int S, double* q) const {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) q[i] = rec(L::QC + 5 * S + i);
+  }
+  __device__ __forceinline__ void mom(int s, double* P) const {
+#pragma unroll
+    for (int m = 0; m < 4; ++m) P[m] = rec(L::PT + 4 * tab->seq_mask[s] + m);
+  }
+  __device__ __forceinline__ void gluon(int g, cx<double>* J) const {   // the external current itself
+    double pol[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) pol[i] = rec(L::EPS + 5 * g + i);
+    v2::ext_gluon(pol, (gc >> g) & 1 ? 1 : -1, g >= 2, J);
+  }
+  __device__ __forceinline__ int offJ(int s) const { return o->J[s] + h(tab->seq_mask[s]) * 8; }
+  __device__ __forceinline__ int offX(int s, int b) const { return o->X[s] + (h(tab->seq_mask[s]) * 2 + b) * 8; }
+  __device__ __forceinline__ int offPsi(int m, int p, int a) const {
+    return o->psi[m][p] + (h(tab->prefix_mask[p * kFact[K - m]][m]) * 2 + a) * 8;
+  }
+  __device__ __forceinline__ int offChi(int g, int b) const { return o->chi[g] + (h(1 << g) * 2 + b) * 8; }
+  __device__ __forceinline__ int offQg(int g, int ab) const { return o->qg[g] + (h(1 << g) * 4 + ab) * 8; }
+  __device__ __forceinline__ int offZ(int g, int g2, int b) const {
+    return o->z[g * kMaxGluons + g2] + (h(1 << g | 1 << g2) * 2 + b) * 8;
+  }
+  __device__ __forceinline__ int offY(int s, int g, int b) const {
+    return o->y[s][g] + (h(tab->seq_mask[s] | 1 << g) * 2 + b) * 8;
+  }
+  __device__ __forceinline__ int offQQ(int g, int g2, int ab) const {
+    return o->qq[g * kMaxGluons + g2] + (h(1 << g | 1 << g2) * 4 + ab) * 8;
+  }
+  __device__ __forceinline__ void J(int s, cx<double>* v) const { ld(offJ(s), v); }
+
+  // current of a canonical split list: three- and four-gluon vertices summed
+  __device__ __forceinline__ void vertices(cx<double>* acc, int n3, const int16_t (*v3)[2], int n4,
+                                           const int16_t (*v4)[3]) const {
+    for (int k = 0; k < n3; ++k) {
+      const int16_t rl = v3[k][0], rr = v3[k][1];
+      cx<double> JL[4], JR[4];
+      double PL[4], PR[4];
+      J(v2::rslot(rl), JL);
+      J(v2::rslot(rr), JR);
+      mom(v2::rslot(rl), PL);
+      mom(v2::rslot(rr), PR);
+      v2::v3_acc(acc, JL, JR, PL, PR, v2::rneg(rl) != v2::rneg(rr));
+    }
+    for (int k = 0; k < n4; ++k) {
+      const int16_t ra = v4[k][0], rb = v4[k][1], rc = v4[k][2];
+      cx<double> JA[4], JB[4], JC[4];
+      J(v2::rslot(ra), JA);
+      J(v2::rslot(rb), JB);
+      J(v2::rslot(rc), JC);
+      v2::v4_acc(acc, JA, JB, JC, gs, v2::rneg(ra) ^ v2::rneg(rb) ^ v2::rneg(rc));
+    }
+  }
+};
+
+// psi_M of prefix p for both top helicities (each current's gamma.J entries shared by the two)
+template <int K, bool LOCAL, int M>
+__device__ __forceinline__ void task_psi(const View<K, LOCAL>& V, int p) {
+  using L = v2::EvLayout<K>;
+  const int c0 = p * kFact[K - M];
+  v2::Slash<double> g[M];
+#pragma unroll
+  for (int j = 0; j < M; ++j) {
+    const int16_t r = V.tab->sub[c0][j][M];
+    cx<double> Jr[4];
+    if constexpr (M == 1) V.gluon(v2::rslot(r), Jr);
+    else V.J(v2::rslot(r), Jr);
+    g[j] = v2::slash_of(Jr, v2::rneg(r));
+  }
+  double q[5];
+  V.qc(V.tab->prefix_mask[c0][M], q);
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    cx<double> acc[4] = {};
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+      cx<double> s[4];
+      if (j == 0) V.top(L::UB + 8 * a, s);
+      else V.ld(V.offPsi(j, c0 / kFact[K - j], a), s);
+      v2::row_slash_acc(acc, s, g[j]);
+    }
+    cx<double> out[4];
+    v2::row_prop(acc, q, out);
+    V.st(V.offPsi(M, p, a), out);
+  }
+}
+
+// One task of the passes: an item (or a few that share work) for the view's helicities.
+template <int K, bool LOCAL>
+__device__ __forceinline__ void run_task(const View<K, LOCAL>& V, uint32_t task) {
+  using L = v2::EvLayout<K>;
+  const int type = task & 15, a_ = (task >> 4) & 1023, b_ = (task >> 14) & 63;
+  switch (type) {
+    case Tab64::kJ1: {
+      cx<double> J[4];
+      V.gluon(a_, J);
+      V.st(V.offJ(a_), J);
+      break;
+    }
+    case Tab64::kJq0: {   // ubar gamma^mu v of the four top helicity pairs
+#pragma unroll
+      for (int ab = 0; ab < 4; ++ab) {
+        cx<double> u[4], v[4], Jq[4];
+        V.top(L::UB + 8 * (ab >> 1), u);
+        V.top(L::VV + 8 * (ab & 1), v);
+        v2::quark_current(u, v, Jq);
+        V.st(V.o->q0 + ab * 8, Jq);
+      }
+      break;
+    }
+    case Tab64::kChi: {   // chi(g), and ubar gamma^mu chi(g)
+      cx<double> J[4];
+      V.gluon(a_, J);
+      double q[5];
+      V.qc(((1 << K) - 1) ^ (1 << a_), q);
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        cx<double> v[4], X[4], chi[4];
+        V.top(L::VV + 8 * b, v);
+        v2::gamma_col(J, v, X);
+        col_prop(X, q, chi);
+        V.st(V.offChi(a_, b), chi);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+          cx<double> u[4], Jq[4];
+          V.top(L::UB + 8 * a, u);
+          v2::quark_current(u, chi, Jq);
+          V.st(V.offQg(a_, 2 * a + b), Jq);
+        }
+      }
+      break;
+    }
+    case Tab64::kPsi:
+      if (b_ == 1) task_psi<K, LOCAL, 1>(V, a_);
+      if constexpr (K >= 4) if (b_ == 2) task_psi<K, LOCAL, 2>(V, a_);
+      if constexpr (K >= 5) if (b_ == 3) task_psi<K, LOCAL, 3>(V, a_);
+      break;
+    case Tab64::kSeq: {   // J of a sequence of two or more gluons; X for those of three or more
+      cx<double> acc[4] = {}, J[4];
+      V.vertices(acc, V.tab->seq_nv3[a_], V.tab->seq_v3[a_], V.tab->seq_nv4[a_], V.tab->seq_v4[a_]);
+      const double f = V.rec(L::GP + V.tab->seq_mask[a_]);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) J[m] = v2::cscale(f, acc[m]);
+      V.st(V.offJ(a_), J);
+      if (V.o->X[a_] >= 0) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          cx<double> v[4], X[4];
+          V.top(L::VV + 8 * b, v);
+          v2::gamma_col(J, v, X);
+          V.st(V.offX(a_, b), X);
+        }
+      }
+      break;
+    }
+    case Tab64::kZ: {   // Z(g, h) and Z(h, g) of a canonical pair: J(h, g) = -J(g, h)
+      const int m = V.tab->seq_mask[a_], g = __ffs(m) - 1, g2 = __ffs(m & (m - 1)) - 1;
+      cx<double> J[4];
+      V.J(a_, J);
+      cx<double> Jg[4], Jh[4];
+      V.J(g, Jg);
+      V.J(g2, Jh);
+      const v2::Slash<double> sg = v2::slash_of(Jg, false), sh = v2::slash_of(Jh, false);
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        cx<double> v[4], X[4], c[4];
+        V.top(L::VV + 8 * b, v);
+        v2::gamma_col(J, v, X);
+        cx<double> z[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[i] = v2::cneg(X[i]);
+        V.ld(V.offChi(g2, b), c);
+        col_slash_acc(X, sg, c);
+        V.st(V.offZ(g, g2, b), X);
+        V.ld(V.offChi(g, b), c);
+        col_slash_acc(z, sh, c);
+        V.st(V.offZ(g2, g, b), z);
+      }
+      break;
+    }
+    case Tab64::kY: {   // (gamma.J_s) chi(g)
+      cx<double> J[4];
+      V.J(a_, J);
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        cx<double> c[4], Y[4];
+        V.ld(V.offChi(b_, b), c);
+        v2::gamma_col(J, c, Y);
+        V.st(V.offY(a_, b_, b), Y);
+      }
+      break;
+    }
+    default: {   // kQQ: psi_1(g) gamma^mu chi(h), four top helicity pairs
+#pragma unroll
+      for (int ab = 0; ab < 4; ++ab) {
+        cx<double> s[4], c[4], Jq[4];
+        V.ld(V.offPsi(1, a_, ab >> 1), s);
+        V.ld(V.offChi(b_, ab & 1), c);
+        v2::quark_current(s, c, Jq);
+        V.st(V.offQQ(a_, b_, ab), Jq);
+      }
+      break;
+    }
+  }
+}
+
+// One thread per (event, task of the pass): tasks [t0, t0 + ntask) of the table, warps on one task of 32 consecutive
+// events.  Bound by the FP64 pipe.
+template <int K>
+__global__ void __launch_bounds__(128)
+k_pass64(const double* __restrict__ rec, int64_t nevt, const Tables* __restrict__ tab, const Tab64* __restrict__ t64,
+         double gs, int t0, int ntask, double* __restrict__ share) {
+  const int64_t npage = (nevt + kPage - 1) / kPage;
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t j = t / (npage * kPage);
+  if (j >= ntask) return;
+  const int64_t e = t - j * npage * kPage;
+  if (e >= nevt) return;
+  const uint32_t task = t64->task[t0 + j];
+  View<K, false> V;
+  V.in = rec + (e / kPage) * v2::EvLayout<K>::NITEM * kPage + (e % kPage);
+  V.buf = share + (e / kPage) * static_cast<int64_t>(t64->stride) * kPage + (e % kPage);
+  V.tab = tab;
+  V.t = t64;
+  V.o = &t64->sh;
+  V.gc = static_cast<int>(task >> 20);
+  V.gs = gs;
+  run_task<K, false>(V, task);
+}
+
+constexpr int kME = 0, kJamps = 1, kLhe = 2;
+
+// The amplitudes of one (event, combination) for the four top helicity pairs and what the mode makes of them:
+// kME: out[slot * stride + e] = the weighted sum of the colour sums; kJamps: FP32 jamps, rows slot * 4 + 2 top +
+// antitop of jout (zeros for weight 0); kLhe: the colour sum of every helicity in its own row of out (zero for
+// weight 0) and the weighted |jamp|^2 of every ordering in j2.
+template <int K, int MODE, bool LOCAL>
+__device__ __forceinline__ void slot64(const View<K, LOCAL>& V, int64_t e, int slot, const uint32_t* __restrict__ mask,
+                                       const double* __restrict__ ctri, const MeConst& cst, double* __restrict__ out,
+                                       int64_t stride, float2* __restrict__ jout, double* __restrict__ j2) {
+  using L = v2::EvLayout<K>;
+  constexpr int npar = K + 2, NCOL = v2::Sizes<K>::ncol, NFULL = v2::Sizes<K>::nfull, NSUB = 1 << K;
+  constexpr bool kNegK = (K & 1) == 0, kNegK1 = !kNegK;   // reflection signs of K and K-1 gluons: negative?
+  const Tables* tab = V.tab;
+  const Tab64* t = V.t;
+  int w[4];
+  {
+    int hb = 0;
+#pragma unroll
+    for (int g = 0; g < K; ++g)
+      if ((V.gc >> g) & 1) hb |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab)
+      w[ab] = hel_weight(mask, hb | ((ab >> 1) << (npar - 3)) | ((ab & 1) << (npar - 4)), npar, cst.conj);
+  }
+  cx<double> A[4][NCOL];
+  // all gluons on one current, contracted with the four quark currents
+  {
+    const double fz = V.rec(L::GP + NSUB - 1);
+    for (int f = 0; f < NFULL; ++f) {
+      cx<double> acc[4] = {}, JF[4];
+      V.vertices(acc, tab->full_nv3[f], tab->full_v3[f], tab->full_nv4[f], tab->full_v4[f]);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) JF[m] = v2::cscale(fz, acc[m]);
+      const int c = t->full_c[f], cr = t->full_cr[f];
+#pragma unroll
+      for (int ab = 0; ab < 4; ++ab) {
+        cx<double> Jq[4];
+        V.ld(V.o->q0 + ab * 8, Jq);
+        const cx<double> x = v2::mdot(Jq, JF);
+        A[ab][c] = x;
+        A[ab][cr] = kNegK ? v2::cneg(x) : x;
+      }
+    }
+  }
+  auto add = [&](int ab, int c, cx<double> x, bool neg) {
+    A[ab][c].r = neg ? A[ab][c].r - x.r : A[ab][c].r + x.r;
+    A[ab][c].i = neg ? A[ab][c].i - x.i : A[ab][c].i + x.i;
+  };
+  // the first K-1 gluons on one current, the last on chi
+  for (int i = 0; i < NCOL / 2; ++i) {
+    const int s = t->t1[i][0], g = t->t1[i][1], c = t->t1[i][2], cr = t->t1[i][3];
+    cx<double> J[4];
+    V.J(s, J);
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab) {
+      cx<double> Jq[4];
+      V.ld(V.offQg(g, ab), Jq);
+      const cx<double> x = v2::mdot(Jq, J);
+      add(ab, c, x, false);
+      add(ab, cr, x, kNegK1);
+    }
+  }
+  if constexpr (K == 5) {
+    // one gluon on the top, the other four on one current, or three of them and the last on chi
+    for (int i = 0; i < NCOL / 2; ++i) {
+      const int s = t->t2[i][0], g = t->t2[i][1], c = t->t2[i][2], cr = t->t2[i][3];
+      cx<double> X[2][4];
+#pragma unroll
+      for (int b = 0; b < 2; ++b) V.ld(V.offX(s, b), X[b]);
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        cx<double> p[4];
+        V.ld(V.offPsi(1, g, a), p);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          cx<double> x = {};
+          v2::sdot_acc(x, p, X[b], false);
+          add(2 * a + b, c, x, false);
+          add(2 * a + b, cr, x, true);
+        }
+      }
+    }
+    for (int i = 0; i < NCOL / 2; ++i) {
+      const int s = t->t3[i][0], g = t->t3[i][1] / kMaxGluons, g2 = t->t3[i][1] % kMaxGluons, c = t->t3[i][2],
+                cr = t->t3[i][3];
+      cx<double> J[4];
+      V.J(s, J);
+#pragma unroll
+      for (int ab = 0; ab < 4; ++ab) {
+        cx<double> Jq[4];
+        V.ld(V.offQQ(g, g2, ab), Jq);
+        const cx<double> x = v2::mdot(Jq, J);
+        add(ab, c, x, false);
+        add(ab, cr, x, false);
+      }
+    }
+  }
+  // the orderings of the last three gluons after a common prefix: six consecutive orderings, x < y < z in
+  // lexicographic order (xyz xzy yxz yzx zxy zyx), added up in registers
+  for (int p = 0; p < NCOL / 6; ++p) {
+    for (int ab = 0; ab < 4; ++ab) {
+      if (!w[ab]) continue;
+      const int a = ab >> 1, b = ab & 1;
+      cx<double> acc[6] = {};
+      if constexpr (K >= 4) {
+        cx<double> s[4];
+        V.ld(V.offPsi(K - 3, p, a), s);
+        constexpr int c3[3] = {0, 1, 2}, r3[3] = {5, 3, 4};   // J(xyz) = J(zyx), ...
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          cx<double> X[4];
+          V.ld(V.offX(t->g3[p][i], b), X);
+          v2::sdot_acc(acc[c3[i]], s, X, false);
+          acc[r3[i]] = acc[c3[i]];
+        }
+        constexpr int cy[3] = {0, 1, 3}, ry[3] = {2, 4, 5};   // (xy)z, (xz)y, (yz)x: J(yx) = -J(xy)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          cx<double> Y[4], v = {};
+          V.ld(V.offY(t->gy[p][i][0], t->gy[p][i][1], b), Y);
+          v2::sdot_acc(v, s, Y, false);
+          acc[cy[i]].r += v.r; acc[cy[i]].i += v.i;
+          acc[ry[i]].r -= v.r; acc[ry[i]].i -= v.i;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        cx<double> s[4];
+        V.ld(V.offPsi(K - 2, 3 * p + i, a), s);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int z = t->gz[p][2 * i + q];
+          cx<double> Z[4];
+          V.ld(V.offZ(z / kMaxGluons, z % kMaxGluons, b), Z);
+          v2::sdot_acc(acc[2 * i + q], s, Z, false);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < 6; ++c) add(ab, 6 * p + c, acc[c], false);
+    }
+  }
+
+  if constexpr (MODE == kJamps) {
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab) {
+      float2* row = jout + (e * (2 << K) + slot * 4 + ab) * NCOL;
+      for (int c = 0; c < NCOL; ++c)
+        row[c] = w[ab] ? make_float2(static_cast<float>(A[ab][c].r), static_cast<float>(A[ab][c].i)) : make_float2(0.f, 0.f);
+    }
+  } else {
+    if constexpr (MODE == kLhe) {
+      const double d[4] = {static_cast<double>(w[0]), static_cast<double>(w[1]), static_cast<double>(w[2]),
+                           static_cast<double>(w[3])};
+      for (int c = 0; c < NCOL; ++c) {
+        double s = 0.0;
+#pragma unroll
+        for (int ab = 0; ab < 4; ++ab) s = fma(d[ab], fma(A[ab][c].r, A[ab][c].r, A[ab][c].i * A[ab][c].i), s);
+        j2[(static_cast<int64_t>(slot) * NCOL + c) * stride + e] = s;
+      }
+    }
+    double total = 0.0;
+    for (int ab = 0; ab < 4; ++ab) {
+      double v = 0.0;
+      if (w[ab]) v = v2::colour_sum<NCOL, double>(A[ab], ctri) * cst.colour_scale;
+      if constexpr (MODE == kLhe) out[(slot * 4 + ab) * stride + e] = v;
+      else total += w[ab] > 1 ? v + v : v;
+    }
+    if constexpr (MODE == kME) out[slot * stride + e] = total;
+  }
+}
+
+// Thread -> (event, slot) of the launch shape (as k_me_gluonhel); share = null: LOCAL.
+template <int K, int MODE, bool LOCAL>
+__device__ __forceinline__ void thread64(const double* __restrict__ rec, int64_t e, int slot, int gc,
+                                         const Tables* __restrict__ tab, const Tab64* __restrict__ t64,
+                                         const uint32_t* __restrict__ mask, const double* __restrict__ ctri,
+                                         const MeConst& cst, double* __restrict__ out, int64_t stride,
+                                         float2* __restrict__ jout, const double* __restrict__ share,
+                                         double* __restrict__ j2) {
+  View<K, LOCAL> V;
+  V.in = rec + (e / kPage) * v2::EvLayout<K>::NITEM * kPage + (e % kPage);
+  V.tab = tab;
+  V.t = t64;
+  V.o = LOCAL ? &t64->loc : &t64->sh;
+  V.gc = gc;
+  V.gs = cst.gs;
+  if constexpr (LOCAL) {
+    double own[Loc<K>::n];
+    V.buf = own;
+    for (int i = 0; i < t64->nltask; ++i) run_task<K, true>(V, t64->ltask[i]);
+    slot64<K, MODE, true>(V, e, slot, mask, ctri, cst, out, stride, jout, j2);
+  } else {
+    V.buf = const_cast<double*>(share) + (e / kPage) * static_cast<int64_t>(t64->stride) * kPage + (e % kPage);
+    slot64<K, MODE, false>(V, e, slot, mask, ctri, cst, out, stride, jout, j2);
+  }
+}
+
+}  // namespace m64
+}  // namespace mg

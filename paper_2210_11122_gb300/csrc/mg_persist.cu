@@ -6,10 +6,11 @@
 // thread blocks drain a common queue of work tiles than as one launch per job.  Here the queue holds
 // (job, gluon-helicity slot, 128-event tile) triples, the jobs ordered by falling cost per tile (more
 // gluons first, so the longest tiles start first); each 128-thread block takes the next tile from an
-// atomic counter until the queue is empty, and runs the same per-thread FP64 work as k_me_gluonhel (the
-// per-event record from k_event_prep; the currents and quark-line prefixes shared between a job's
-// gluon-helicity combinations from its k_share_level / k_prefix_level passes where its context's FP64
-// shape shares them and the job's buffer fits 2 GiB, else built in the thread).  The results are
+// atomic counter until the queue is empty, and runs the same per-thread FP64 work as the
+// single-job kernels (the
+// per-event record from k_event_prep; the items shared between a job's gluon-helicity combinations from its
+// launch_pass64 where its context's FP64 shape shares them and the job's buffer fits 2 GiB, else built in
+// the thread).  The results are
 // bit-identical to mg_sigmakin(MG_FP64), with or without the shared currents.
 #include <cuda_runtime.h>
 
@@ -21,6 +22,7 @@
 #include "mg_ctx.h"
 #include "mg_internal.h"
 #include "mg_kernels.h"
+#include "mg_me64.cuh"
 #include "mg_me_kernel.cuh"
 
 namespace mg {
@@ -36,7 +38,8 @@ struct PJob {
   const int* nslot;
   const uint32_t* mask;
   const double* ctri;
-  const double* share;      // the job's shared currents and prefixes (k_share_level), or null: none
+  const Tab64* t64;
+  const double* share;      // the job's shared items (launch_pass64), or null: every combination on its own
   double* part;             // part[slot * stride + e]
   int64_t nevt, stride, tile0;
   int K, ntile_ev;
@@ -48,6 +51,16 @@ struct PBatch {
   int64_t ntiles;
   PJob job[kMaxJobs];
 };
+
+template <int K>
+__device__ __forceinline__ void run64(const PJob& J, int64_t e, int slot, int gc) {
+  if (J.share)
+    m64::thread64<K, m64::kME, false>(J.rec, e, slot, gc, J.tab, J.t64, J.mask, J.ctri, J.cst, J.part, J.stride, nullptr,
+                                      J.share, nullptr);
+  else
+    m64::thread64<K, m64::kME, true>(J.rec, e, slot, gc, J.tab, J.t64, J.mask, J.ctri, J.cst, J.part, J.stride, nullptr,
+                                     nullptr, nullptr);
+}
 
 __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_constant__ PBatch b,
                                                               unsigned long long* __restrict__ next) {
@@ -70,44 +83,14 @@ __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_co
     const int64_t e = (t - static_cast<int64_t>(slot) * J.ntile_ev) * kTileEv + threadIdx.x;
     if (e >= J.nevt || slot >= *J.nslot) continue;
     const int gc = J.gslots[slot];
-    if (J.share) {
-      switch (J.K) {
-        case 2:
-          v2::me_slot<2, double, false, true, false, true>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst,
-                                                           J.part, J.stride, nullptr, 0, J.share, nullptr);
-          break;
-        case 3:
-          v2::me_slot<3, double, false, true, false, true>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst,
-                                                           J.part, J.stride, nullptr, 0, J.share, nullptr);
-          break;
-        case 4:
-          v2::me_slot<4, double, false, true, false, true>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst,
-                                                           J.part, J.stride, nullptr, 0, J.share, nullptr);
-          break;
-        default:
-          v2::me_slot<5, double, false, true, false, true>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst,
-                                                           J.part, J.stride, nullptr, 0, J.share, nullptr);
-          break;
-      }
-      continue;
-    }
     switch (J.K) {
       case 2:
         v2::me_slot<2, double, false, true, false>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst, J.part,
-                                                   J.stride, nullptr, 0, nullptr, nullptr);
+                                                   J.stride, nullptr, 0, nullptr);
         break;
-      case 3:
-        v2::me_slot<3, double, false, true, false>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst, J.part,
-                                                   J.stride, nullptr, 0, nullptr, nullptr);
-        break;
-      case 4:
-        v2::me_slot<4, double, false, true, false>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst, J.part,
-                                                   J.stride, nullptr, 0, nullptr, nullptr);
-        break;
-      default:
-        v2::me_slot<5, double, false, true, false>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst, J.part,
-                                                   J.stride, nullptr, 0, nullptr, nullptr);
-        break;
+      case 3: run64<3>(J, e, slot, gc); break;
+      case 4: run64<4>(J, e, slot, gc); break;
+      default: run64<5>(J, e, slot, gc); break;
     }
   }
 }
@@ -170,20 +153,21 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     cst.conj = 1;   // one of each pair of flipped helicities
     cst.colour_scale = cst.gs * cst.gs / static_cast<double>(c->colour_den);
     if (mg::launch_event_prep(c->K, false, j.mom_dev, j.nevt, cst, c->d_prep, st) != cudaSuccess) { s = MG_ECUDA; break; }
-    // the job's currents and quark-line prefixes shared between its gluon-helicity combinations, where its
+    // the job's items shared between its gluon-helicity combinations, where its
     // context's FP64 shape asks for them and the whole job's buffer stays within 2 GiB
     const double* share = nullptr;
     const int64_t sdoubles = stride * mg::share_doubles(c->K);
-    if (c->shape[MG_FP64].shared && sdoubles <= (int64_t(1) << 28)) {
+    if (c->shape[MG_FP64].shared && c->K >= 3 && sdoubles <= (int64_t(1) << 28)) {
       s = grow_d(&c->d_share, &c->share_cap, sdoubles);
       if (s != MG_OK) break;
-      if (mg::launch_share(c->K, c->d_prep, j.nevt, c->d_tab, cst, c->d_share, st) != cudaSuccess) { s = MG_ECUDA; break; }
+      if (mg::launch_pass64(c->K, c->d_prep, j.nevt, c->d_tab, c->d_tab64, cst, c->d_share, st) != cudaSuccess) { s = MG_ECUDA; break; }
       share = c->d_share;
     }
     mg::pers::PJob& p = batch->job[batch->njobs++];
     p.share = share;
     p.rec = c->d_prep;
     p.tab = c->d_tab;
+    p.t64 = c->d_tab64;
     p.gslots = c->d_hslots;
     p.nslot = c->d_nhslots;
     p.mask = c->d_mask;

@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <numeric>
 #include <vector>
 
@@ -56,21 +57,6 @@ void build_tables(int K, Tables& t) {
       if (s.front() < s.back()) { slot_of[s] = static_cast<int>(seqs.size()); seqs.push_back(s); }
   }
   t.nseq = static_cast<int>(seqs.size());
-  t.share_n = 0;
-  for (int i = 0; i < t.nseq; ++i) {
-    t.share_base[i] = static_cast<int16_t>(t.share_n);
-    t.share_n += 1 << seqs[i].size();
-  }
-  t.pref_levels = K - 1 < 3 ? K - 1 : 3;
-  int nodes = 0;
-  for (int m = 0; m < kMaxGluons; ++m) t.pref_off[m] = 0;
-  for (int m = 1; m <= t.pref_levels; ++m) {
-    int orderings = 1;   // ordered prefixes of m gluons: K! / (K - m)!
-    for (int i = 0; i < m; ++i) orderings *= K - i;
-    t.pref_off[m] = nodes;
-    nodes += (orderings << m) * 2;
-  }
-  t.share_stride = t.share_n * 24 + nodes * 8;
   auto ref = [&](const std::vector<int>& s) -> int16_t {
     if (s.size() == 1) return pack(s[0], false);
     if (s.front() < s.back()) return pack(slot_of.at(s), false);
@@ -149,6 +135,140 @@ void build_tables(int K, Tables& t) {
       t.full_idx[c] = static_cast<int16_t>(-full_of.at(r) - 1);
     }
   }
+}
+
+void build_tab64(int K, const Tables& t, Tab64& o) {
+  std::memset(&o, 0, sizeof(o));
+  o.K = K;
+  const int top = 1 << (K - 1);
+  auto nh = [&](int mask) { return 1 << __builtin_popcount(mask & (top - 1)); };
+  auto fact = [](int n) { return factorial(n); };
+  // ---- offsets: per helicity assignment (shared buffer) and for one assignment (a combination's own items) ----
+  for (int own = 0; own < 2; ++own) {
+    Tab64::Off& f = own ? o.loc : o.sh;
+    int at = 0;
+    auto take = [&](int mask, int entries) { const int r = at; at += 8 * entries * (own ? 1 : nh(mask)); return r; };
+    std::memset(&f, 0xff, sizeof(f));   // -1: none
+    for (int s = 0; s < t.nseq; ++s) {
+      f.J[s] = take(t.seq_mask[s], 1);
+      if (t.seq_len[s] >= 3) f.X[s] = take(t.seq_mask[s], 2);
+    }
+    for (int m = 1; m <= K - 2; ++m)
+      for (int p = 0; p < t.ncol / fact(K - m); ++p) f.psi[m][p] = take(t.prefix_mask[p * fact(K - m)][m], 2);
+    for (int g = 0; g < K; ++g) {
+      f.chi[g] = take(1 << g, 2);
+      f.qg[g] = take(1 << g, 4);
+    }
+    f.q0 = take(0, 4);
+    for (int g = 0; g < K; ++g)
+      for (int h = 0; h < K; ++h) {
+        if (g == h) continue;
+        f.z[g * kMaxGluons + h] = take(1 << g | 1 << h, 2);
+        if (K == 5) f.qq[g * kMaxGluons + h] = take(1 << g | 1 << h, 4);
+      }
+    if (K >= 4)
+      for (int s = 0; s < t.nseq; ++s)
+        for (int g = 0; g < K; ++g)
+          if (t.seq_len[s] == 2 && !((t.seq_mask[s] >> g) & 1)) f.y[s][g] = take(t.seq_mask[s] | 1 << g, 2);
+    (own ? o.nloc : o.stride) = at;
+  }
+  // ---- tasks ----
+  int nt = 0;
+  o.nltask = 0;
+  auto tasks = [&](Tab64::Type type, int a, int b, int mask) {
+    const uint32_t base = static_cast<uint32_t>(type) | static_cast<uint32_t>(a) << 4 | static_cast<uint32_t>(b) << 14;
+    o.ltask[o.nltask++] = base;
+    for (int gc = 0; gc < top; ++gc)
+      if ((gc & ~mask) == 0) o.task[nt++] = base | static_cast<uint32_t>(gc) << 20;
+  };
+  auto seqs = [&](Tab64::Type type, int len) {
+    for (int s = 0; s < t.nseq; ++s)
+      if (t.seq_len[s] == len) tasks(type, s, 0, t.seq_mask[s]);
+  };
+  auto psis = [&](int m) {
+    for (int p = 0; p < t.ncol / fact(K - m); ++p) tasks(Tab64::kPsi, p, m, t.prefix_mask[p * fact(K - m)][m]);
+  };
+  auto next_pass = [&] { o.pass0[++o.npass] = nt; };
+  for (int g = 0; g < K; ++g) tasks(Tab64::kJ1, g, 0, 1 << g);
+  tasks(Tab64::kJq0, 0, 0, 0);
+  psis(1);
+  if (K == 3) next_pass();   // (three gluons: four short passes instead of two)
+  for (int g = 0; g < K; ++g) tasks(Tab64::kChi, g, 0, 1 << g);
+  next_pass();
+  seqs(Tab64::kSeq, 2);
+  if (K == 5)
+    for (int g = 0; g < K; ++g)
+      for (int h = 0; h < K; ++h)
+        if (g != h) tasks(Tab64::kQQ, g, h, 1 << g | 1 << h);
+  next_pass();
+  if (K >= 4) {
+    seqs(Tab64::kSeq, 3);
+    for (int s = 0; s < t.nseq; ++s)
+      for (int g = 0; g < K; ++g)
+        if (o.sh.y[s][g] >= 0) tasks(Tab64::kY, s, g, t.seq_mask[s] | 1 << g);
+    psis(2);
+  }
+  seqs(Tab64::kZ, 2);
+  next_pass();
+  if (K == 5) {
+    seqs(Tab64::kSeq, 4);
+    psis(3);
+    next_pass();
+  }
+  // ---- terms of the amplitudes ----
+  std::vector<int> p(K);
+  std::iota(p.begin(), p.end(), 0);
+  std::map<std::vector<int>, int> rank;
+  std::vector<std::vector<int>> perms;
+  do { rank[p] = static_cast<int>(perms.size()); perms.push_back(p); } while (std::next_permutation(p.begin(), p.end()));
+  auto reversed = [&](int c, int i, int j) {   // the ordering with positions [i, j) reversed
+    std::vector<int> q = perms[c];
+    std::reverse(q.begin() + i, q.begin() + j);
+    return rank.at(q);
+  };
+  int n1 = 0, n2 = 0, n3 = 0;
+  for (int c = 0; c < t.ncol; ++c) {
+    const std::vector<int>& s = perms[c];
+    if (t.full_idx[c] >= 0) {
+      o.full_c[t.full_idx[c]] = static_cast<int16_t>(c);
+      o.full_cr[t.full_idx[c]] = static_cast<int16_t>(reversed(c, 0, K));
+    }
+    auto entry = [&](int16_t* e, int i, int j, int key) {
+      e[0] = static_cast<int16_t>(t.sub[c][i][j] >> 1);
+      e[1] = static_cast<int16_t>(key);
+      e[2] = static_cast<int16_t>(c);
+      e[3] = static_cast<int16_t>(reversed(c, i, j));
+    };
+    if (s[0] < s[K - 2]) entry(o.t1[n1++], 0, K - 1, s[K - 1]);
+    if (K == 5 && s[1] < s[4]) entry(o.t2[n2++], 1, 5, s[0]);
+    if (K == 5 && s[1] < s[3]) entry(o.t3[n3++], 1, 4, s[0] * kMaxGluons + s[4]);
+  }
+  for (int g = 0; g < t.ncol / 6; ++g)
+    for (int i = 0; i < 6; ++i) {
+      const int c = 6 * g + i;
+      const std::vector<int>& s = perms[c];
+      o.gz[g][i] = static_cast<int16_t>(s[K - 2] * kMaxGluons + s[K - 1]);
+      if (K >= 4) {
+        if (i < 3) o.g3[g][i] = static_cast<int16_t>(t.sub[c][K - 3][K] >> 1);
+        const int y = i == 0 ? 0 : i == 1 ? 1 : i == 3 ? 2 : -1;
+        if (y >= 0) {
+          o.gy[g][y][0] = static_cast<int16_t>(t.sub[c][K - 3][K - 1] >> 1);
+          o.gy[g][y][1] = static_cast<int16_t>(s[K - 1]);
+        }
+      }
+    }
+}
+
+const Tab64& tab64_host(int K) {
+  static Tab64 tabs[kMaxGluons + 1];
+  static std::once_flag once[kMaxGluons + 1];
+  std::call_once(once[K], [K] {
+    Tables* t = new Tables;
+    build_tables(K, *t);
+    build_tab64(K, *t, tabs[K]);
+    delete t;
+  });
+  return tabs[K];
 }
 
 }  // namespace mg
