@@ -192,6 +192,11 @@ cudaError_t fp64_slots(mg_ctx* ctx, const double* mom, const double* rec, int64_
                      out, stride, jout, shape, shared ? ctx->d_share : nullptr, nullptr, st);
 }
 
+cudaError_t fp64_hel_sum(mg_ctx* ctx, int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st) {
+  if (ctx->K == 2) return launch_hel_sum(ctx->d_part, ctx->d_nhslots, nevt, stride, norm, me, st);
+  return launch_hel_sum_rows(ctx->K, ctx->d_part, ctx->d_hslots, ctx->d_nhslots, ctx->d_mask, nevt, stride, norm, me, st);
+}
+
 bool mixed_in_kernel(const mg_ctx* ctx, mg_precision precision) {
   return precision == MG_MIXED && ctx->prm.wt == 0.0 && ctx->shape[precision].warp &&
          !ctx->shape[precision].tc_apart && me_warp_available(ctx->K, true);
@@ -730,7 +735,7 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
                                        ctx->d_part, cst_stride, st, fp32 ? ctx->d_flag : nullptr, ctx->d_tcerr,
                                        ctx->tc_stall));
       if (fp32) MG_CUDA(join_repair(ctx, st));
-      if (half)
+      if (half)   // (the colour pass writes a row per helicity for every process)
         MG_CUDA(mg::launch_hel_sum_rows(ctx->K, ctx->d_part, slots, nslots, ctx->d_mask, n, cst_stride, norm, me_dev + e0, st));
       else
         MG_CUDA(mg::launch_hel_sum(ctx->d_part, ctx->d_nrows, n, cst_stride, norm, me_dev + e0, st));
@@ -776,7 +781,8 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
                                      maxslot, nslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part,
                                      stride, st, nullptr, ctx->shape[precision], ctx->d_flag));
     if (fp32) MG_CUDA(join_repair(ctx, st));
-    MG_CUDA(mg::launch_hel_sum(ctx->d_part, nslots, nevt, stride, norm, me_dev, st));
+    MG_CUDA(half ? mg::fp64_hel_sum(ctx, nevt, stride, norm, me_dev, st)
+                 : mg::launch_hel_sum(ctx->d_part, nslots, nevt, stride, norm, me_dev, st));
   } else {
     MG_CUDA(mg::launch_me_helicity(ctx->K, precision == MG_FP32_AMP, mom_dev, nevt, ctx->d_tab, ctx->d_good, ctx->nhel,
                                    ctx->d_ngood, ctx->d_ctri, cst, ctx->d_part, stride, st));

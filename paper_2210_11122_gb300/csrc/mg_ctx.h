@@ -84,6 +84,8 @@ int64_t share_chunk(int K, int64_t stride);
 // (d_share, share_doubles(K) * pad(n) doubles, 3 to 5 gluons), else every combination on its own.
 cudaError_t fp64_slots(mg_ctx* ctx, const double* mom, const double* rec, int64_t n, bool shared, const MeConst& cst,
                        double* out, int64_t stride, float2* jout, MeShape shape, cudaStream_t st);
+// The helicity sum of fp64_slots' colour sums in d_part (per combination for 2 gluons, per helicity for 3 to 5).
+cudaError_t fp64_hel_sum(mg_ctx* ctx, int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st);
 // MG_MIXED on the lane-group kernel: colour sums on the tensor cores inside it, per-slot outputs
 bool mixed_in_kernel(const mg_ctx* ctx, mg_precision precision);
 mg_status ctx_reserve(mg_ctx* ctx, int64_t nevt, mg_precision precision);

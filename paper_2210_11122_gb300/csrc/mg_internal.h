@@ -78,8 +78,8 @@ void build_tables(int K, Tables& t);
 // pext_bits order; entries are 8 doubles (4 complex) times what the comment says.
 // ----------------------------------------------------------------------------------------
 struct Tab64 {
-  enum Type { kJ1, kJq0, kChi, kPsi, kSeq, kZ, kY, kQQ };
-  static constexpr int kMaxTask = 1500, kMaxLTask = 260, kMaxPass = 5;
+  enum Type { kJ1, kJq0, kChi, kPsi, kSeq, kZ, kY, kFull, kQQ };
+  static constexpr int kMaxTask = 2500, kMaxLTask = 320, kMaxPass = 6;
   struct Off {
     int J[kMaxSeq];                        // current of a canonical sequence (1)
     int X[kMaxSeq];                        // (gamma.J) v, three or more gluons (antitop helicity: 2); -1: none
@@ -89,6 +89,7 @@ struct Tab64 {
     int q0;                                // ubar gamma^mu v (4)
     int z[kMaxGluons * kMaxGluons];        // last two gluons (2)
     int y[kMaxSeq][kMaxGluons];            // (gamma.J_pair) chi(g) (2); -1: none
+    int full[kMaxNcol / 2];                // ubar gamma^mu v times a canonical full current (4 complex numbers)
     int qq[kMaxGluons * kMaxGluons];       // psi_1(g) gamma^mu chi(h), 5 gluons (4)
   };
   int K, stride, nloc;                     // doubles per event of the shared buffer, of one combination's own items
@@ -98,9 +99,10 @@ struct Tab64 {
   int nltask;
   uint32_t ltask[kMaxLTask];               // the same tasks without helicities, in an order that respects dependences
   int16_t full_c[kMaxNcol / 2], full_cr[kMaxNcol / 2];   // orderings of a full current and of its reversal
-  int16_t t1[kMaxNcol / 2][4];             // sequence of K-1 gluons, last gluon, ordering, ordering reversed in the sequence
-  int16_t t2[kMaxNcol / 2][4];             // 5 gluons: sequence of the last 4, first gluon, ordering, reversed
-  int16_t t3[kMaxNcol / 2][4];             // 5 gluons: sequence of the middle 3, first * 5 + last gluon, ordering, reversed
+  int16_t t1[kMaxNcol / 2][3];             // by last gluon: sequence of K-1, ordering, ordering reversed in the sequence
+  int16_t t2[kMaxNcol / 2][3];             // 5 gluons, by first gluon: sequence of the last 4, ordering, reversed
+  int16_t t3[kMaxNcol / 2][3];             // 5 gluons, by (first, last) gluon: sequence of the middle 3, ordering, reversed
+  int16_t t3q[kMaxGluons * (kMaxGluons - 1)][2];   // t3's (first, last) gluons, three entries each
   int16_t g3[kMaxNcol / 6][3];             // six orderings with a common prefix of K-3: sequences xyz, xzy, yxz
   int16_t gy[kMaxNcol / 6][3][2];          // (pair, last): (xy, z), (xz, y), (yz, x)
   int16_t gz[kMaxNcol / 6][6];             // last two gluons, first * 5 + second, of the six orderings

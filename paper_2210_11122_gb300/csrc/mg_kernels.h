@@ -83,10 +83,10 @@ cudaError_t launch_me_gluonhel(int K, bool fp32, bool per_hel, const double* mom
                                const int* evlist = nullptr, const int* nlist = nullptr, int rows_out = 0);
 // FP64 matrix elements of 3 to 5 gluons from the FP64 records of nevt events (mg_me64.cuh).  launch_pass64 fills the
 // items shared between gluon-helicity combinations (tab64_host(K).stride doubles per event, page-interleaved), a
-// few launches; launch_me64 runs one thread per (event, combination hslots[slot]), reading them, or with share = null
-// computing its own (the same bits).  Output: out[slot * stride + e] the weighted sum over the combination's
-// helicities (cst.conj = 1); or, with jout, FP32 jamps in rows of 2 * 2^K per event; or, with j2, the colour sum of
-// every helicity in rows slot * 4 + 2 top + antitop and the weighted jamp squares j2[(slot * ncol + sigma) * stride + e].
+// few launches; launch_me64 runs one thread per (event, helicity of the combinations hslots), reading them, or with
+// share = null one per (event, combination) computing its own (the same bits).  Output, rows r = slot * 4 + 2 top +
+// antitop (cst.conj = 1): the colour sums out[r * stride + e], zero for weight 0; with jout the FP32 jamps instead (2^(K+1)
+// rows per event); with j2 also the weighted jamp squares j2[(r * ncol + sigma) * stride + e].
 cudaError_t launch_pass64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const MeConst& cst,
                           double* share, cudaStream_t st);
 cudaError_t launch_me64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const int* hslots,

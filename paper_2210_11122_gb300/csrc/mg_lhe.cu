@@ -63,7 +63,8 @@ __device__ __forceinline__ double coupling_factor(double a0, double mu, double* 
 }
 
 // One thread per event: helicity sum (ascending helicity index), helicity and colour choices, coupling.
-// part rows: slot * 4 + 2 top + antitop (launch_me64 with j2); j2: per-slot jamp-square sums.
+// part rows: slot * 4 + 2 top + antitop (launch_me64 with j2); j2: jamp-square sums, per
+// helicity row (3 to 5 gluons) or per slot (2).
 template <int K>
 __global__ void __launch_bounds__(128)
 k_lhe_epilogue(const double* __restrict__ part, const double* __restrict__ j2, const int* __restrict__ gslots,
@@ -116,7 +117,7 @@ k_lhe_epilogue(const double* __restrict__ part, const double* __restrict__ j2, c
     double totc = 0.0;
     for (int c = 0; c < NCOL; ++c) {
       double acc = 0.0;
-      for (int s = 0; s < nslot; ++s) acc += j2[(static_cast<int64_t>(s) * NCOL + c) * stride + e];
+      for (int s = 0; s < (K >= 3 ? 4 * nslot : nslot); ++s) acc += j2[(static_cast<int64_t>(s) * NCOL + c) * stride + e];
       w[c] = acc;
       totc += acc;
     }
@@ -224,7 +225,7 @@ mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, cons
   ctx->last = st;
   const int K = ctx->K;
   // chunks of whole pages that keep the per-slot jamp-square sums within 2^27 doubles (1 GiB)
-  const int64_t per_event = static_cast<int64_t>(1 << (K - 1)) * ctx->ncol;
+  const int64_t per_event = static_cast<int64_t>(K >= 3 ? ctx->nhel / 2 : 1 << (K - 1)) * ctx->ncol;
   int64_t chunk = (int64_t(1) << 27) / per_event / mg::kPage * mg::kPage;
   const int64_t stride_all = pad_page(nevt);
   if (chunk < mg::kPage) chunk = mg::kPage;

@@ -37,9 +37,9 @@ __device__ constexpr int kFact[6] = {1, 1, 2, 6, 24, 120};
 
 // doubles of one combination's own items (LOCAL)
 template <int K> struct Loc;
-template <> struct Loc<3> { static constexpr int n = 368; };
-template <> struct Loc<4> { static constexpr int n = 1232; };
-template <> struct Loc<5> { static constexpr int n = 5352; };
+template <> struct Loc<3> { static constexpr int n = 392; };
+template <> struct Loc<4> { static constexpr int n = 1328; };
+template <> struct Loc<5> { static constexpr int n = 5832; };
 
 // (Qslash + m) f on a column spinor, coefficients as row_prop's
 __device__ __forceinline__ void col_prop(const cx<double>* s, const double* q, cx<double>* o) {
@@ -122,6 +122,7 @@ struct View {
   __device__ __forceinline__ int offQQ(int g, int g2, int ab) const {
     return o->qq[g * kMaxGluons + g2] + (h(1 << g | 1 << g2) * 4 + ab) * 8;
   }
+  __device__ __forceinline__ int offFull(int f) const { return o->full[f] + h((1 << K) - 1) * 8; }
   __device__ __forceinline__ void J(int s, cx<double>* v) const { ld(offJ(s), v); }
 
   // current of a canonical split list: three- and four-gluon vertices summed
@@ -273,6 +274,22 @@ __device__ __forceinline__ void run_task(const View<K, LOCAL>& V, uint32_t task)
       }
       break;
     }
+    case Tab64::kFull: {   // all gluons on one current, contracted with the four quark currents: 4 complex numbers
+      cx<double> acc[4] = {}, x[4];
+      V.vertices(acc, V.tab->full_nv3[a_], V.tab->full_v3[a_], V.tab->full_nv4[a_], V.tab->full_v4[a_]);
+      const double f = V.rec(L::GP + (1 << K) - 1);
+      cx<double> JF[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) JF[m] = v2::cscale(f, acc[m]);
+#pragma unroll
+      for (int ab = 0; ab < 4; ++ab) {
+        cx<double> Jq[4];
+        V.ld(V.o->q0 + ab * 8, Jq);
+        x[ab] = v2::mdot(Jq, JF);
+      }
+      V.st(V.offFull(a_), x);
+      break;
+    }
     case Tab64::kY: {   // (gamma.J_s) chi(g)
       cx<double> J[4];
       V.J(a_, J);
@@ -325,184 +342,156 @@ k_pass64(const double* __restrict__ rec, int64_t nevt, const Tables* __restrict_
 
 constexpr int kME = 0, kJamps = 1, kLhe = 2;
 
-// The amplitudes of one (event, combination) for the four top helicity pairs and what the mode makes of them:
-// kME: out[slot * stride + e] = the weighted sum of the colour sums; kJamps: FP32 jamps, rows slot * 4 + 2 top +
-// antitop of jout (zeros for weight 0); kLhe: the colour sum of every helicity in its own row of out (zero for
-// weight 0) and the weighted |jamp|^2 of every ordering in j2.
+// The amplitudes of one (event, combination, top helicity pair ab = 2 top + antitop) and what the mode makes of them,
+// in row slot * 4 + ab: kME: out[row * stride + e] = the colour sum (0 for weight 0); kJamps: FP32 jamps of jout's
+// row (zeros for weight 0); kLhe: kME and j2[(row * ncol + sigma) * stride + e] = weight * |jamp|^2.
 template <int K, int MODE, bool LOCAL>
-__device__ __forceinline__ void slot64(const View<K, LOCAL>& V, int64_t e, int slot, const uint32_t* __restrict__ mask,
-                                       const double* __restrict__ ctri, const MeConst& cst, double* __restrict__ out,
-                                       int64_t stride, float2* __restrict__ jout, double* __restrict__ j2) {
-  using L = v2::EvLayout<K>;
-  constexpr int npar = K + 2, NCOL = v2::Sizes<K>::ncol, NFULL = v2::Sizes<K>::nfull, NSUB = 1 << K;
+__device__ __forceinline__ void slot64(const View<K, LOCAL>& V, int64_t e, int slot, int ab,
+                                       const uint32_t* __restrict__ mask, const double* __restrict__ ctri,
+                                       const MeConst& cst, double* __restrict__ out, int64_t stride,
+                                       float2* __restrict__ jout, double* __restrict__ j2) {
+  constexpr int npar = K + 2, NCOL = v2::Sizes<K>::ncol, NFULL = v2::Sizes<K>::nfull;
   constexpr bool kNegK = (K & 1) == 0, kNegK1 = !kNegK;   // reflection signs of K and K-1 gluons: negative?
-  const Tables* tab = V.tab;
   const Tab64* t = V.t;
-  int w[4];
-  {
-    int hb = 0;
+  const int a = ab >> 1, b = ab & 1, row = slot * 4 + ab;
+  int hb = (a << (npar - 3)) | (b << (npar - 4));
 #pragma unroll
-    for (int g = 0; g < K; ++g)
-      if ((V.gc >> g) & 1) hb |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
-#pragma unroll
-    for (int ab = 0; ab < 4; ++ab)
-      w[ab] = hel_weight(mask, hb | ((ab >> 1) << (npar - 3)) | ((ab & 1) << (npar - 4)), npar, cst.conj);
-  }
-  cx<double> A[4][NCOL];
-  // all gluons on one current, contracted with the four quark currents
-  {
-    const double fz = V.rec(L::GP + NSUB - 1);
-    for (int f = 0; f < NFULL; ++f) {
-      cx<double> acc[4] = {}, JF[4];
-      V.vertices(acc, tab->full_nv3[f], tab->full_v3[f], tab->full_nv4[f], tab->full_v4[f]);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) JF[m] = v2::cscale(fz, acc[m]);
-      const int c = t->full_c[f], cr = t->full_cr[f];
-#pragma unroll
-      for (int ab = 0; ab < 4; ++ab) {
-        cx<double> Jq[4];
-        V.ld(V.o->q0 + ab * 8, Jq);
-        const cx<double> x = v2::mdot(Jq, JF);
-        A[ab][c] = x;
-        A[ab][cr] = kNegK ? v2::cneg(x) : x;
-      }
+  for (int g = 0; g < K; ++g)
+    if ((V.gc >> g) & 1) hb |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
+  const int w = hel_weight(mask, hb, npar, cst.conj);
+  if (!w) {
+    if constexpr (MODE == kJamps) {
+      for (int c = 0; c < NCOL; ++c) jout[(e * (2 << K) + row) * NCOL + c] = make_float2(0.f, 0.f);
+    } else {
+      out[row * stride + e] = 0.0;
+      if constexpr (MODE == kLhe)
+        for (int c = 0; c < NCOL; ++c) j2[(static_cast<int64_t>(row) * NCOL + c) * stride + e] = 0.0;
     }
+    return;
   }
-  auto add = [&](int ab, int c, cx<double> x, bool neg) {
-    A[ab][c].r = neg ? A[ab][c].r - x.r : A[ab][c].r + x.r;
-    A[ab][c].i = neg ? A[ab][c].i - x.i : A[ab][c].i + x.i;
+  cx<double> A[NCOL];
+  for (int f = 0; f < NFULL; ++f) {   // all gluons on one current
+    const double* p = V.buf + static_cast<int64_t>(V.offFull(f) + 2 * ab) * View<K, LOCAL>::ST;
+    const cx<double> x = {p[0], p[View<K, LOCAL>::ST]};
+    A[t->full_c[f]] = x;
+    A[t->full_cr[f]] = kNegK ? v2::cneg(x) : x;
+  }
+  auto add = [&](int c, cx<double> x, bool neg) {
+    A[c].r = neg ? A[c].r - x.r : A[c].r + x.r;
+    A[c].i = neg ? A[c].i - x.i : A[c].i + x.i;
   };
   // the first K-1 gluons on one current, the last on chi
-  for (int i = 0; i < NCOL / 2; ++i) {
-    const int s = t->t1[i][0], g = t->t1[i][1], c = t->t1[i][2], cr = t->t1[i][3];
-    cx<double> J[4];
-    V.J(s, J);
-#pragma unroll
-    for (int ab = 0; ab < 4; ++ab) {
-      cx<double> Jq[4];
-      V.ld(V.offQg(g, ab), Jq);
+  constexpr int NLAST = NCOL / 2 / K;
+  for (int g = 0; g < K; ++g) {
+    cx<double> Jq[4];
+    V.ld(V.offQg(g, ab), Jq);
+    for (int i = g * NLAST; i < (g + 1) * NLAST; ++i) {
+      cx<double> J[4];
+      V.J(t->t1[i][0], J);
       const cx<double> x = v2::mdot(Jq, J);
-      add(ab, c, x, false);
-      add(ab, cr, x, kNegK1);
+      add(t->t1[i][1], x, false);
+      add(t->t1[i][2], x, kNegK1);
     }
   }
   if constexpr (K == 5) {
-    // one gluon on the top, the other four on one current, or three of them and the last on chi
-    for (int i = 0; i < NCOL / 2; ++i) {
-      const int s = t->t2[i][0], g = t->t2[i][1], c = t->t2[i][2], cr = t->t2[i][3];
-      cx<double> X[2][4];
-#pragma unroll
-      for (int b = 0; b < 2; ++b) V.ld(V.offX(s, b), X[b]);
-#pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        cx<double> p[4];
-        V.ld(V.offPsi(1, g, a), p);
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          cx<double> x = {};
-          v2::sdot_acc(x, p, X[b], false);
-          add(2 * a + b, c, x, false);
-          add(2 * a + b, cr, x, true);
-        }
+    // one gluon on the top, the other four on one current
+    for (int g = 0; g < K; ++g) {
+      cx<double> s[4];
+      V.ld(V.offPsi(1, g, a), s);
+      for (int i = g * NLAST; i < (g + 1) * NLAST; ++i) {
+        cx<double> X[4], x = {};
+        V.ld(V.offX(t->t2[i][0], b), X);
+        v2::sdot_acc(x, s, X, false);
+        add(t->t2[i][1], x, false);
+        add(t->t2[i][2], x, true);
       }
     }
-    for (int i = 0; i < NCOL / 2; ++i) {
-      const int s = t->t3[i][0], g = t->t3[i][1] / kMaxGluons, g2 = t->t3[i][1] % kMaxGluons, c = t->t3[i][2],
-                cr = t->t3[i][3];
-      cx<double> J[4];
-      V.J(s, J);
+    // or three of them and the last on chi
+    for (int q = 0; q < K * (K - 1); ++q) {
+      cx<double> Jq[4];
+      V.ld(V.offQQ(t->t3q[q][0], t->t3q[q][1], ab), Jq);
 #pragma unroll
-      for (int ab = 0; ab < 4; ++ab) {
-        cx<double> Jq[4];
-        V.ld(V.offQQ(g, g2, ab), Jq);
+      for (int i = 0; i < 3; ++i) {
+        cx<double> J[4];
+        V.J(t->t3[3 * q + i][0], J);
         const cx<double> x = v2::mdot(Jq, J);
-        add(ab, c, x, false);
-        add(ab, cr, x, false);
+        add(t->t3[3 * q + i][1], x, false);
+        add(t->t3[3 * q + i][2], x, false);
       }
     }
   }
   // the orderings of the last three gluons after a common prefix: six consecutive orderings, x < y < z in
   // lexicographic order (xyz xzy yxz yzx zxy zyx), added up in registers
   for (int p = 0; p < NCOL / 6; ++p) {
-    for (int ab = 0; ab < 4; ++ab) {
-      if (!w[ab]) continue;
-      const int a = ab >> 1, b = ab & 1;
-      cx<double> acc[6] = {};
-      if constexpr (K >= 4) {
-        cx<double> s[4];
-        V.ld(V.offPsi(K - 3, p, a), s);
-        constexpr int c3[3] = {0, 1, 2}, r3[3] = {5, 3, 4};   // J(xyz) = J(zyx), ...
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          cx<double> X[4];
-          V.ld(V.offX(t->g3[p][i], b), X);
-          v2::sdot_acc(acc[c3[i]], s, X, false);
-          acc[r3[i]] = acc[c3[i]];
-        }
-        constexpr int cy[3] = {0, 1, 3}, ry[3] = {2, 4, 5};   // (xy)z, (xz)y, (yz)x: J(yx) = -J(xy)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          cx<double> Y[4], v = {};
-          V.ld(V.offY(t->gy[p][i][0], t->gy[p][i][1], b), Y);
-          v2::sdot_acc(v, s, Y, false);
-          acc[cy[i]].r += v.r; acc[cy[i]].i += v.i;
-          acc[ry[i]].r -= v.r; acc[ry[i]].i -= v.i;
-        }
-      }
+    cx<double> acc[6] = {};
+    if constexpr (K >= 4) {
+      cx<double> s[4];
+      V.ld(V.offPsi(K - 3, p, a), s);
+      constexpr int c3[3] = {0, 1, 2}, r3[3] = {5, 3, 4};   // J(xyz) = J(zyx), ...
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        cx<double> s[4];
-        V.ld(V.offPsi(K - 2, 3 * p + i, a), s);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int z = t->gz[p][2 * i + q];
-          cx<double> Z[4];
-          V.ld(V.offZ(z / kMaxGluons, z % kMaxGluons, b), Z);
-          v2::sdot_acc(acc[2 * i + q], s, Z, false);
-        }
+        cx<double> X[4];
+        V.ld(V.offX(t->g3[p][i], b), X);
+        v2::sdot_acc(acc[c3[i]], s, X, false);
+        acc[r3[i]] = acc[c3[i]];
       }
+      constexpr int cy[3] = {0, 1, 3}, ry[3] = {2, 4, 5};   // (xy)z, (xz)y, (yz)x: J(yx) = -J(xy)
 #pragma unroll
-      for (int c = 0; c < 6; ++c) add(ab, 6 * p + c, acc[c], false);
+      for (int i = 0; i < 3; ++i) {
+        cx<double> Y[4], v = {};
+        V.ld(V.offY(t->gy[p][i][0], t->gy[p][i][1], b), Y);
+        v2::sdot_acc(v, s, Y, false);
+        acc[cy[i]].r += v.r; acc[cy[i]].i += v.i;
+        acc[ry[i]].r -= v.r; acc[ry[i]].i -= v.i;
+      }
     }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      cx<double> s[4];
+      V.ld(V.offPsi(K - 2, 3 * p + i, a), s);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int z = t->gz[p][2 * i + q];
+        cx<double> Z[4];
+        V.ld(V.offZ(z / kMaxGluons, z % kMaxGluons, b), Z);
+        v2::sdot_acc(acc[2 * i + q], s, Z, false);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 6; ++c) add(6 * p + c, acc[c], false);
   }
 
   if constexpr (MODE == kJamps) {
-#pragma unroll
-    for (int ab = 0; ab < 4; ++ab) {
-      float2* row = jout + (e * (2 << K) + slot * 4 + ab) * NCOL;
-      for (int c = 0; c < NCOL; ++c)
-        row[c] = w[ab] ? make_float2(static_cast<float>(A[ab][c].r), static_cast<float>(A[ab][c].i)) : make_float2(0.f, 0.f);
-    }
+    float2* o = jout + (e * (2 << K) + row) * NCOL;
+    for (int c = 0; c < NCOL; ++c) o[c] = make_float2(static_cast<float>(A[c].r), static_cast<float>(A[c].i));
   } else {
-    if constexpr (MODE == kLhe) {
-      const double d[4] = {static_cast<double>(w[0]), static_cast<double>(w[1]), static_cast<double>(w[2]),
-                           static_cast<double>(w[3])};
-      for (int c = 0; c < NCOL; ++c) {
-        double s = 0.0;
-#pragma unroll
-        for (int ab = 0; ab < 4; ++ab) s = fma(d[ab], fma(A[ab][c].r, A[ab][c].r, A[ab][c].i * A[ab][c].i), s);
-        j2[(static_cast<int64_t>(slot) * NCOL + c) * stride + e] = s;
-      }
-    }
-    double total = 0.0;
-    for (int ab = 0; ab < 4; ++ab) {
-      double v = 0.0;
-      if (w[ab]) v = v2::colour_sum<NCOL, double>(A[ab], ctri) * cst.colour_scale;
-      if constexpr (MODE == kLhe) out[(slot * 4 + ab) * stride + e] = v;
-      else total += w[ab] > 1 ? v + v : v;
-    }
-    if constexpr (MODE == kME) out[slot * stride + e] = total;
+    if constexpr (MODE == kLhe)
+      for (int c = 0; c < NCOL; ++c)
+        j2[(static_cast<int64_t>(row) * NCOL + c) * stride + e] =
+            static_cast<double>(w) * fma(A[c].r, A[c].r, A[c].i * A[c].i);
+    out[row * stride + e] = v2::colour_sum<NCOL, double>(A, ctri) * cst.colour_scale;
   }
 }
 
-// Thread -> (event, slot) of the launch shape (as k_me_gluonhel); share = null: LOCAL.
+// A warp takes one top helicity pair of one combination (the all-gluon currents, which the pairs share, are items
+// of the last pass): a thread doing all four pairs made 4 times longer warps, of which gg->ttgg's 10,007 events are
+// 4.1 per sub-partition, so the busiest had 5; measured 2.81 vs 3.19 ms there, gg->ttggg + TC colour 7.60 vs 8.60 ms
+// per 2,049 events, gg->ttg 12.05 vs 12.13 ms per 524,288.
+// Events per block of 128 threads: with the shared items 32 (a page), one warp for each top helicity pair of a
+// combination; without them 128, a thread doing the four pairs with the items it has built.
+template <bool LOCAL> __host__ __device__ constexpr int events_per_block() { return LOCAL ? 128 : 32; }
+
+// One thread of a block on event tile `tile` of combination `slot`.
 template <int K, int MODE, bool LOCAL>
-__device__ __forceinline__ void thread64(const double* __restrict__ rec, int64_t e, int slot, int gc,
+__device__ __forceinline__ void thread64(const double* __restrict__ rec, int64_t nevt, int64_t tile, int slot, int gc,
                                          const Tables* __restrict__ tab, const Tab64* __restrict__ t64,
                                          const uint32_t* __restrict__ mask, const double* __restrict__ ctri,
                                          const MeConst& cst, double* __restrict__ out, int64_t stride,
                                          float2* __restrict__ jout, const double* __restrict__ share,
                                          double* __restrict__ j2) {
+  constexpr int NEV = events_per_block<LOCAL>();
+  const int64_t e = tile * NEV + threadIdx.x % NEV;
+  if (e >= nevt) return;
   View<K, LOCAL> V;
   V.in = rec + (e / kPage) * v2::EvLayout<K>::NITEM * kPage + (e % kPage);
   V.tab = tab;
@@ -514,10 +503,10 @@ __device__ __forceinline__ void thread64(const double* __restrict__ rec, int64_t
     double own[Loc<K>::n];
     V.buf = own;
     for (int i = 0; i < t64->nltask; ++i) run_task<K, true>(V, t64->ltask[i]);
-    slot64<K, MODE, true>(V, e, slot, mask, ctri, cst, out, stride, jout, j2);
+    for (int ab = 0; ab < 4; ++ab) slot64<K, MODE, true>(V, e, slot, ab, mask, ctri, cst, out, stride, jout, j2);
   } else {
     V.buf = const_cast<double*>(share) + (e / kPage) * static_cast<int64_t>(t64->stride) * kPage + (e % kPage);
-    slot64<K, MODE, false>(V, e, slot, mask, ctri, cst, out, stride, jout, j2);
+    slot64<K, MODE, false>(V, e, slot, threadIdx.x / NEV, mask, ctri, cst, out, stride, jout, j2);
   }
 }
 

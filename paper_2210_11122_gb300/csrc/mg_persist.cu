@@ -4,7 +4,7 @@
 // The paper (Sec. 4) finds the GPU throughput still growing up to batches of ~16k events: smaller batches
 // leave the device underfilled.  A batch of many small jobs therefore runs better as one launch whose
 // thread blocks drain a common queue of work tiles than as one launch per job.  Here the queue holds
-// (job, gluon-helicity slot, 128-event tile) triples, the jobs ordered by falling cost per tile (more
+// (job, gluon-helicity slot, tile of 32 or 128 events) triples, the jobs ordered by falling cost per tile (more
 // gluons first, so the longest tiles start first); each 128-thread block takes the next tile from an
 // atomic counter until the queue is empty, and runs the same per-thread FP64 work as the
 // single-job kernels (the
@@ -29,7 +29,8 @@ namespace mg {
 namespace pers {
 
 constexpr int kMaxJobs = 64;   // the job table travels as the kernel's parameter (8 KB)
-constexpr int kTileEv = 128;
+constexpr int kTileEv = 128;   // events per tile of the jobs without shared items (one thread each)
+static_assert(kTileEv == m64::events_per_block<true>() && kTileEv == kMeThreads, "a tile is a block");
 
 struct PJob {
   const double* rec;        // per-event FP64 record
@@ -53,13 +54,13 @@ struct PBatch {
 };
 
 template <int K>
-__device__ __forceinline__ void run64(const PJob& J, int64_t e, int slot, int gc) {
+__device__ __forceinline__ void run64(const PJob& J, int64_t tile, int slot, int gc) {
   if (J.share)
-    m64::thread64<K, m64::kME, false>(J.rec, e, slot, gc, J.tab, J.t64, J.mask, J.ctri, J.cst, J.part, J.stride, nullptr,
-                                      J.share, nullptr);
+    m64::thread64<K, m64::kME, false>(J.rec, J.nevt, tile, slot, gc, J.tab, J.t64, J.mask, J.ctri, J.cst, J.part, J.stride,
+                                      nullptr, J.share, nullptr);
   else
-    m64::thread64<K, m64::kME, true>(J.rec, e, slot, gc, J.tab, J.t64, J.mask, J.ctri, J.cst, J.part, J.stride, nullptr,
-                                     nullptr, nullptr);
+    m64::thread64<K, m64::kME, true>(J.rec, J.nevt, tile, slot, gc, J.tab, J.t64, J.mask, J.ctri, J.cst, J.part, J.stride,
+                                     nullptr, nullptr, nullptr);
 }
 
 __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_constant__ PBatch b,
@@ -80,17 +81,20 @@ __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_co
     const PJob& J = b.job[lo];
     const int64_t t = tile - J.tile0;
     const int slot = static_cast<int>(t / J.ntile_ev);
-    const int64_t e = (t - static_cast<int64_t>(slot) * J.ntile_ev) * kTileEv + threadIdx.x;
-    if (e >= J.nevt || slot >= *J.nslot) continue;
+    const int64_t etile = t - static_cast<int64_t>(slot) * J.ntile_ev;
+    if (slot >= *J.nslot) continue;
     const int gc = J.gslots[slot];
     switch (J.K) {
-      case 2:
-        v2::me_slot<2, double, false, true, false>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst, J.part,
-                                                   J.stride, nullptr, 0, nullptr);
+      case 2: {
+        const int64_t e = etile * kTileEv + threadIdx.x;
+        if (e < J.nevt)
+          v2::me_slot<2, double, false, true, false>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst, J.part,
+                                                     J.stride, nullptr, 0, nullptr);
         break;
-      case 3: run64<3>(J, e, slot, gc); break;
-      case 4: run64<4>(J, e, slot, gc); break;
-      default: run64<5>(J, e, slot, gc); break;
+      }
+      case 3: run64<3>(J, etile, slot, gc); break;
+      case 4: run64<4>(J, etile, slot, gc); break;
+      default: run64<5>(J, etile, slot, gc); break;
     }
   }
 }
@@ -176,7 +180,8 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     p.nevt = j.nevt;
     p.stride = stride;
     p.K = c->K;
-    p.ntile_ev = static_cast<int>((j.nevt + mg::pers::kTileEv - 1) / mg::pers::kTileEv);
+    const int tev = share ? mg::m64::events_per_block<false>() : mg::pers::kTileEv;
+    p.ntile_ev = static_cast<int>((j.nevt + tev - 1) / tev);
     p.tile0 = batch->ntiles;
     p.cst = cst;
     batch->ntiles += static_cast<int64_t>(p.ntile_ev) << (c->K - 1);   // every possible slot; absent ones exit at once
@@ -202,7 +207,7 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
       const mg_batch_job& j = jobs[i];
       if (j.nevt == 0) continue;
       const double norm = 1.0 / (256.0 * mg::factorial(j.ctx->ng));
-      if (mg::launch_hel_sum(j.ctx->d_part, j.ctx->d_nhslots, j.nevt, pad_pg(j.nevt), norm, j.me_dev, st) != cudaSuccess)
+      if (mg::fp64_hel_sum(j.ctx, j.nevt, pad_pg(j.nevt), norm, j.me_dev, st) != cudaSuccess)
         s = MG_ECUDA;
     }
   }

@@ -166,6 +166,7 @@ void build_tab64(int K, const Tables& t, Tab64& o) {
         f.z[g * kMaxGluons + h] = take(1 << g | 1 << h, 2);
         if (K == 5) f.qq[g * kMaxGluons + h] = take(1 << g | 1 << h, 4);
       }
+    for (int i = 0; i < t.nfull; ++i) f.full[i] = take((1 << K) - 1, 1);
     if (K >= 4)
       for (int s = 0; s < t.nseq; ++s)
         for (int g = 0; g < K; ++g)
@@ -209,11 +210,20 @@ void build_tab64(int K, const Tables& t, Tab64& o) {
     psis(2);
   }
   seqs(Tab64::kZ, 2);
-  next_pass();
-  if (K == 5) {
-    seqs(Tab64::kSeq, 4);
-    psis(3);
+  auto fulls = [&] {
+    for (int i = 0; i < t.nfull; ++i) tasks(Tab64::kFull, i, 0, (1 << K) - 1);
     next_pass();
+  };
+  if (K == 3) {
+    fulls();
+  } else {
+    next_pass();
+    if (K == 5) {
+      seqs(Tab64::kSeq, 4);
+      psis(3);
+      next_pass();
+    }
+    fulls();
   }
   // ---- terms of the amplitudes ----
   std::vector<int> p(K);
@@ -226,23 +236,34 @@ void build_tab64(int K, const Tables& t, Tab64& o) {
     std::reverse(q.begin() + i, q.begin() + j);
     return rank.at(q);
   };
-  int n1 = 0, n2 = 0, n3 = 0;
-  for (int c = 0; c < t.ncol; ++c) {
-    const std::vector<int>& s = perms[c];
+  for (int c = 0; c < t.ncol; ++c)
     if (t.full_idx[c] >= 0) {
       o.full_c[t.full_idx[c]] = static_cast<int16_t>(c);
       o.full_cr[t.full_idx[c]] = static_cast<int16_t>(reversed(c, 0, K));
     }
-    auto entry = [&](int16_t* e, int i, int j, int key) {
-      e[0] = static_cast<int16_t>(t.sub[c][i][j] >> 1);
-      e[1] = static_cast<int16_t>(key);
-      e[2] = static_cast<int16_t>(c);
-      e[3] = static_cast<int16_t>(reversed(c, i, j));
-    };
-    if (s[0] < s[K - 2]) entry(o.t1[n1++], 0, K - 1, s[K - 1]);
-    if (K == 5 && s[1] < s[4]) entry(o.t2[n2++], 1, 5, s[0]);
-    if (K == 5 && s[1] < s[3]) entry(o.t3[n3++], 1, 4, s[0] * kMaxGluons + s[4]);
-  }
+  auto entry = [&](int16_t* e, int c, int i, int j) {
+    e[0] = static_cast<int16_t>(t.sub[c][i][j] >> 1);
+    e[1] = static_cast<int16_t>(c);
+    e[2] = static_cast<int16_t>(reversed(c, i, j));
+  };
+  int n1 = 0, n2 = 0, n3 = 0;
+  for (int g = 0; g < K; ++g)
+    for (int c = 0; c < t.ncol; ++c) {
+      const std::vector<int>& s = perms[c];
+      if (s[K - 1] == g && s[0] < s[K - 2]) entry(o.t1[n1++], c, 0, K - 1);
+      if (K == 5 && s[0] == g && s[1] < s[4]) entry(o.t2[n2++], c, 1, 5);
+    }
+  if (K == 5)
+    for (int g = 0; g < K; ++g)
+      for (int h = 0; h < K; ++h) {
+        if (g == h) continue;
+        o.t3q[n3 / 3][0] = static_cast<int16_t>(g);
+        o.t3q[n3 / 3][1] = static_cast<int16_t>(h);
+        for (int c = 0; c < t.ncol; ++c) {
+          const std::vector<int>& s = perms[c];
+          if (s[0] == g && s[4] == h && s[1] < s[3]) entry(o.t3[n3++], c, 1, 4);
+        }
+      }
   for (int g = 0; g < t.ncol / 6; ++g)
     for (int i = 0; i < 6; ++i) {
       const int c = 6 * g + i;
