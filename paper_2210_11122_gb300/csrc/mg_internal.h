@@ -106,9 +106,19 @@ struct Tab64 {
   int16_t g3[kMaxNcol / 6][3];             // six orderings with a common prefix of K-3: sequences xyz, xzy, yxz
   int16_t gy[kMaxNcol / 6][3][2];          // (pair, last): (xy, z), (xz, y), (yz, x)
   int16_t gz[kMaxNcol / 6][6];             // last two gluons, first * 5 + second, of the six orderings
+  // Colour sum of 4 and 5 gluons in a basis that block-diagonalises the colour matrix C.  C is unchanged when both
+  // orderings have gluons 0 and 1 swapped, gluons 2 and 3 swapped, or are reversed; on an orbit of these three commuting
+  // involutions (8 orderings, or 4 where the reversal equals a product of swaps) the sums with signs (-1)^(k & m) have
+  // no C entries between different sign patterns k.  Orbit member m = bit 0: 0 <-> 1, bit 1: 2 <-> 3, bit 2:
+  // reversed; the combination of pattern k replaces the jamp of member k.
+  int n8, n4, nblk;                        // orbits of 8 and of 4; blocks
+  uint8_t orb8[14][8], orb4[2][4];         // jamp indices
+  uint8_t blk_n[8], blk[8][16];            // a block's size and jamp indices
+  double blk_c[964];                       // its packed upper triangle (off-diagonal doubled), block after block
 };
 
-void build_tab64(int K, const Tables& t, Tab64& o);
+// num: the integer colour matrix (colour_matrix_exact)
+void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64& o);
 const Tab64& tab64_host(int K);            // built once per process (K = 3..5)
 
 }  // namespace mg

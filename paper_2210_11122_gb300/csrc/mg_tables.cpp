@@ -137,7 +137,7 @@ void build_tables(int K, Tables& t) {
   }
 }
 
-void build_tab64(int K, const Tables& t, Tab64& o) {
+void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64& o) {
   std::memset(&o, 0, sizeof(o));
   o.K = K;
   const int top = 1 << (K - 1);
@@ -278,6 +278,53 @@ void build_tab64(int K, const Tables& t, Tab64& o) {
         }
       }
     }
+  // ---- colour sum in the symmetry-adapted basis (4 and 5 gluons) ----
+  if (K < 4) return;
+  auto image = [&](int c, int m) {   // ordering c with gluons 0,1 and 2,3 swapped and reversed as m's bits say
+    std::vector<int> q = perms[c];
+    for (int& g : q) {
+      if ((m & 1) && g < 2) g = 1 - g;
+      else if ((m & 2) && (g == 2 || g == 3)) g = 5 - g;
+    }
+    if (m & 4) std::reverse(q.begin(), q.end());
+    return rank.at(q);
+  };
+  std::vector<bool> seen(t.ncol, false);
+  struct Vec { int at; std::vector<int> sign; int norm; };   // a basis combination: jamp index it replaces, signs
+  std::vector<Vec> blocks[8];
+  for (int c = 0; c < t.ncol; ++c) {
+    if (seen[c]) continue;
+    int self = 0;   // the product of swaps that equals the reversal on this orbit, if any (never the identity)
+    for (int m = 1; m < 4; ++m)
+      if (image(c, m) == image(c, 4)) self = m;
+    const int n = self ? 4 : 8;
+    uint8_t* orb = self ? o.orb4[o.n4++] : o.orb8[o.n8++];
+    for (int m = 0; m < n; ++m) {
+      orb[m] = static_cast<uint8_t>(image(c, m));
+      seen[orb[m]] = true;
+    }
+    for (int k = 0; k < n; ++k) {
+      Vec v{orb[k], std::vector<int>(t.ncol, 0), n};
+      for (int m = 0; m < n; ++m) v.sign[orb[m]] = __builtin_popcount(k & m) & 1 ? -1 : 1;
+      blocks[self ? k | (__builtin_popcount(k & self) & 1) << 2 : k].push_back(v);
+    }
+  }
+  o.nblk = 8;
+  int nc = 0;
+  for (int b = 0; b < 8; ++b) {
+    o.blk_n[b] = static_cast<uint8_t>(blocks[b].size());
+    for (size_t i = 0; i < blocks[b].size(); ++i) {
+      o.blk[b][i] = static_cast<uint8_t>(blocks[b][i].at);
+      for (size_t j = i; j < blocks[b].size(); ++j) {
+        int64_t s = 0;
+        for (int x = 0; x < t.ncol; ++x)
+          for (int y = 0; y < t.ncol; ++y)
+            s += num[static_cast<size_t>(x) * t.ncol + y] * blocks[b][i].sign[x] * blocks[b][j].sign[y];
+        // (exact: an integer over a power of two)
+        o.blk_c[nc++] = (i == j ? 1.0 : 2.0) * static_cast<double>(s) / (blocks[b][i].norm * blocks[b][j].norm);
+      }
+    }
+  }
 }
 
 const Tab64& tab64_host(int K) {
@@ -286,7 +333,10 @@ const Tab64& tab64_host(int K) {
   std::call_once(once[K], [K] {
     Tables* t = new Tables;
     build_tables(K, *t);
-    build_tab64(K, *t, tabs[K]);
+    std::vector<int64_t> num;
+    int64_t den;
+    colour_matrix_exact(K, num, den);
+    build_tab64(K, *t, num, tabs[K]);
     delete t;
   });
   return tabs[K];
