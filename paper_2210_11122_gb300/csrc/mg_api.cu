@@ -184,17 +184,18 @@ cudaError_t fp64_slots(mg_ctx* ctx, const double* mom, const double* rec, int64_
   if (ctx->K == 2)
     return launch_me_gluonhel(2, false, false, mom, const_cast<double*>(rec), n, ctx->d_tab, ctx->d_hslots, 2,
                               ctx->d_nhslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, out, stride, st, jout, shape);
+  const int* lin = jout ? nullptr : ctx->d_lin;   // (a sum of colour sums may be taken in either basis)
   if (shared) {
-    const cudaError_t e = launch_pass64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, cst, ctx->d_share, st);
+    const cudaError_t e = launch_pass64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, cst, lin, ctx->d_share, st);
     if (e != cudaSuccess) return e;
   }
-  return launch_me64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, ctx->d_hslots, ctx->d_nhslots, ctx->d_mask, ctx->d_ctri, cst,
+  return launch_me64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, ctx->d_hslots, ctx->d_nhslots, lin, ctx->d_mask, ctx->d_ctri, cst,
                      out, stride, jout, shape, shared ? ctx->d_share : nullptr, nullptr, st);
 }
 
 cudaError_t fp64_hel_sum(mg_ctx* ctx, int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st) {
   if (ctx->K == 2) return launch_hel_sum(ctx->d_part, ctx->d_nhslots, nevt, stride, norm, me, st);
-  return launch_hel_sum_rows(ctx->K, ctx->d_part, ctx->d_hslots, ctx->d_nhslots, ctx->d_mask, nevt, stride, norm, me, st);
+  return launch_hel_sum_rows(ctx->K, ctx->d_part, ctx->d_hslots, ctx->d_nhslots, ctx->d_lin, ctx->d_mask, nevt, stride, norm, me, st);
 }
 
 bool mixed_in_kernel(const mg_ctx* ctx, mg_precision precision) {
@@ -249,7 +250,8 @@ mg_status ctx_copy_mask(mg_ctx* dst, const mg_ctx* src, cudaStream_t st) {
                   cp(dst->d_ngood, src->d_ngood, sizeof(int)) && cp(dst->d_maxr, src->d_maxr, 128 * sizeof(double)) &&
                   cp(dst->d_gslots, src->d_gslots, 32 * sizeof(int)) && cp(dst->d_ngslots, src->d_ngslots, sizeof(int)) &&
                   cp(dst->d_nrows, src->d_nrows, sizeof(int)) && cp(dst->d_hslots, src->d_hslots, 16 * sizeof(int)) &&
-                  cp(dst->d_nhslots, src->d_nhslots, sizeof(int)) && cp(dst->d_nhrows, src->d_nhrows, sizeof(int));
+                  cp(dst->d_nhslots, src->d_nhslots, sizeof(int)) && cp(dst->d_nhrows, src->d_nhrows, sizeof(int)) &&
+                  cp(dst->d_lin, src->d_lin, sizeof(int));
   if (!ok) { cudaGetLastError(); return MG_ECUDA; }
   dst->mask_ready = true;
   return MG_OK;
@@ -380,6 +382,7 @@ void mg_destroy(mg_ctx* ctx) {
   mg::dev_free(ctx->d_hslots);
   mg::dev_free(ctx->d_nhslots);
   mg::dev_free(ctx->d_nhrows);
+  mg::dev_free(ctx->d_lin);
   mg::dev_free(ctx->d_cmat);
   mg::dev_free(ctx->d_cumma);
   mg::dev_free(ctx->d_tcerr);
@@ -492,6 +495,7 @@ mg_status mg_create(mg_process proc, const mg_params* params, mg_ctx** out) {
     if (mg::dev_alloc(&c->d_gslots, 32 * sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_ngslots, sizeof(int)) != cudaSuccess ||
         mg::dev_alloc(&c->d_hslots, 16 * sizeof(int)) != cudaSuccess ||
         mg::dev_alloc(&c->d_nhslots, sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_nhrows, sizeof(int)) != cudaSuccess ||
+        mg::dev_alloc(&c->d_lin, sizeof(int)) != cudaSuccess ||
         mg::dev_alloc(&c->d_allg, 32 * sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_nallg, sizeof(int)) != cudaSuccess) {
       st = MG_ENOMEM;
       break;
@@ -499,7 +503,7 @@ mg_status mg_create(mg_process proc, const mg_params* params, mg_ctx** out) {
     if (cudaMemcpy(c->d_allg, all.data(), ng2 * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->d_nallg, &ng2, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(c->d_ngslots, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->d_nhslots, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(c->d_nhrows, 0, sizeof(int)) != cudaSuccess) {
+        cudaMemset(c->d_nhrows, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->d_lin, 0, sizeof(int)) != cudaSuccess) {
       st = MG_ECUDA;
       break;
     }
@@ -614,7 +618,7 @@ mg_status mg_hel_filter(mg_ctx* ctx, const double* mom_dev, int64_t nevt, void* 
   MG_CUDA(mg::launch_hel_mask(ctx->d_part, ctx->d_tot, ctx->nhel, w, stride, ctx->prm.hel_tau, ctx->d_maxr,
                               ctx->d_mask, ctx->d_good, ctx->d_ngood, st));
   MG_CUDA(mg::launch_gluon_slots(ctx->d_mask, ctx->K, ctx->d_gslots, ctx->d_ngslots, ctx->d_nrows, ctx->d_hslots,
-                                 ctx->d_nhslots, ctx->d_nhrows, st));
+                                 ctx->d_nhslots, ctx->d_nhrows, ctx->d_lin, st));
   ctx->mask_ready = true;
   return MG_OK;
 }
@@ -736,7 +740,7 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
                                        ctx->tc_stall));
       if (fp32) MG_CUDA(join_repair(ctx, st));
       if (half)   // (the colour pass writes a row per helicity for every process)
-        MG_CUDA(mg::launch_hel_sum_rows(ctx->K, ctx->d_part, slots, nslots, ctx->d_mask, n, cst_stride, norm, me_dev + e0, st));
+        MG_CUDA(mg::launch_hel_sum_rows(ctx->K, ctx->d_part, slots, nslots, nullptr, ctx->d_mask, n, cst_stride, norm, me_dev + e0, st));
       else
         MG_CUDA(mg::launch_hel_sum(ctx->d_part, ctx->d_nrows, n, cst_stride, norm, me_dev + e0, st));
     }

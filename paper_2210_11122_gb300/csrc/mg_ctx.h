@@ -28,6 +28,7 @@ struct mg_ctx {
   int* d_hslots = nullptr;    // FP64: one of each pair of flipped gluon combinations (hel_weight)
   int* d_nhslots = nullptr;
   int* d_nhrows = nullptr;
+  int* d_lin = nullptr;       // 1: every helicity is good (FP64 sums over linear polarisations)
   void* d_cmat = nullptr;     // colour matrix numerators as the packed FP16 tensor-core operand
   void* d_cumma = nullptr;    // the same as the tcgen05 B operand (canonical no-swizzle K-major layout)
   int* d_tcerr = nullptr;     // nonzero: a bounded wait of the tcgen05 colour kernel gave up

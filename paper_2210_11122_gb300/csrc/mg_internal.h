@@ -79,7 +79,7 @@ void build_tables(int K, Tables& t);
 // ----------------------------------------------------------------------------------------
 struct Tab64 {
   enum Type { kJ1, kJq0, kChi, kPsi, kSeq, kZ, kY, kFull, kQQ };
-  static constexpr int kMaxTask = 2500, kMaxLTask = 320, kMaxPass = 6;
+  static constexpr int kMaxTask = 2500, kMaxTaskL = 4200, kMaxLTask = 320, kMaxPass = 6;
   struct Off {
     int J[kMaxSeq];                        // current of a canonical sequence (1)
     int X[kMaxSeq];                        // (gamma.J) v, three or more gluons (antitop helicity: 2); -1: none
@@ -92,10 +92,29 @@ struct Tab64 {
     int full[kMaxNcol / 2];                // ubar gamma^mu v times a canonical full current (4 complex numbers)
     int qq[kMaxGluons * kMaxGluons];       // psi_1(g) gamma^mu chi(h), 5 gluons (4)
   };
-  int K, stride, nloc;                     // doubles per event of the shared buffer, of one combination's own items
+  // Linear gluon polarisations (mg_me64l.cuh): one entry per polarisation combination of the whole gluon set; currents
+  // are real (4 doubles), the others 8 doubles times what the comment says, top helicity -1 only.
+  struct OffL {
+    int J[kMaxSeq];
+    int psi[kMaxGluons - 1][60];           // (1)
+    int qv[kMaxGluons - 1][60];            // psi_m gamma^mu v, m <= K - 3 (antitop helicity: 2)
+    int chi[kMaxGluons], qg[kMaxGluons];   // (2)
+    int q0;                                // (2)
+    int z[kMaxGluons * kMaxGluons];        // (2)
+    int y[kMaxSeq][kMaxGluons];            // 5 gluons (2)
+    int full[kMaxNcol / 2];                // 2 complex numbers (4 doubles)
+    int qq[kMaxGluons * kMaxGluons];       // 4 and 5 gluons (2)
+  };
+  int K, stride;                           // doubles per event of the shared buffer (either basis)
+  int nloc, nlocl;                         // doubles of one combination's own items
   Off sh, loc;
+  OffL shl, locl;
   int npass, pass0[kMaxPass + 1];
   uint32_t task[kMaxTask];                 // type | a << 4 | b << 14 | gluon helicities << 20, by pass
+  int pass0l[kMaxPass + 1];
+  uint32_t taskl[kMaxTaskL];               // the same for linear polarisations
+  int nltaskl;
+  uint32_t ltaskl[kMaxLTask];
   int nltask;
   uint32_t ltask[kMaxLTask];               // the same tasks without helicities, in an order that respects dependences
   int16_t full_c[kMaxNcol / 2], full_cr[kMaxNcol / 2];   // orderings of a full current and of its reversal

@@ -87,11 +87,15 @@ cudaError_t launch_me_gluonhel(int K, bool fp32, bool per_hel, const double* mom
 // share = null one per (event, combination) computing its own (the same bits).  Output, rows r = slot * 4 + 2 top +
 // antitop (cst.conj = 1): the colour sums out[r * stride + e], zero for weight 0; with jout the FP32 jamps instead (2^(K+1)
 // rows per event); with j2 also the weighted jamp squares j2[(r * ncol + sigma) * stride + e].
+// lin (may be null; colour sums only): a device flag, nonzero where every helicity is good: then the sum runs over
+// linear gluon polarisations (mg_me64l.cuh), rows 2 * polarisations + antitop helicity; the same for both calls and for
+// launch_hel_sum_rows.
 cudaError_t launch_pass64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const MeConst& cst,
-                          double* share, cudaStream_t st);
+                          const int* lin, double* share, cudaStream_t st);
 cudaError_t launch_me64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const int* hslots,
-                        const int* nslot, const uint32_t* mask, const double* ctri, const MeConst& cst, double* out,
-                        int64_t stride, float2* jout, MeShape shape, const double* share, double* j2, cudaStream_t st);
+                        const int* nslot, const int* lin, const uint32_t* mask, const double* ctri, const MeConst& cst,
+                        double* out, int64_t stride, float2* jout, MeShape shape, const double* share, double* j2,
+                        cudaStream_t st);
 int64_t event_record_bytes(int K, bool fp32);
 // The FP32 modes' recomputation of events evlist[0..*nlist) with double-float amplitudes (mg_me_dd.cu):
 // launch_me_gluonhel's contract for prep == NULL, per_hel false, FP32 colour table ctri32 (the per-thread
@@ -144,11 +148,13 @@ cudaError_t launch_colour_tc(int ncol, const float2* jamps, int64_t nevt, int ro
                              const void* cmat, double scale, double* out, int64_t stride, cudaStream_t st,
                              const uint8_t* skip = nullptr);
 // gslots: the gluon-helicity combinations with a good helicity (*n of them, *nrows = 4 *n); hslots: those with
-// gluon K-1 of helicity -1 for which the combination or its flip has a good helicity (*nh, *nhrows = 4 *nh).
+// gluon K-1 of helicity -1 for which the combination or its flip has a good helicity (*nh, *nhrows = 4 *nh); *lin = 1
+// if every helicity is good, else 0.
 cudaError_t launch_gluon_slots(const uint32_t* mask, int K, int* gslots, int* n, int* nrows, int* hslots, int* nh,
-                               int* nhrows, cudaStream_t st);
-// me[e] = norm * sum over the rows of hslots (slot * 4 + 2 top + antitop) of hel_weight * part[row * stride + e]
-cudaError_t launch_hel_sum_rows(int K, const double* part, const int* hslots, const int* nh, const uint32_t* mask,
+                               int* nhrows, int* lin, cudaStream_t st);
+// me[e] = norm * sum over the rows of hslots (slot * 4 + 2 top + antitop) of hel_weight * part[row * stride + e]; where
+// *lin != 0 (lin may be null) over all 2^(K+1) rows of the linear polarisations, each for 2^(K+1) times its value
+cudaError_t launch_hel_sum_rows(int K, const double* part, const int* hslots, const int* nh, const int* lin, const uint32_t* mask,
                                 int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st);
 cudaError_t launch_hel_sum(const double* part, const int* nslot, int64_t nevt, int64_t stride, double norm,
                            double* me, cudaStream_t st);

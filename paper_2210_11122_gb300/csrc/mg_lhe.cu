@@ -181,8 +181,8 @@ mg_status grow_buf(double** buf, int64_t* cap, int64_t need) {
 cudaError_t lhe_me(int K, const double* rec, int64_t nevt, const mg_ctx* c, const mg::MeConst& cst, double* part,
                    double* j2, int64_t stride, const double* share, cudaStream_t st) {
   if (K >= 3)
-    return mg::launch_me64(K, rec, nevt, c->d_tab, c->d_tab64, c->d_hslots, c->d_nhslots, c->d_mask, c->d_ctri, cst, part,
-                           stride, nullptr, mg::MeShape(), share, j2, st);
+    return mg::launch_me64(K, rec, nevt, c->d_tab, c->d_tab64, c->d_hslots, c->d_nhslots, nullptr, c->d_mask, c->d_ctri,
+                           cst, part, stride, nullptr, mg::MeShape(), share, j2, st);
   constexpr int tev = mg::kMeThreads;
   const dim3 grid(static_cast<unsigned>((nevt + tev - 1) / tev), 2);
   mg::v2::k_me_gluonhel<2, double, false, true, false, true><<<grid, mg::kMeThreads, 0, st>>>(
@@ -253,7 +253,7 @@ mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, cons
     const int64_t stride = pad_page(n);
     const double* mom_c = mom_dev + (e0 / mg::kPage) * ctx->npar * 4 * mg::kPage;
     if (mg::launch_event_prep(K, false, mom_c, n, cst, ctx->d_prep, st) != cudaSuccess) return MG_ECUDA;
-    if (shared && mg::launch_pass64(K, ctx->d_prep, n, ctx->d_tab, ctx->d_tab64, cst, ctx->d_share, st) != cudaSuccess) return MG_ECUDA;
+    if (shared && mg::launch_pass64(K, ctx->d_prep, n, ctx->d_tab, ctx->d_tab64, cst, nullptr, ctx->d_share, st) != cudaSuccess) return MG_ECUDA;
     if (lhe_me(K, ctx->d_prep, n, ctx, cst, ctx->d_part, ctx->d_j2, stride, shared ? ctx->d_share : nullptr, st) !=
         cudaSuccess)
       return MG_ECUDA;

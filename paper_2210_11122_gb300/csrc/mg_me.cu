@@ -389,12 +389,18 @@ __global__ void k_hel_sum(const double* __restrict__ part, const int* __restrict
 
 // me[e] = norm * sum over the rows (slot * 4 + 2 top + antitop) of one of each pair of flipped helicities
 __global__ void k_hel_sum_rows(int K, const double* __restrict__ part, const int* __restrict__ hslots,
-                               const int* __restrict__ nh_dev, const uint32_t* __restrict__ mask, int64_t nevt,
-                               int64_t stride, double norm, double* __restrict__ me) {
+                               const int* __restrict__ nh_dev, const int* __restrict__ lin,
+                               const uint32_t* __restrict__ mask, int64_t nevt, int64_t stride, double norm,
+                               double* __restrict__ me) {
   const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (e >= nevt) return;
   const int nh = *nh_dev, npar = K + 2;
   double s = 0.0;
+  if (lin && *lin) {
+    for (int r = 0; r < (2 << K); ++r) s += part[r * stride + e];
+    me[e] = s * (norm * static_cast<double>(2 << K));
+    return;
+  }
   for (int k = 0; k < nh; ++k) {
     const int gc = hslots[k];
     int hb = 0;
@@ -479,12 +485,13 @@ cudaError_t launch_hel_sum(const double* part, const int* nslot, int64_t nevt, i
   return cudaGetLastError();
 }
 
-cudaError_t launch_hel_sum_rows(int K, const double* part, const int* hslots, const int* nh, const uint32_t* mask,
-                                int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st) {
+cudaError_t launch_hel_sum_rows(int K, const double* part, const int* hslots, const int* nh, const int* lin,
+                                const uint32_t* mask, int64_t nevt, int64_t stride, double norm, double* me,
+                                cudaStream_t st) {
   const int threads = 256;
   const unsigned blocks = static_cast<unsigned>((nevt + threads - 1) / threads);
   if (blocks == 0) return cudaSuccess;
-  { k_hel_sum_rows<<<blocks, threads, 0, st>>>(K, part, hslots, nh, mask, nevt, stride, norm, me); mg::note_launch(); }
+  { k_hel_sum_rows<<<blocks, threads, 0, st>>>(K, part, hslots, nh, lin, mask, nevt, stride, norm, me); mg::note_launch(); }
   return cudaGetLastError();
 }
 

@@ -71,10 +71,13 @@ __global__ void __launch_bounds__(128) k_event_flags(const double* __restrict__ 
 // one of each pair of flipped combinations (launch_gluon_slots).
 __global__ void k_gluon_slots(const uint32_t* __restrict__ mask, int K, int* __restrict__ gslots, int* __restrict__ n,
                               int* __restrict__ nrows, int* __restrict__ hslots, int* __restrict__ nh,
-                              int* __restrict__ nhrows) {
+                              int* __restrict__ nhrows, int* __restrict__ lin) {
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const int npar = K + 2;
   int cnt = 0, hcnt = 0;
+  bool all = true;
+  for (int h = 0; h < (1 << npar); ++h) all = all && ((mask[h >> 5] >> (h & 31)) & 1u);
+  *lin = all ? 1 : 0;
   for (int gc = 0; gc < (1 << K); ++gc) {
     int hb = 0;
     for (int g = 0; g < K; ++g)
@@ -97,8 +100,8 @@ __global__ void k_gluon_slots(const uint32_t* __restrict__ mask, int K, int* __r
 }  // namespace v2
 
 cudaError_t launch_gluon_slots(const uint32_t* mask, int K, int* gslots, int* n, int* nrows, int* hslots, int* nh,
-                               int* nhrows, cudaStream_t st) {
-  { v2::k_gluon_slots<<<1, 32, 0, st>>>(mask, K, gslots, n, nrows, hslots, nh, nhrows); mg::note_launch(); }
+                               int* nhrows, int* lin, cudaStream_t st) {
+  { v2::k_gluon_slots<<<1, 32, 0, st>>>(mask, K, gslots, n, nrows, hslots, nh, nhrows, lin); mg::note_launch(); }
   return cudaGetLastError();
 }
 

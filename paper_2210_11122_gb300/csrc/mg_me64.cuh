@@ -316,30 +316,6 @@ __device__ __forceinline__ void run_task(const View<K, LOCAL>& V, uint32_t task)
   }
 }
 
-// One thread per (event, task of the pass): tasks [t0, t0 + ntask) of the table, warps on one task of 32 consecutive
-// events.  Bound by the FP64 pipe.
-template <int K>
-__global__ void __launch_bounds__(128)
-k_pass64(const double* __restrict__ rec, int64_t nevt, const Tables* __restrict__ tab, const Tab64* __restrict__ t64,
-         double gs, int t0, int ntask, double* __restrict__ share) {
-  const int64_t npage = (nevt + kPage - 1) / kPage;
-  const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t j = t / (npage * kPage);
-  if (j >= ntask) return;
-  const int64_t e = t - j * npage * kPage;
-  if (e >= nevt) return;
-  const uint32_t task = t64->task[t0 + j];
-  View<K, false> V;
-  V.in = rec + (e / kPage) * v2::EvLayout<K>::NITEM * kPage + (e % kPage);
-  V.buf = share + (e / kPage) * static_cast<int64_t>(t64->stride) * kPage + (e % kPage);
-  V.tab = tab;
-  V.t = t64;
-  V.o = &t64->sh;
-  V.gc = static_cast<int>(task >> 20);
-  V.gs = gs;
-  run_task<K, false>(V, task);
-}
-
 constexpr int kME = 0, kJamps = 1, kLhe = 2;
 
 // sums and differences of the 2^N complex numbers a[0 .. 2^N) over each bit of their index
@@ -530,43 +506,6 @@ __device__ __forceinline__ void slot64(const View<K, LOCAL>& V, int64_t e, int s
         j2[(static_cast<int64_t>(row) * NCOL + c) * stride + e] =
             static_cast<double>(w) * fma(A[c].r, A[c].r, A[c].i * A[c].i);
     out[row * stride + e] = colour_sum64<K>(A, t, ctri) * cst.colour_scale;
-  }
-}
-
-// A warp takes one top helicity pair of one combination (the all-gluon currents, which the pairs share, are items
-// of the last pass): a thread doing all four pairs made 4 times longer warps, of which gg->ttgg's 10,007 events are
-// 4.1 per sub-partition, so the busiest had 5; measured 2.81 vs 3.19 ms there, gg->ttggg + TC colour 7.60 vs 8.60 ms
-// per 2,049 events, gg->ttg 12.05 vs 12.13 ms per 524,288.
-// Events per block of 128 threads: with the shared items 32 (a page), one warp for each top helicity pair of a
-// combination; without them 128, a thread doing the four pairs with the items it has built.
-template <bool LOCAL> __host__ __device__ constexpr int events_per_block() { return LOCAL ? 128 : 32; }
-
-// One thread of a block on event tile `tile` of combination `slot`.
-template <int K, int MODE, bool LOCAL>
-__device__ __forceinline__ void thread64(const double* __restrict__ rec, int64_t nevt, int64_t tile, int slot, int gc,
-                                         const Tables* __restrict__ tab, const Tab64* __restrict__ t64,
-                                         const uint32_t* __restrict__ mask, const double* __restrict__ ctri,
-                                         const MeConst& cst, double* __restrict__ out, int64_t stride,
-                                         float2* __restrict__ jout, const double* __restrict__ share,
-                                         double* __restrict__ j2) {
-  constexpr int NEV = events_per_block<LOCAL>();
-  const int64_t e = tile * NEV + threadIdx.x % NEV;
-  if (e >= nevt) return;
-  View<K, LOCAL> V;
-  V.in = rec + (e / kPage) * v2::EvLayout<K>::NITEM * kPage + (e % kPage);
-  V.tab = tab;
-  V.t = t64;
-  V.o = LOCAL ? &t64->loc : &t64->sh;
-  V.gc = gc;
-  V.gs = cst.gs;
-  if constexpr (LOCAL) {
-    double own[Loc<K>::n];
-    V.buf = own;
-    for (int i = 0; i < t64->nltask; ++i) run_task<K, true>(V, t64->ltask[i]);
-    for (int ab = 0; ab < 4; ++ab) slot64<K, MODE, true>(V, e, slot, ab, mask, ctri, cst, out, stride, jout, j2);
-  } else {
-    V.buf = const_cast<double*>(share) + (e / kPage) * static_cast<int64_t>(t64->stride) * kPage + (e % kPage);
-    slot64<K, MODE, false>(V, e, slot, threadIdx.x / NEV, mask, ctri, cst, out, stride, jout, j2);
   }
 }
 

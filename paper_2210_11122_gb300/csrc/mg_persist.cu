@@ -22,21 +22,21 @@
 #include "mg_ctx.h"
 #include "mg_internal.h"
 #include "mg_kernels.h"
-#include "mg_me64.cuh"
+#include "mg_me64l.cuh"
 #include "mg_me_kernel.cuh"
 
 namespace mg {
 namespace pers {
 
 constexpr int kMaxJobs = 64;   // the job table travels as the kernel's parameter (8 KB)
-constexpr int kTileEv = 128;   // events per tile of the jobs without shared items (one thread each)
-static_assert(kTileEv == m64::events_per_block<true>() && kTileEv == kMeThreads, "a tile is a block");
+constexpr int kTileEv = kMeThreads;   // events per tile of 2 gluons (one thread each); 32 with 3 to 5 (thread64)
 
 struct PJob {
   const double* rec;        // per-event FP64 record
   const Tables* tab;
   const int* gslots;        // gluon-helicity combinations (one of each flipped pair) with a good helicity
   const int* nslot;
+  const int* lin;           // nonzero: linear polarisations (3 to 5 gluons)
   const uint32_t* mask;
   const double* ctri;
   const Tab64* t64;
@@ -54,13 +54,13 @@ struct PBatch {
 };
 
 template <int K>
-__device__ __forceinline__ void run64(const PJob& J, int64_t tile, int slot, int gc) {
+__device__ __forceinline__ void run64(const PJob& J, int64_t tile, int blk) {
   if (J.share)
-    m64::thread64<K, m64::kME, false>(J.rec, J.nevt, tile, slot, gc, J.tab, J.t64, J.mask, J.ctri, J.cst, J.part, J.stride,
-                                      nullptr, J.share, nullptr);
+    m64::thread64<K, m64::kME, false>(J.rec, J.nevt, tile, blk, J.tab, J.t64, J.gslots, J.nslot, J.lin, J.mask, J.ctri, J.cst,
+                                      J.part, J.stride, nullptr, J.share, nullptr);
   else
-    m64::thread64<K, m64::kME, true>(J.rec, J.nevt, tile, slot, gc, J.tab, J.t64, J.mask, J.ctri, J.cst, J.part, J.stride,
-                                     nullptr, nullptr, nullptr);
+    m64::thread64<K, m64::kME, true>(J.rec, J.nevt, tile, blk, J.tab, J.t64, J.gslots, J.nslot, J.lin, J.mask, J.ctri, J.cst,
+                                     J.part, J.stride, nullptr, nullptr, nullptr);
 }
 
 __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_constant__ PBatch b,
@@ -82,19 +82,17 @@ __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_co
     const int64_t t = tile - J.tile0;
     const int slot = static_cast<int>(t / J.ntile_ev);
     const int64_t etile = t - static_cast<int64_t>(slot) * J.ntile_ev;
-    if (slot >= *J.nslot) continue;
-    const int gc = J.gslots[slot];
     switch (J.K) {
       case 2: {
         const int64_t e = etile * kTileEv + threadIdx.x;
-        if (e < J.nevt)
-          v2::me_slot<2, double, false, true, false>(nullptr, J.rec, e, slot, gc, J.tab, J.mask, J.ctri, J.cst, J.part,
-                                                     J.stride, nullptr, 0, nullptr);
+        if (e < J.nevt && slot < *J.nslot)
+          v2::me_slot<2, double, false, true, false>(nullptr, J.rec, e, slot, J.gslots[slot], J.tab, J.mask, J.ctri, J.cst,
+                                                     J.part, J.stride, nullptr, 0, nullptr);
         break;
       }
-      case 3: run64<3>(J, etile, slot, gc); break;
-      case 4: run64<4>(J, etile, slot, gc); break;
-      default: run64<5>(J, etile, slot, gc); break;
+      case 3: run64<3>(J, etile, slot); break;
+      case 4: run64<4>(J, etile, slot); break;
+      default: run64<5>(J, etile, slot); break;
     }
   }
 }
@@ -164,7 +162,7 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     if (c->shape[MG_FP64].shared && c->K >= 3 && sdoubles <= (int64_t(1) << 28)) {
       s = grow_d(&c->d_share, &c->share_cap, sdoubles);
       if (s != MG_OK) break;
-      if (mg::launch_pass64(c->K, c->d_prep, j.nevt, c->d_tab, c->d_tab64, cst, c->d_share, st) != cudaSuccess) { s = MG_ECUDA; break; }
+      if (mg::launch_pass64(c->K, c->d_prep, j.nevt, c->d_tab, c->d_tab64, cst, c->d_lin, c->d_share, st) != cudaSuccess) { s = MG_ECUDA; break; }
       share = c->d_share;
     }
     mg::pers::PJob& p = batch->job[batch->njobs++];
@@ -174,13 +172,14 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     p.t64 = c->d_tab64;
     p.gslots = c->d_hslots;
     p.nslot = c->d_nhslots;
+    p.lin = c->d_lin;
     p.mask = c->d_mask;
     p.ctri = c->d_ctri;
     p.part = c->d_part;
     p.nevt = j.nevt;
     p.stride = stride;
     p.K = c->K;
-    const int tev = share ? mg::m64::events_per_block<false>() : mg::pers::kTileEv;
+    const int tev = c->K == 2 ? mg::pers::kTileEv : mg::kPage;
     p.ntile_ev = static_cast<int>((j.nevt + tev - 1) / tev);
     p.tile0 = batch->ntiles;
     p.cst = cst;

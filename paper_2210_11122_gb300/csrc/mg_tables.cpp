@@ -173,10 +173,53 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
           if (t.seq_len[s] == 2 && !((t.seq_mask[s] >> g) & 1)) f.y[s][g] = take(t.seq_mask[s] | 1 << g, 2);
     (own ? o.nloc : o.stride) = at;
   }
+  // ---- linear polarisations ----
+  for (int own = 0; own < 2; ++own) {
+    Tab64::OffL& f = own ? o.locl : o.shl;
+    int at = 0;
+    auto take = [&](int mask, int doubles) {
+      const int r = at;
+      at += doubles * (own ? 1 : 1 << __builtin_popcount(mask));
+      return r;
+    };
+    std::memset(&f, 0xff, sizeof(f));
+    for (int s = 0; s < t.nseq; ++s) f.J[s] = take(t.seq_mask[s], 4);
+    for (int m = 1; m <= K - 2; ++m)
+      for (int p = 0; p < t.ncol / fact(K - m); ++p) {
+        const int mask = t.prefix_mask[p * fact(K - m)][m];
+        f.psi[m][p] = take(mask, 8);
+        if (m <= K - 3) f.qv[m][p] = take(mask, 16);
+      }
+    for (int g = 0; g < K; ++g) {
+      f.chi[g] = take(1 << g, 16);
+      f.qg[g] = take(1 << g, 16);
+    }
+    f.q0 = take(0, 16);
+    for (int g = 0; g < K; ++g)
+      for (int h = 0; h < K; ++h) {
+        if (g == h) continue;
+        f.z[g * kMaxGluons + h] = take(1 << g | 1 << h, 16);
+        if (K >= 4) f.qq[g * kMaxGluons + h] = take(1 << g | 1 << h, 16);
+      }
+    for (int i = 0; i < t.nfull; ++i) f.full[i] = take((1 << K) - 1, 4);
+    if (K == 5)
+      for (int s = 0; s < t.nseq; ++s)
+        for (int g = 0; g < K; ++g)
+          if (t.seq_len[s] == 2 && !((t.seq_mask[s] >> g) & 1)) f.y[s][g] = take(t.seq_mask[s] | 1 << g, 16);
+    if (own) o.nlocl = at;
+    else if (at > o.stride) o.stride = at;
+  }
   // ---- tasks ----
-  int nt = 0;
-  o.nltask = 0;
+  int nt = 0, ntl = 0;
+  o.nltask = o.nltaskl = 0;
+  auto tasksl = [&](Tab64::Type type, int a, int b, int mask) {
+    const uint32_t base = static_cast<uint32_t>(type) | static_cast<uint32_t>(a) << 4 | static_cast<uint32_t>(b) << 14;
+    o.ltaskl[o.nltaskl++] = base;
+    for (int gc = 0; gc < (1 << K); ++gc)
+      if ((gc & ~mask) == 0) o.taskl[ntl++] = base | static_cast<uint32_t>(gc) << 20;
+  };
   auto tasks = [&](Tab64::Type type, int a, int b, int mask) {
+    if (type != Tab64::kY || K == 5) tasksl(type, a, b, mask);
     const uint32_t base = static_cast<uint32_t>(type) | static_cast<uint32_t>(a) << 4 | static_cast<uint32_t>(b) << 14;
     o.ltask[o.nltask++] = base;
     for (int gc = 0; gc < top; ++gc)
@@ -189,7 +232,10 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
   auto psis = [&](int m) {
     for (int p = 0; p < t.ncol / fact(K - m); ++p) tasks(Tab64::kPsi, p, m, t.prefix_mask[p * fact(K - m)][m]);
   };
-  auto next_pass = [&] { o.pass0[++o.npass] = nt; };
+  auto next_pass = [&] {
+    o.pass0[++o.npass] = nt;
+    o.pass0l[o.npass] = ntl;
+  };
   for (int g = 0; g < K; ++g) tasks(Tab64::kJ1, g, 0, 1 << g);
   tasks(Tab64::kJq0, 0, 0, 0);
   psis(1);
@@ -197,10 +243,13 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
   for (int g = 0; g < K; ++g) tasks(Tab64::kChi, g, 0, 1 << g);
   next_pass();
   seqs(Tab64::kSeq, 2);
-  if (K == 5)
+  if (K >= 4)
     for (int g = 0; g < K; ++g)
       for (int h = 0; h < K; ++h)
-        if (g != h) tasks(Tab64::kQQ, g, h, 1 << g | 1 << h);
+        if (g != h) {
+          if (K == 5) tasks(Tab64::kQQ, g, h, 1 << g | 1 << h);
+          else tasksl(Tab64::kQQ, g, h, 1 << g | 1 << h);
+        }
   next_pass();
   if (K >= 4) {
     seqs(Tab64::kSeq, 3);
