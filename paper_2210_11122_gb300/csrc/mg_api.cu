@@ -171,8 +171,9 @@ cudaError_t free_raw(void* p, bool host) {
 
 int64_t share_doubles(int K) { return K >= 3 ? tab64_host(K).stride : 0; }
 
-int64_t share_chunk(int K, int64_t stride) {
-  const int64_t per_event = share_doubles(K);   // doubles
+int64_t amp_doubles(int K) { return K >= 3 ? (int64_t(4) << K) * factorial(K) : 0; }
+
+int64_t share_chunk(int64_t per_event, int64_t stride) {
   if (per_event == 0) return stride;
   int64_t chunk = (int64_t(1) << 28) / per_event / kPage * kPage;       // 2^28 doubles = 2 GiB
   if (chunk < kPage) chunk = kPage;
@@ -180,17 +181,27 @@ int64_t share_chunk(int K, int64_t stride) {
 }
 
 cudaError_t fp64_slots(mg_ctx* ctx, const double* mom, const double* rec, int64_t n, bool shared, const MeConst& cst,
-                       double* out, int64_t stride, float2* jout, MeShape shape, cudaStream_t st) {
+                       double* out, int64_t stride, MeShape shape, cudaStream_t st) {
   if (ctx->K == 2)
     return launch_me_gluonhel(2, false, false, mom, const_cast<double*>(rec), n, ctx->d_tab, ctx->d_hslots, 2,
-                              ctx->d_nhslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, out, stride, st, jout, shape);
-  const int* lin = jout ? nullptr : ctx->d_lin;   // (a sum of colour sums may be taken in either basis)
+                              ctx->d_nhslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, out, stride, st, nullptr, shape);
   if (shared) {
-    const cudaError_t e = launch_pass64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, cst, lin, ctx->d_share, st);
+    const cudaError_t e = launch_pass64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, cst, ctx->d_lin, ctx->d_share, st);
     if (e != cudaSuccess) return e;
   }
-  return launch_me64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, ctx->d_hslots, ctx->d_nhslots, lin, ctx->d_mask, ctx->d_ctri, cst,
-                     out, stride, jout, shape, shared ? ctx->d_share : nullptr, nullptr, st);
+  return launch_me64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, ctx->d_hslots, ctx->d_nhslots, ctx->d_lin, ctx->d_mask,
+                     ctx->d_ctri, cst, out, stride, shape, shared ? ctx->d_share : nullptr, st);
+}
+
+cudaError_t fp64_amps(mg_ctx* ctx, const double* rec, int64_t n, bool shared, const MeConst& cst, double** amp, MeShape shape,
+                      cudaStream_t st) {
+  *amp = ctx->d_share + (shared ? pad32(n) * share_doubles(ctx->K) : 0);
+  if (shared) {
+    const cudaError_t e = launch_pass64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, cst, nullptr, ctx->d_share, st);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_me64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, ctx->d_hslots, ctx->d_nhslots, nullptr, ctx->d_mask, ctx->d_ctri,
+                     cst, *amp, 0, shape, shared ? ctx->d_share : nullptr, st);
 }
 
 cudaError_t fp64_hel_sum(mg_ctx* ctx, int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st) {
@@ -383,6 +394,7 @@ void mg_destroy(mg_ctx* ctx) {
   mg::dev_free(ctx->d_nhslots);
   mg::dev_free(ctx->d_nhrows);
   mg::dev_free(ctx->d_lin);
+  mg::dev_free(ctx->d_nallrows);
   mg::dev_free(ctx->d_cmat);
   mg::dev_free(ctx->d_cumma);
   mg::dev_free(ctx->d_tcerr);
@@ -495,12 +507,14 @@ mg_status mg_create(mg_process proc, const mg_params* params, mg_ctx** out) {
     if (mg::dev_alloc(&c->d_gslots, 32 * sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_ngslots, sizeof(int)) != cudaSuccess ||
         mg::dev_alloc(&c->d_hslots, 16 * sizeof(int)) != cudaSuccess ||
         mg::dev_alloc(&c->d_nhslots, sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_nhrows, sizeof(int)) != cudaSuccess ||
-        mg::dev_alloc(&c->d_lin, sizeof(int)) != cudaSuccess ||
+        mg::dev_alloc(&c->d_lin, sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_nallrows, sizeof(int)) != cudaSuccess ||
         mg::dev_alloc(&c->d_allg, 32 * sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_nallg, sizeof(int)) != cudaSuccess) {
       st = MG_ENOMEM;
       break;
     }
-    if (cudaMemcpy(c->d_allg, all.data(), ng2 * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
+    const int nallrows = c->nhel / 2;
+    if (cudaMemcpy(c->d_nallrows, &nallrows, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(c->d_allg, all.data(), ng2 * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(c->d_nallg, &ng2, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(c->d_ngslots, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->d_nhslots, 0, sizeof(int)) != cudaSuccess ||
         cudaMemset(c->d_nhrows, 0, sizeof(int)) != cudaSuccess || cudaMemset(c->d_lin, 0, sizeof(int)) != cudaSuccess) {
@@ -686,10 +700,12 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
     if (chunk > stride) chunk = stride;
     // FP64 amplitudes: optionally the currents shared between gluon-helicity combinations (as MG_FP64)
     const bool shared = !fp32 && ctx->shape[precision].shared && ctx->K >= 3;
-    if (shared) {
-      const int64_t sc = mg::share_chunk(ctx->K, stride);
+    const bool amps = !fp32 && ctx->K >= 3;
+    if (amps) {
+      const int64_t need = (shared ? mg::share_doubles(ctx->K) : 0) + mg::amp_doubles(ctx->K);
+      const int64_t sc = mg::share_chunk(need, stride);
       if (sc < chunk) chunk = sc;
-      s = grow(&ctx->d_share, &ctx->share_cap, chunk * mg::share_doubles(ctx->K));
+      s = grow(&ctx->d_share, &ctx->share_cap, chunk * need);
       if (s != MG_OK) return s;
     }
     if (ctx->jamp_cap < chunk * per_event) {
@@ -724,22 +740,28 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
         MG_CUDA(mg::launch_me_warp(ctx->K, ctx->d_prep, n, ctx->d_tab, ctx->d_gslots, 1 << ctx->K, ctx->d_ngslots,
                                    ctx->d_mask, ctx->d_cfull, ctx->d_cmat, 1, cst, ctx->d_part, cst_stride, ctx->d_jamps,
                                    ctx->d_flag, st));
-      else if (!fp32)
-        MG_CUDA(mg::fp64_slots(ctx, mom_c, ctx->d_prep, n, shared, cst, ctx->d_part, cst_stride, ctx->d_jamps,
-                               ctx->shape[precision], st));
+      else if (amps) {
+        double* amp = nullptr;
+        MG_CUDA(mg::fp64_amps(ctx, ctx->d_prep, n, shared, cst, &amp, ctx->shape[precision], st));
+        MG_CUDA(mg::launch_helicities(ctx->K, amp, n, ctx->d_tab64, ctx->d_mask, ctx->d_ctri, cst.colour_scale, nullptr, 0,
+                                      ctx->d_jamps, nullptr, st));
+      }
       else
-        MG_CUDA(mg::launch_me_gluonhel(ctx->K, true, false, mom_c, ctx->d_prep, n, ctx->d_tab, slots, maxslot, nslots,
+        MG_CUDA(mg::launch_me_gluonhel(ctx->K, fp32, false, mom_c, ctx->d_prep, n, ctx->d_tab, slots, maxslot, nslots,
                                        ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, ctx->d_part, cst_stride, st,
-                                       ctx->d_jamps, ctx->shape[precision], ctx->d_flag));
+                                       ctx->d_jamps, ctx->shape[precision], fp32 ? ctx->d_flag : nullptr));
+      const int* nrows = amps ? ctx->d_nallrows : half ? ctx->d_nhrows : ctx->d_nrows;
       if (ctx->shape[precision].tc_sync)
-        MG_CUDA(mg::launch_colour_tc(ctx->ncol, ctx->d_jamps, n, rows, half ? ctx->d_nhrows : ctx->d_nrows, ctx->d_cmat, cst.colour_scale,
+        MG_CUDA(mg::launch_colour_tc(ctx->ncol, ctx->d_jamps, n, rows, nrows, ctx->d_cmat, cst.colour_scale,
                                      ctx->d_part, cst_stride, st, fp32 ? ctx->d_flag : nullptr));
       else
-        MG_CUDA(mg::launch_colour_umma(ctx->ncol, ctx->d_jamps, n, rows, half ? ctx->d_nhrows : ctx->d_nrows, ctx->d_cumma, cst.colour_scale,
+        MG_CUDA(mg::launch_colour_umma(ctx->ncol, ctx->d_jamps, n, rows, nrows, ctx->d_cumma, cst.colour_scale,
                                        ctx->d_part, cst_stride, st, fp32 ? ctx->d_flag : nullptr, ctx->d_tcerr,
                                        ctx->tc_stall));
       if (fp32) MG_CUDA(join_repair(ctx, st));
-      if (half)   // (the colour pass writes a row per helicity for every process)
+      if (amps)
+        MG_CUDA(mg::launch_hel_sum_top(ctx->K, ctx->d_part, ctx->d_mask, n, cst_stride, norm, me_dev + e0, st));
+      else if (half)   // (2 gluons: the colour pass writes a row per helicity of the half list)
         MG_CUDA(mg::launch_hel_sum_rows(ctx->K, ctx->d_part, slots, nslots, nullptr, ctx->d_mask, n, cst_stride, norm, me_dev + e0, st));
       else
         MG_CUDA(mg::launch_hel_sum(ctx->d_part, ctx->d_nrows, n, cst_stride, norm, me_dev + e0, st));
@@ -763,7 +785,7 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
     const bool shared = !fp32 && ctx->shape[precision].shared && ctx->K >= 3;
     if (!fp32) {
       // with shared items, in chunks of events that bound their buffer
-      const int64_t chunk = shared ? mg::share_chunk(ctx->K, stride) : stride;
+      const int64_t chunk = shared ? mg::share_chunk(mg::share_doubles(ctx->K), stride) : stride;
       if (shared) s = grow(&ctx->d_share, &ctx->share_cap, chunk * mg::share_doubles(ctx->K));
       if (s != MG_OK) return s;
       const int64_t nitem = mg::event_record_bytes(ctx->K, false) / 8;
@@ -771,7 +793,7 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
         const int64_t n = nevt - e0 < chunk ? nevt - e0 : chunk;
         MG_CUDA(mg::fp64_slots(ctx, mom_dev + (e0 / mg::kPage) * ctx->npar * 4 * mg::kPage,
                                ctx->d_prep + (e0 / mg::kPage) * nitem * mg::kPage, n, shared, cst, ctx->d_part + e0, stride,
-                               nullptr, ctx->shape[precision], st));
+                               ctx->shape[precision], st));
       }
     } else if (fused)
       MG_CUDA(mg::launch_me_fused(ctx->K, true, mom_dev, nevt, ctx->d_gslots, ctx->d_ngslots, ctx->d_mask, cst,

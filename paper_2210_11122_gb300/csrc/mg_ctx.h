@@ -28,6 +28,7 @@ struct mg_ctx {
   int* d_hslots = nullptr;    // FP64: one of each pair of flipped gluon combinations (hel_weight)
   int* d_nhslots = nullptr;
   int* d_nhrows = nullptr;
+  int* d_nallrows = nullptr;  // nhel / 2: the rows of launch_helicities
   int* d_lin = nullptr;       // 1: every helicity is good (FP64 sums over linear polarisations)
   void* d_cmat = nullptr;     // colour matrix numerators as the packed FP16 tensor-core operand
   void* d_cumma = nullptr;    // the same as the tcgen05 B operand (canonical no-swizzle K-major layout)
@@ -76,15 +77,21 @@ struct mg_ctx {
 
 
 namespace mg {
-// doubles per event of the items shared between FP64 gluon-helicity combinations (0 for 2 gluons: none are), and
-// events per chunk (the buffer stays within 2 GiB)
+// FP64: doubles per event of the items shared between combinations (0 for 2 gluons: none are) and of the amplitudes of
+// every row (LHE choices and FP64 amplitudes for the tensor-core colour sum, 3 to 5 gluons); a buffer of per_event doubles
+// in chunks of events of at most 2 GiB
 int64_t share_doubles(int K);
-int64_t share_chunk(int K, int64_t stride);
-// FP64 amplitudes of n events (from a page boundary: momenta mom, FP64 records rec; zero top width) for the context's
-// half list of gluon-helicity combinations: colour sums or jamps as launch_me64.  shared: through the items buffer
-// (d_share, share_doubles(K) * pad(n) doubles, 3 to 5 gluons), else every combination on its own.
+int64_t amp_doubles(int K);
+int64_t share_chunk(int64_t per_event, int64_t stride);
+// FP64 colour sums of n events (from a page boundary: momenta mom, FP64 records rec; zero top width) in rows of out, for
+// fp64_hel_sum.  shared: through the items buffer (d_share, share_doubles(K) * pad(n) doubles, 3 to 5 gluons), else every
+// combination on its own.
 cudaError_t fp64_slots(mg_ctx* ctx, const double* mom, const double* rec, int64_t n, bool shared, const MeConst& cst,
-                       double* out, int64_t stride, float2* jout, MeShape shape, cudaStream_t st);
+                       double* out, int64_t stride, MeShape shape, cudaStream_t st);
+// FP64 amplitudes of n events, 3 to 5 gluons, for launch_helicities; d_share holds amp_doubles(K) and, shared, also
+// share_doubles(K) doubles for each of pad(n) events; the amplitudes' place in it is returned in *amp.
+cudaError_t fp64_amps(mg_ctx* ctx, const double* rec, int64_t n, bool shared, const MeConst& cst, double** amp, MeShape shape,
+                      cudaStream_t st);
 // The helicity sum of fp64_slots' colour sums in d_part (per combination for 2 gluons, per helicity for 3 to 5).
 cudaError_t fp64_hel_sum(mg_ctx* ctx, int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st);
 // MG_MIXED on the lane-group kernel: colour sums on the tensor cores inside it, per-slot outputs

@@ -81,21 +81,23 @@ cudaError_t launch_me_gluonhel(int K, bool fp32, bool per_hel, const double* mom
                                double* out, int64_t stride, cudaStream_t st, float2* jout = nullptr,
                                MeShape shape = MeShape(), const uint8_t* skip = nullptr,
                                const int* evlist = nullptr, const int* nlist = nullptr, int rows_out = 0);
-// FP64 matrix elements of 3 to 5 gluons from the FP64 records of nevt events (mg_me64.cuh).  launch_pass64 fills the
-// items shared between gluon-helicity combinations (tab64_host(K).stride doubles per event, page-interleaved), a
-// few launches; launch_me64 runs one thread per (event, helicity of the combinations hslots), reading them, or with
-// share = null one per (event, combination) computing its own (the same bits).  Output, rows r = slot * 4 + 2 top +
-// antitop (cst.conj = 1): the colour sums out[r * stride + e], zero for weight 0; with jout the FP32 jamps instead (2^(K+1)
-// rows per event); with j2 also the weighted jamp squares j2[(r * ncol + sigma) * stride + e].
-// lin (may be null; colour sums only): a device flag, nonzero where every helicity is good: then the sum runs over
-// linear gluon polarisations (mg_me64l.cuh), rows 2 * polarisations + antitop helicity; the same for both calls and for
-// launch_hel_sum_rows.
+// FP64 matrix elements of 3 to 5 gluons from the FP64 records of nevt events (mg_me64.cuh, mg_me64l.cuh).  launch_pass64
+// fills the items shared between combinations (tab64_host(K).stride doubles per event, page-interleaved), a few launches;
+// launch_me64 reads them, or with share = null every thread computes its own (the same bits).
+// lin != null: the colour sums out[r * stride + e] of one of each pair of flipped helicities (cst.conj = 1), rows r = slot
+// * 4 + 2 top + antitop of hslots, 0 for weight 0; or, where *lin != 0 (every helicity good), of the linear gluon
+// polarisations, rows 2 * polarisations + antitop helicity (launch_hel_sum_rows takes the same flag).
+// lin = null: the linear polarisations' amplitudes into out, interleaved by page (2^(K+2) ncol doubles per event), which
+// launch_helicities turns into the helicities' with top helicity -1, rows 2 * gluon helicities + antitop helicity: as
+// FP32 jamps in jout, or (jout null) as colour sums out[row * stride + e] and the weighted jamp squares summed over each
+// antitop helicity's rows, j2[(b * ncol + sigma) * stride + e].
 cudaError_t launch_pass64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const MeConst& cst,
                           const int* lin, double* share, cudaStream_t st);
 cudaError_t launch_me64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const int* hslots,
                         const int* nslot, const int* lin, const uint32_t* mask, const double* ctri, const MeConst& cst,
-                        double* out, int64_t stride, float2* jout, MeShape shape, const double* share, double* j2,
-                        cudaStream_t st);
+                        double* out, int64_t stride, MeShape shape, const double* share, cudaStream_t st);
+cudaError_t launch_helicities(int K, double* amp, int64_t nevt, const Tab64* t64, const uint32_t* mask, const double* ctri,
+                              double scale, double* out, int64_t stride, float2* jout, double* j2, cudaStream_t st);
 int64_t event_record_bytes(int K, bool fp32);
 // The FP32 modes' recomputation of events evlist[0..*nlist) with double-float amplitudes (mg_me_dd.cu):
 // launch_me_gluonhel's contract for prep == NULL, per_hel false, FP32 colour table ctri32 (the per-thread
@@ -152,6 +154,9 @@ cudaError_t launch_colour_tc(int ncol, const float2* jamps, int64_t nevt, int ro
 // if every helicity is good, else 0.
 cudaError_t launch_gluon_slots(const uint32_t* mask, int K, int* gslots, int* n, int* nrows, int* hslots, int* nh,
                                int* nhrows, int* lin, cudaStream_t st);
+// me[e] = norm * sum over launch_helicities' rows of hel_weight * part[row * stride + e]
+cudaError_t launch_hel_sum_top(int K, const double* part, const uint32_t* mask, int64_t nevt, int64_t stride, double norm,
+                               double* me, cudaStream_t st);
 // me[e] = norm * sum over the rows of hslots (slot * 4 + 2 top + antitop) of hel_weight * part[row * stride + e]; where
 // *lin != 0 (lin may be null) over all 2^(K+1) rows of the linear polarisations, each for 2^(K+1) times its value
 cudaError_t launch_hel_sum_rows(int K, const double* part, const int* hslots, const int* nh, const int* lin, const uint32_t* mask,

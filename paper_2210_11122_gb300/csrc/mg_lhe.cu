@@ -63,8 +63,8 @@ __device__ __forceinline__ double coupling_factor(double a0, double mu, double* 
 }
 
 // One thread per event: helicity sum (ascending helicity index), helicity and colour choices, coupling.
-// part rows: slot * 4 + 2 top + antitop (launch_me64 with j2); j2: jamp-square sums, per
-// helicity row (3 to 5 gluons) or per slot (2).
+// part rows: launch_helicities' (3 to 5 gluons) or slot * 4 + 2 top + antitop (2); j2: jamp-square sums, per antitop
+// helicity or per slot.
 template <int K>
 __global__ void __launch_bounds__(128)
 k_lhe_epilogue(const double* __restrict__ part, const double* __restrict__ j2, const int* __restrict__ gslots,
@@ -85,6 +85,7 @@ k_lhe_epilogue(const double* __restrict__ part, const double* __restrict__ j2, c
 #pragma unroll
     for (int g = 0; g < K; ++g) gc |= ((h >> (npar - 1 - (g < 2 ? g : g + 2))) & 1) << g;
     const int a = (h >> (npar - 3)) & 1, b = (h >> (npar - 4)) & 1;
+    if constexpr (K >= 3) return a ? 2 * ((1 << K) - 1 - gc) + (1 - b) : 2 * gc + b;   // (launch_helicities' rows)
     // the flipped helicity has the same |M_h|^2, in the slot of the flipped combination
     if (gc >> (K - 1)) return slot_of[(1 << K) - 1 - gc] * 4 + 2 * (1 - a) + (1 - b);
     return slot_of[gc] * 4 + 2 * a + b;
@@ -117,7 +118,7 @@ k_lhe_epilogue(const double* __restrict__ part, const double* __restrict__ j2, c
     double totc = 0.0;
     for (int c = 0; c < NCOL; ++c) {
       double acc = 0.0;
-      for (int s = 0; s < (K >= 3 ? 4 * nslot : nslot); ++s) acc += j2[(static_cast<int64_t>(s) * NCOL + c) * stride + e];
+      for (int s = 0; s < (K >= 3 ? 2 : nslot); ++s) acc += j2[(static_cast<int64_t>(s) * NCOL + c) * stride + e];
       w[c] = acc;
       totc += acc;
     }
@@ -176,13 +177,9 @@ mg_status grow_buf(double** buf, int64_t* cap, int64_t need) {
   return MG_OK;
 }
 
-// The slots' colour sums per helicity and jamp squares; share: the chunk's items from launch_pass64 (3 to 5 gluons),
-// or null: every combination on its own (the same bits)
-cudaError_t lhe_me(int K, const double* rec, int64_t nevt, const mg_ctx* c, const mg::MeConst& cst, double* part,
-                   double* j2, int64_t stride, const double* share, cudaStream_t st) {
-  if (K >= 3)
-    return mg::launch_me64(K, rec, nevt, c->d_tab, c->d_tab64, c->d_hslots, c->d_nhslots, nullptr, c->d_mask, c->d_ctri,
-                           cst, part, stride, nullptr, mg::MeShape(), share, j2, st);
+// 2 gluons: the colour sum of every helicity of the half list in its own row and the jamp squares per slot
+cudaError_t lhe_me2(const double* rec, int64_t nevt, const mg_ctx* c, const mg::MeConst& cst, double* part, double* j2,
+                    int64_t stride, cudaStream_t st) {
   constexpr int tev = mg::kMeThreads;
   const dim3 grid(static_cast<unsigned>((nevt + tev - 1) / tev), 2);
   mg::v2::k_me_gluonhel<2, double, false, true, false, true><<<grid, mg::kMeThreads, 0, st>>>(
@@ -224,22 +221,17 @@ mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, cons
   }
   ctx->last = st;
   const int K = ctx->K;
-  // chunks of whole pages that keep the per-slot jamp-square sums within 2^27 doubles (1 GiB)
-  const int64_t per_event = static_cast<int64_t>(K >= 3 ? ctx->nhel / 2 : 1 << (K - 1)) * ctx->ncol;
-  int64_t chunk = (int64_t(1) << 27) / per_event / mg::kPage * mg::kPage;
+  // 3 to 5 gluons: the amplitudes (and, as the FP64 launch shape says, the shared items) in chunks of whole pages of at
+  // most 2 GiB; 2 gluons: chunks of 2^27 doubles of jamp squares
+  const int64_t j2rows = 2 * ctx->ncol;   // per antitop helicity, or per slot
   const int64_t stride_all = pad_page(nevt);
-  if (chunk < mg::kPage) chunk = mg::kPage;
-  if (chunk > stride_all) chunk = stride_all;
-  // the FP64 launch shape's choice of shared items (chunks within their buffer)
   const bool shared = ctx->shape[MG_FP64].shared && K >= 3;
-  if (shared) {
-    const int64_t sc = mg::share_chunk(K, stride_all);
-    if (sc < chunk) chunk = sc;
-  }
+  const int64_t need = (shared ? mg::share_doubles(K) : 0) + mg::amp_doubles(K);
+  int64_t chunk = K >= 3 ? mg::share_chunk(need, stride_all) : mg::share_chunk(2 * j2rows, stride_all);
   mg_status s = grow_buf(&ctx->d_part, &ctx->part_cap, chunk * ctx->nhel);
   if (s == MG_OK) s = grow_buf(&ctx->d_prep, &ctx->prep_cap, chunk * mg::event_record_bytes(K, false) / 8 + 1);
-  if (s == MG_OK) s = grow_buf(&ctx->d_j2, &ctx->j2_cap, chunk * per_event);
-  if (s == MG_OK && shared) s = grow_buf(&ctx->d_share, &ctx->share_cap, chunk * mg::share_doubles(K));
+  if (s == MG_OK) s = grow_buf(&ctx->d_j2, &ctx->j2_cap, chunk * j2rows);
+  if (s == MG_OK && need > 0) s = grow_buf(&ctx->d_share, &ctx->share_cap, chunk * need);
   if (s != MG_OK) return s;
   mg::MeConst cst;
   cst.gs = std::sqrt(4.0 * 3.14159265358979323846 * ctx->prm.alphas);
@@ -253,10 +245,15 @@ mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, cons
     const int64_t stride = pad_page(n);
     const double* mom_c = mom_dev + (e0 / mg::kPage) * ctx->npar * 4 * mg::kPage;
     if (mg::launch_event_prep(K, false, mom_c, n, cst, ctx->d_prep, st) != cudaSuccess) return MG_ECUDA;
-    if (shared && mg::launch_pass64(K, ctx->d_prep, n, ctx->d_tab, ctx->d_tab64, cst, nullptr, ctx->d_share, st) != cudaSuccess) return MG_ECUDA;
-    if (lhe_me(K, ctx->d_prep, n, ctx, cst, ctx->d_part, ctx->d_j2, stride, shared ? ctx->d_share : nullptr, st) !=
-        cudaSuccess)
+    if (K >= 3) {
+      double* amp = nullptr;
+      if (mg::fp64_amps(ctx, ctx->d_prep, n, shared, cst, &amp, ctx->shape[MG_FP64], st) != cudaSuccess ||
+          mg::launch_helicities(K, amp, n, ctx->d_tab64, ctx->d_mask, ctx->d_ctri, cst.colour_scale, ctx->d_part, stride, nullptr,
+                                ctx->d_j2, st) != cudaSuccess)
+        return MG_ECUDA;
+    } else if (lhe_me2(ctx->d_prep, n, ctx, cst, ctx->d_part, ctx->d_j2, stride, st) != cudaSuccess) {
       return MG_ECUDA;
+    }
     if (lhe_epilogue(K, ctx->d_j2, ctx, mom_c, n, stride, norm, running_alphas, rnd_hel_dev ? rnd_hel_dev + e0 : nullptr,
                      rnd_col_dev ? rnd_col_dev + e0 : nullptr, me_dev + e0, hel_dev ? hel_dev + e0 : nullptr,
                      col_dev ? col_dev + e0 : nullptr, alphas_dev ? alphas_dev + e0 : nullptr, st) != cudaSuccess)

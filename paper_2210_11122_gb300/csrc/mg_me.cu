@@ -414,6 +414,23 @@ __global__ void k_hel_sum_rows(int K, const double* __restrict__ part, const int
   me[e] = s * norm;
 }
 
+// me[e] = norm * sum over the rows 2 * gluon helicities + antitop helicity (top helicity -1)
+__global__ void k_hel_sum_top(int K, const double* __restrict__ part, const uint32_t* __restrict__ mask, int64_t nevt,
+                              int64_t stride, double norm, double* __restrict__ me) {
+  const int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  if (e >= nevt) return;
+  const int npar = K + 2;
+  double s = 0.0;
+  for (int r = 0; r < (2 << K); ++r) {
+    int h = (r & 1) << (npar - 4);
+    for (int g = 0; g < K; ++g)
+      if ((r >> (g + 1)) & 1) h |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
+    const int w = hel_weight(mask, h, npar, 1);
+    if (w) s = fma(static_cast<double>(w), part[r * stride + e], s);
+  }
+  me[e] = s * norm;
+}
+
 // helicity filter, step 1: maxr[h] = max over the warm-up events of part[h][e] / tot[e]
 // (one block per helicity, fixed-shape tree reduction: order-independent maximum).
 __global__ void k_hel_ratio_max(const double* __restrict__ part, const double* __restrict__ tot, int64_t nevt,
@@ -492,6 +509,15 @@ cudaError_t launch_hel_sum_rows(int K, const double* part, const int* hslots, co
   const unsigned blocks = static_cast<unsigned>((nevt + threads - 1) / threads);
   if (blocks == 0) return cudaSuccess;
   { k_hel_sum_rows<<<blocks, threads, 0, st>>>(K, part, hslots, nh, lin, mask, nevt, stride, norm, me); mg::note_launch(); }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_hel_sum_top(int K, const double* part, const uint32_t* mask, int64_t nevt, int64_t stride, double norm,
+                               double* me, cudaStream_t st) {
+  const int threads = 256;
+  const unsigned blocks = static_cast<unsigned>((nevt + threads - 1) / threads);
+  if (blocks == 0) return cudaSuccess;
+  { k_hel_sum_top<<<blocks, threads, 0, st>>>(K, part, mask, nevt, stride, norm, me); mg::note_launch(); }
   return cudaGetLastError();
 }
 

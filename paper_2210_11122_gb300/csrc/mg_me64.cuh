@@ -316,8 +316,6 @@ __device__ __forceinline__ void run_task(const View<K, LOCAL>& V, uint32_t task)
   }
 }
 
-constexpr int kME = 0, kJamps = 1, kLhe = 2;
-
 // sums and differences of the 2^N complex numbers a[0 .. 2^N) over each bit of their index
 template <int N>
 __device__ __forceinline__ void signed_sums(cx<double>* a) {
@@ -378,14 +376,12 @@ __device__ __forceinline__ double colour_sum64(cx<double>* A, const Tab64* __res
   }
 }
 
-// The amplitudes of one (event, combination, top helicity pair ab = 2 top + antitop) and what the mode makes of them,
-// in row slot * 4 + ab: kME: out[row * stride + e] = the colour sum (0 for weight 0); kJamps: FP32 jamps of jout's
-// row (zeros for weight 0); kLhe: kME and j2[(row * ncol + sigma) * stride + e] = weight * |jamp|^2.
-template <int K, int MODE, bool LOCAL>
+// The colour sum of one (event, combination, top helicity pair ab = 2 top + antitop) into row slot * 4 + ab:
+// out[row * stride + e], 0 for weight 0.
+template <int K, bool LOCAL>
 __device__ __forceinline__ void slot64(const View<K, LOCAL>& V, int64_t e, int slot, int ab,
                                        const uint32_t* __restrict__ mask, const double* __restrict__ ctri,
-                                       const MeConst& cst, double* __restrict__ out, int64_t stride,
-                                       float2* __restrict__ jout, double* __restrict__ j2) {
+                                       const MeConst& cst, double* __restrict__ out, int64_t stride) {
   constexpr int npar = K + 2, NCOL = v2::Sizes<K>::ncol, NFULL = v2::Sizes<K>::nfull;
   constexpr bool kNegK = (K & 1) == 0, kNegK1 = !kNegK;   // reflection signs of K and K-1 gluons: negative?
   const Tab64* t = V.t;
@@ -396,13 +392,7 @@ __device__ __forceinline__ void slot64(const View<K, LOCAL>& V, int64_t e, int s
     if ((V.gc >> g) & 1) hb |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
   const int w = hel_weight(mask, hb, npar, cst.conj);
   if (!w) {
-    if constexpr (MODE == kJamps) {
-      for (int c = 0; c < NCOL; ++c) jout[(e * (2 << K) + row) * NCOL + c] = make_float2(0.f, 0.f);
-    } else {
-      out[row * stride + e] = 0.0;
-      if constexpr (MODE == kLhe)
-        for (int c = 0; c < NCOL; ++c) j2[(static_cast<int64_t>(row) * NCOL + c) * stride + e] = 0.0;
-    }
+    out[row * stride + e] = 0.0;
     return;
   }
   cx<double> A[NCOL];
@@ -497,16 +487,7 @@ __device__ __forceinline__ void slot64(const View<K, LOCAL>& V, int64_t e, int s
     for (int c = 0; c < 6; ++c) add(6 * p + c, acc[c], false);
   }
 
-  if constexpr (MODE == kJamps) {
-    float2* o = jout + (e * (2 << K) + row) * NCOL;
-    for (int c = 0; c < NCOL; ++c) o[c] = make_float2(static_cast<float>(A[c].r), static_cast<float>(A[c].i));
-  } else {
-    if constexpr (MODE == kLhe)
-      for (int c = 0; c < NCOL; ++c)
-        j2[(static_cast<int64_t>(row) * NCOL + c) * stride + e] =
-            static_cast<double>(w) * fma(A[c].r, A[c].r, A[c].i * A[c].i);
-    out[row * stride + e] = colour_sum64<K>(A, t, ctri) * cst.colour_scale;
-  }
+  out[row * stride + e] = colour_sum64<K>(A, t, ctri) * cst.colour_scale;
 }
 
 }  // namespace m64

@@ -336,14 +336,12 @@ __device__ __forceinline__ void run_task_l(const ViewL<K, LOCAL>& V, uint32_t ta
   }
 }
 
-// The colour sum of one (event, polarisation combination, antitop helicity b) into out.
+// The amplitudes of one (event, polarisation combination, antitop helicity b).
 template <int K, bool LOCAL>
-__device__ __forceinline__ void row64_l(const ViewL<K, LOCAL>& V, int b, const double* __restrict__ ctri, double scale,
-                                        double* __restrict__ out) {
+__device__ __forceinline__ void row64_l(const ViewL<K, LOCAL>& V, int b, cx<double>* A) {
   constexpr int NCOL = v2::Sizes<K>::ncol, NFULL = v2::Sizes<K>::nfull;
   constexpr bool kNegK = (K & 1) == 0, kNegK1 = !kNegK;
   const Tab64* t = V.t;
-  cx<double> A[NCOL];
   for (int f = 0; f < NFULL; ++f) {
     const double* p = V.buf + static_cast<int64_t>(V.offFull(f) + 2 * b) * ViewL<K, LOCAL>::ST;
     const cx<double> x = {p[0], p[ViewL<K, LOCAL>::ST]};
@@ -438,7 +436,14 @@ __device__ __forceinline__ void row64_l(const ViewL<K, LOCAL>& V, int b, const d
 #pragma unroll
     for (int c = 0; c < 6; ++c) add(6 * p + c, acc[c], false);
   }
-  *out = colour_sum64<K>(A, t, ctri) * scale;
+}
+
+// amplitude of (event, row, ordering) in a buffer of all of them, interleaved by page
+template <int K>
+__host__ __device__ constexpr int amp_doubles() { return (2 << K) * v2::Sizes<K>::ncol * 2; }
+template <int K>
+__device__ __forceinline__ double* amp_at(double* amp, int64_t e, int row, int c) {
+  return amp + (e / kPage) * static_cast<int64_t>(amp_doubles<K>()) * kPage + (row * v2::Sizes<K>::ncol + c) * 2 * kPage + e % kPage;
 }
 
 // A warp takes one top helicity pair of one combination (the all-gluon currents, which the pairs share, are items
@@ -446,45 +451,84 @@ __device__ __forceinline__ void row64_l(const ViewL<K, LOCAL>& V, int b, const d
 // 4.1 per sub-partition, so the busiest had 5; measured 2.81 vs 3.19 ms there, gg->ttggg + TC colour 7.60 vs 8.60 ms
 // per 2,049 events, gg->ttg 12.05 vs 12.13 ms per 524,288.
 //
-// One thread of a block (32 events x 4 warps) on event tile `tile`, block `blk` < 2^(K-1) of the tile.  lin (kME only,
-// may be null): *lin != 0: linear polarisations, warp w on row 4 blk + w = 2 * polarisations + antitop helicity; else
-// helicities: with the shared items warp w on the top helicity pair w of combination hslots[blk]; without them (LOCAL)
-// on the four pairs of combination hslots[4 blk + w], whose items it builds once.
-template <int K, int MODE, bool LOCAL>
+// One thread of a block (32 events x 4 warps) on event tile `tile`, block `blk` < 2^(K-1) of the tile.
+// amp (AMP): the amplitudes of row 4 blk + w = 2 * polarisations + antitop helicity for warp w.  Else the colour sums:
+// *lin != 0: of the same row, into out[row * stride + e]; *lin = 0: of helicities, with the shared items warp w on the
+// top helicity pair w of combination hslots[blk]; without them (LOCAL) on the four pairs of combination
+// hslots[4 blk + w], whose items it builds once.
+template <int K, bool AMP, bool LOCAL>
 __device__ __forceinline__ void thread64(const double* __restrict__ rec, int64_t nevt, int64_t tile, int blk,
                                          const Tables* __restrict__ tab, const Tab64* __restrict__ t64,
                                          const int* __restrict__ hslots, const int* __restrict__ nslot,
                                          const int* __restrict__ lin, const uint32_t* __restrict__ mask,
                                          const double* __restrict__ ctri, const MeConst& cst, double* __restrict__ out,
-                                         int64_t stride, float2* __restrict__ jout, const double* __restrict__ share,
-                                         double* __restrict__ j2) {
+                                         int64_t stride, const double* __restrict__ share) {
+  constexpr int NCOL = v2::Sizes<K>::ncol;
   const int64_t e = tile * kPage + threadIdx.x % kPage;
   const int warp = threadIdx.x / kPage;
   if (e >= nevt) return;
   const double* in = rec + (e / kPage) * v2::EvLayout<K>::NITEM * kPage + (e % kPage);
-  double own[LOCAL ? (Loc<K>::n > LocL<K>::n ? Loc<K>::n : LocL<K>::n) : 1];
+  double own[!LOCAL ? 1 : AMP || Loc<K>::n < LocL<K>::n ? LocL<K>::n : Loc<K>::n];
   double* buf = own;
   if constexpr (!LOCAL)
     buf = const_cast<double*>(share) + (e / kPage) * static_cast<int64_t>(t64->stride) * kPage + (e % kPage);
-  if constexpr (MODE == kME) {
-    if (lin && *lin) {
-      const int row = 4 * blk + warp;
-      const ViewL<K, LOCAL> V = {in, buf, tab, t64, LOCAL ? &t64->locl : &t64->shl, row >> 1, cst.gs};
-      if constexpr (LOCAL)
-        for (int i = 0; i < t64->nltaskl; ++i) run_task_l<K, true>(V, t64->ltaskl[i]);
-      row64_l<K, LOCAL>(V, row & 1, ctri, cst.colour_scale, out + row * stride + e);
-      return;
+  if (AMP || *lin) {
+    const int row = 4 * blk + warp;
+    const ViewL<K, LOCAL> V = {in, buf, tab, t64, LOCAL ? &t64->locl : &t64->shl, row >> 1, cst.gs};
+    if constexpr (LOCAL)
+      for (int i = 0; i < t64->nltaskl; ++i) run_task_l<K, true>(V, t64->ltaskl[i]);
+    cx<double> A[NCOL];
+    row64_l<K, LOCAL>(V, row & 1, A);
+    if constexpr (AMP) {
+      double* p = amp_at<K>(out, e, row, 0);
+      for (int c = 0; c < NCOL; ++c) {
+        p[2 * c * kPage] = A[c].r;
+        p[(2 * c + 1) * kPage] = A[c].i;
+      }
+    } else {
+      out[row * stride + e] = colour_sum64<K>(A, t64, ctri) * cst.colour_scale;
+    }
+    return;
+  }
+  if constexpr (!AMP) {
+    const int slot = LOCAL ? 4 * blk + warp : blk;
+    if (slot >= *nslot) return;
+    const View<K, LOCAL> V = {in, buf, tab, t64, LOCAL ? &t64->loc : &t64->sh, hslots[slot], cst.gs};
+    if constexpr (LOCAL) {
+      for (int i = 0; i < t64->nltask; ++i) run_task<K, true>(V, t64->ltask[i]);
+      for (int ab = 0; ab < 4; ++ab) slot64<K, true>(V, e, slot, ab, mask, ctri, cst, out, stride);
+    } else {
+      slot64<K, false>(V, e, slot, warp, mask, ctri, cst, out, stride);
     }
   }
-  const int slot = LOCAL ? 4 * blk + warp : blk;
-  if (slot >= *nslot) return;
-  const View<K, LOCAL> V = {in, buf, tab, t64, LOCAL ? &t64->loc : &t64->sh, hslots[slot], cst.gs};
-  if constexpr (LOCAL) {
-    for (int i = 0; i < t64->nltask; ++i) run_task<K, true>(V, t64->ltask[i]);
-    for (int ab = 0; ab < 4; ++ab) slot64<K, MODE, true>(V, e, slot, ab, mask, ctri, cst, out, stride, jout, j2);
-  } else {
-    slot64<K, MODE, false>(V, e, slot, warp, mask, ctri, cst, out, stride, jout, j2);
-  }
+}
+
+// From the linear polarisations' amplitudes of one (event, ordering, antitop helicity b) to the helicities': per gluon
+// M(+) = -M(theta) + i s M(phi), M(-) = M(theta) + i s M(phi), s = +1 outgoing (ext_gluon).  a[x]: bit g of x = phi in,
+// helicity +1 out; top helicity -1 throughout.
+template <int K>
+__device__ __forceinline__ void to_helicities(cx<double>* a) {
+#pragma unroll
+  for (int g = 0; g < K; ++g)
+#pragma unroll
+    for (int x = 0; x < (1 << K); ++x)
+      if (!((x >> g) & 1)) {
+        const cx<double> t = a[x], f = a[x | 1 << g];
+        const cx<double> p = g < 2 ? cx<double>{f.i, -f.r} : cx<double>{-f.i, f.r};   // i s M(phi)
+        a[x] = {t.r + p.r, t.i + p.i};
+        a[x | 1 << g] = {p.r - t.r, p.i - t.i};
+      }
+}
+
+// helicity index of gluon helicities x (bit g: +1), top helicity -1, antitop helicity b
+template <int K>
+__device__ __forceinline__ int hel_of_row(int x, int b) {
+  constexpr int npar = K + 2;
+  int h = b << (npar - 4);
+#pragma unroll
+  for (int g = 0; g < K; ++g)
+    if ((x >> g) & 1) h |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
+  return h;
 }
 
 }  // namespace m64

@@ -56,11 +56,11 @@ struct PBatch {
 template <int K>
 __device__ __forceinline__ void run64(const PJob& J, int64_t tile, int blk) {
   if (J.share)
-    m64::thread64<K, m64::kME, false>(J.rec, J.nevt, tile, blk, J.tab, J.t64, J.gslots, J.nslot, J.lin, J.mask, J.ctri, J.cst,
-                                      J.part, J.stride, nullptr, J.share, nullptr);
+    m64::thread64<K, false, false>(J.rec, J.nevt, tile, blk, J.tab, J.t64, J.gslots, J.nslot, J.lin, J.mask, J.ctri, J.cst,
+                                   J.part, J.stride, J.share);
   else
-    m64::thread64<K, m64::kME, true>(J.rec, J.nevt, tile, blk, J.tab, J.t64, J.gslots, J.nslot, J.lin, J.mask, J.ctri, J.cst,
-                                     J.part, J.stride, nullptr, nullptr, nullptr);
+    m64::thread64<K, false, true>(J.rec, J.nevt, tile, blk, J.tab, J.t64, J.gslots, J.nslot, J.lin, J.mask, J.ctri, J.cst,
+                                  J.part, J.stride, nullptr);
 }
 
 __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_constant__ PBatch b,
