@@ -180,11 +180,8 @@ int64_t share_chunk(int64_t per_event, int64_t stride) {
   return chunk < stride ? chunk : stride;
 }
 
-cudaError_t fp64_slots(mg_ctx* ctx, const double* mom, const double* rec, int64_t n, bool shared, const MeConst& cst,
+cudaError_t fp64_slots(mg_ctx* ctx, const double* rec, int64_t n, bool shared, const MeConst& cst,
                        double* out, int64_t stride, MeShape shape, cudaStream_t st) {
-  if (ctx->K == 2)
-    return launch_me_gluonhel(2, false, false, mom, const_cast<double*>(rec), n, ctx->d_tab, ctx->d_hslots, 2,
-                              ctx->d_nhslots, ctx->d_mask, ctx->d_ctri, ctx->d_ctri_f, cst, out, stride, st, nullptr, shape);
   if (shared) {
     const cudaError_t e = launch_pass64(ctx->K, rec, n, ctx->d_tab, ctx->d_tab64, cst, ctx->d_lin, ctx->d_share, st);
     if (e != cudaSuccess) return e;
@@ -205,7 +202,6 @@ cudaError_t fp64_amps(mg_ctx* ctx, const double* rec, int64_t n, bool shared, co
 }
 
 cudaError_t fp64_hel_sum(mg_ctx* ctx, int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st) {
-  if (ctx->K == 2) return launch_hel_sum(ctx->d_part, ctx->d_nhslots, nevt, stride, norm, me, st);
   return launch_hel_sum_rows(ctx->K, ctx->d_part, ctx->d_hslots, ctx->d_nhslots, ctx->d_lin, ctx->d_mask, nevt, stride, norm, me, st);
 }
 
@@ -673,12 +669,17 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
     mg_status s = mg_hel_filter(ctx, mom_dev, nevt, stream);
     if (s != MG_OK) return s;
   }
+  const double norm = 1.0 / (256.0 * mg::factorial(ctx->ng));
+  mg::MeConst cst = me_const(ctx);
+  if (precision == MG_FP64 && ctx->K == 2 && ctx->prm.wt == 0.0) {   // one kernel, no scratch
+    ctx->last = st;
+    MG_CUDA(mg::launch_me64_k2(mom_dev, nevt, ctx->d_mask, ctx->d_ctri, cst, norm, me_dev, st));
+    return MG_OK;
+  }
   const int64_t stride = pad32(nevt);
   mg_status s = grow(&ctx->d_part, &ctx->part_cap, stride * ctx->nhel);
   if (s != MG_OK) return s;
   ctx->last = st;
-  mg::MeConst cst = me_const(ctx);
-  const double norm = 1.0 / (256.0 * mg::factorial(ctx->ng));
   // FP64 amplitudes: one of each pair of flipped helicities (hel_weight)
   const bool half = (precision == MG_FP64 || precision == MG_FP64_TCCOLOR) && ctx->prm.wt == 0.0;
   cst.conj = half ? 1 : 0;
@@ -791,9 +792,8 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
       const int64_t nitem = mg::event_record_bytes(ctx->K, false) / 8;
       for (int64_t e0 = 0; e0 < nevt; e0 += chunk) {
         const int64_t n = nevt - e0 < chunk ? nevt - e0 : chunk;
-        MG_CUDA(mg::fp64_slots(ctx, mom_dev + (e0 / mg::kPage) * ctx->npar * 4 * mg::kPage,
-                               ctx->d_prep + (e0 / mg::kPage) * nitem * mg::kPage, n, shared, cst, ctx->d_part + e0, stride,
-                               ctx->shape[precision], st));
+        MG_CUDA(mg::fp64_slots(ctx, ctx->d_prep + (e0 / mg::kPage) * nitem * mg::kPage, n, shared, cst, ctx->d_part + e0,
+                               stride, ctx->shape[precision], st));
       }
     } else if (fused)
       MG_CUDA(mg::launch_me_fused(ctx->K, true, mom_dev, nevt, ctx->d_gslots, ctx->d_ngslots, ctx->d_mask, cst,

@@ -83,16 +83,16 @@ namespace mg {
 int64_t share_doubles(int K);
 int64_t amp_doubles(int K);
 int64_t share_chunk(int64_t per_event, int64_t stride);
-// FP64 colour sums of n events (from a page boundary: momenta mom, FP64 records rec; zero top width) in rows of out, for
-// fp64_hel_sum.  shared: through the items buffer (d_share, share_doubles(K) * pad(n) doubles, 3 to 5 gluons), else every
-// combination on its own.
-cudaError_t fp64_slots(mg_ctx* ctx, const double* mom, const double* rec, int64_t n, bool shared, const MeConst& cst,
+// FP64 colour sums of n events (from a page boundary: FP64 records rec; zero top width; 3 to 5 gluons) in rows of out, for
+// fp64_hel_sum.  shared: through the items buffer (d_share, share_doubles(K) * pad(n) doubles), else every combination on
+// its own.
+cudaError_t fp64_slots(mg_ctx* ctx, const double* rec, int64_t n, bool shared, const MeConst& cst,
                        double* out, int64_t stride, MeShape shape, cudaStream_t st);
 // FP64 amplitudes of n events, 3 to 5 gluons, for launch_helicities; d_share holds amp_doubles(K) and, shared, also
 // share_doubles(K) doubles for each of pad(n) events; the amplitudes' place in it is returned in *amp.
 cudaError_t fp64_amps(mg_ctx* ctx, const double* rec, int64_t n, bool shared, const MeConst& cst, double** amp, MeShape shape,
                       cudaStream_t st);
-// The helicity sum of fp64_slots' colour sums in d_part (per combination for 2 gluons, per helicity for 3 to 5).
+// The helicity sum of fp64_slots' colour sums in d_part.
 cudaError_t fp64_hel_sum(mg_ctx* ctx, int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st);
 // MG_MIXED on the lane-group kernel: colour sums on the tensor cores inside it, per-slot outputs
 bool mixed_in_kernel(const mg_ctx* ctx, mg_precision precision);

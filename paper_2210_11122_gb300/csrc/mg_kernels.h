@@ -91,6 +91,9 @@ cudaError_t launch_me_gluonhel(int K, bool fp32, bool per_hel, const double* mom
 // launch_helicities turns into the helicities' with top helicity -1, rows 2 * gluon helicities + antitop helicity: as
 // FP32 jamps in jout, or (jout null) as colour sums out[row * stride + e] and the weighted jamp squares summed over each
 // antitop helicity's rows, j2[(b * ncol + sigma) * stride + e].
+// (launch_me64_k2: g g -> t tbar, everything from the momenta to me[e] in one kernel)
+cudaError_t launch_me64_k2(const double* mom, int64_t nevt, const uint32_t* mask, const double* ctri, const MeConst& cst,
+                           double norm, double* me, cudaStream_t st);
 cudaError_t launch_pass64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const MeConst& cst,
                           const int* lin, double* share, cudaStream_t st);
 cudaError_t launch_me64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const int* hslots,

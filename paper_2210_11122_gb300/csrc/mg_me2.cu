@@ -25,6 +25,17 @@
 namespace mg {
 namespace v2 {
 
+// The FP64 jamps of 2 gluons with a record, compiled for 4 resident blocks per SM (at most 128 registers;
+// the unbounded compile takes 168, 3 blocks): more warps hide more of the FP64 pipe's dependent-instruction latency
+__global__ void __launch_bounds__(kMeThreads, 4)
+k_me_gluonhel2(const double* __restrict__ rec, int64_t nevt, const Tables* __restrict__ tab,
+               const int* __restrict__ gslots, const int* __restrict__ nslot_dev, const uint32_t* __restrict__ mask,
+               const double* __restrict__ ctri, MeConst cst, double* __restrict__ out, int64_t stride,
+               float2* __restrict__ jout, int tile_ev, int slot_major) {
+  me_thread<2, double, false, true, true, false>(nullptr, rec, nevt, tab, gslots, nslot_dev, mask, ctri, cst, out, stride,
+                                                 jout, tile_ev, slot_major, nullptr, nullptr, 0, nullptr, nullptr);
+}
+
 // One thread per event: the event's record, AoSoA (page of 32 events, value-major within a page).
 template <int K, class T>
 __global__ void __launch_bounds__(128) k_event_prep(const double* __restrict__ mom, int64_t nevt, MeConst cst,
@@ -143,14 +154,11 @@ static cudaError_t launch_v2(const double* mom, void* prep, int64_t nevt, const 
       return launch_me_static(K, sizeof(T) == 4, rec, nevt, gslots, maxslot, nslot, mask, cst, out, stride, jout, shape,
                               skip, st);
     if constexpr (std::is_same<T, double>::value) {
-      // FP64 with a record: 2 gluons here (the compile for more resident blocks), 3 to 5 in launch_me64
+      // FP64 with a record: only the jamps of 2 gluons (colour sums: launch_me64_k2, launch_me64)
       if constexpr (K == 2) {
-        if (jout)
-          { v2::k_me_gluonhel2<true><<<grid, threads, 0, st>>>(rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride,
-                                                              jout, tev, sm); mg::note_launch(); }
-        else
-          { v2::k_me_gluonhel2<false><<<grid, threads, 0, st>>>(rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride,
-                                                               nullptr, tev, sm); mg::note_launch(); }
+        if (!jout) return cudaErrorInvalidValue;
+        { v2::k_me_gluonhel2<<<grid, threads, 0, st>>>(rec, nevt, tab, gslots, nslot, mask, ctri, cst, out, stride, jout, tev,
+                                                      sm); mg::note_launch(); }
         return cudaGetLastError();
       } else {
         return cudaErrorInvalidValue;

@@ -4,6 +4,7 @@
 
 #include "mg_internal.h"
 #include "mg_kernels.h"
+#include "mg_me64_k2.cuh"
 #include "mg_me64l.cuh"
 
 namespace mg {
@@ -167,6 +168,23 @@ static cudaError_t launch_hel_k(double* amp, int64_t nevt, const Tab64* t64, con
 }
 
 }  // namespace m64
+
+namespace m64 {
+__global__ void __launch_bounds__(kMeThreads, 4)
+k_me64_k2(const double* __restrict__ mom, int64_t nevt, const uint32_t* __restrict__ mask, const double* __restrict__ ctri,
+          MeConst cst, double norm, double* __restrict__ me) {
+  __shared__ K2Block s;
+  k2_page(s, mom, nevt, blockIdx.x, mask, ctri, cst, norm, me);
+}
+}  // namespace m64
+
+cudaError_t launch_me64_k2(const double* mom, int64_t nevt, const uint32_t* mask, const double* ctri, const MeConst& cst,
+                           double norm, double* me, cudaStream_t st) {
+  const unsigned pages = static_cast<unsigned>((nevt + kPage - 1) / kPage);
+  if (pages == 0) return cudaSuccess;
+  { m64::k_me64_k2<<<pages, kMeThreads, 0, st>>>(mom, nevt, mask, ctri, cst, norm, me); mg::note_launch(); }
+  return cudaGetLastError();
+}
 
 cudaError_t launch_pass64(int K, const double* rec, int64_t nevt, const Tables* tab, const Tab64* t64, const MeConst& cst,
                           const int* lin, double* share, cudaStream_t st) {

@@ -284,17 +284,5 @@ k_me_gluonhel(const double* __restrict__ mom, const T* __restrict__ rec, int64_t
                                             tile_ev, slot_major, evlist, nlist, rows_out, skip, j2);
 }
 
-// The FP64 slot kernel of 2 gluons with a record, compiled for 4 resident blocks per SM (at most 128 registers;
-// the unbounded compile takes 168, 3 blocks): more warps hide more of the FP64 pipe's dependent-instruction latency
-template <bool JOUT>
-__global__ void __launch_bounds__(kMeThreads, 4)
-k_me_gluonhel2(const double* __restrict__ rec, int64_t nevt, const Tables* __restrict__ tab,
-               const int* __restrict__ gslots, const int* __restrict__ nslot_dev, const uint32_t* __restrict__ mask,
-               const double* __restrict__ ctri, MeConst cst, double* __restrict__ out, int64_t stride,
-               float2* __restrict__ jout, int tile_ev, int slot_major) {
-  me_thread<2, double, false, true, JOUT, false>(nullptr, rec, nevt, tab, gslots, nslot_dev, mask, ctri, cst, out, stride,
-                                                 jout, tile_ev, slot_major, nullptr, nullptr, 0, nullptr, nullptr);
-}
-
 }  // namespace v2
 }  // namespace mg

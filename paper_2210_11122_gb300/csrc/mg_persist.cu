@@ -4,7 +4,7 @@
 // The paper (Sec. 4) finds the GPU throughput still growing up to batches of ~16k events: smaller batches
 // leave the device underfilled.  A batch of many small jobs therefore runs better as one launch whose
 // thread blocks drain a common queue of work tiles than as one launch per job.  Here the queue holds
-// (job, gluon-helicity slot, tile of 32 or 128 events) triples, the jobs ordered by falling cost per tile (more
+// (job, block of helicities, tile of 32 events) triples, the jobs ordered by falling cost per tile (more
 // gluons first, so the longest tiles start first); each 128-thread block takes the next tile from an
 // atomic counter until the queue is empty, and runs the same per-thread FP64 work as the
 // single-job kernels (the
@@ -22,14 +22,13 @@
 #include "mg_ctx.h"
 #include "mg_internal.h"
 #include "mg_kernels.h"
+#include "mg_me64_k2.cuh"
 #include "mg_me64l.cuh"
-#include "mg_me_kernel.cuh"
 
 namespace mg {
 namespace pers {
 
 constexpr int kMaxJobs = 64;   // the job table travels as the kernel's parameter (8 KB)
-constexpr int kTileEv = kMeThreads;   // events per tile of 2 gluons (one thread each); 32 with 3 to 5 (thread64)
 
 struct PJob {
   const double* rec;        // per-event FP64 record
@@ -41,7 +40,8 @@ struct PJob {
   const double* ctri;
   const Tab64* t64;
   const double* share;      // the job's shared items (launch_pass64), or null: every combination on its own
-  double* part;             // part[slot * stride + e]
+  double* part;             // part[row * stride + e]
+  double norm;              // (2 gluons: rec holds the momenta, part the MEs, which are norm * the helicity sum)
   int64_t nevt, stride, tile0;
   int K, ntile_ev;
   MeConst cst;
@@ -66,6 +66,7 @@ __device__ __forceinline__ void run64(const PJob& J, int64_t tile, int blk) {
 __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_constant__ PBatch b,
                                                               unsigned long long* __restrict__ next) {
   __shared__ long long s_tile;
+  __shared__ m64::K2Block s_k2;
   for (;;) {
     if (threadIdx.x == 0) s_tile = static_cast<long long>(atomicAdd(next, 1ull));
     __syncthreads();
@@ -83,13 +84,7 @@ __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_co
     const int slot = static_cast<int>(t / J.ntile_ev);
     const int64_t etile = t - static_cast<int64_t>(slot) * J.ntile_ev;
     switch (J.K) {
-      case 2: {
-        const int64_t e = etile * kTileEv + threadIdx.x;
-        if (e < J.nevt && slot < *J.nslot)
-          v2::me_slot<2, double, false, true, false>(nullptr, J.rec, e, slot, J.gslots[slot], J.tab, J.mask, J.ctri, J.cst,
-                                                     J.part, J.stride, nullptr, 0, nullptr);
-        break;
-      }
+      case 2: m64::k2_page(s_k2, J.rec, J.nevt, etile, J.mask, J.ctri, J.cst, J.norm, J.part); break;
       case 3: run64<3>(J, etile, slot); break;
       case 4: run64<4>(J, etile, slot); break;
       default: run64<5>(J, etile, slot); break;
@@ -154,7 +149,7 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     cst.wt = c->prm.wt;
     cst.conj = 1;   // one of each pair of flipped helicities
     cst.colour_scale = cst.gs * cst.gs / static_cast<double>(c->colour_den);
-    if (mg::launch_event_prep(c->K, false, j.mom_dev, j.nevt, cst, c->d_prep, st) != cudaSuccess) { s = MG_ECUDA; break; }
+    if (c->K >= 3 && mg::launch_event_prep(c->K, false, j.mom_dev, j.nevt, cst, c->d_prep, st) != cudaSuccess) { s = MG_ECUDA; break; }
     // the job's items shared between its gluon-helicity combinations, where its
     // context's FP64 shape asks for them and the whole job's buffer stays within 2 GiB
     const double* share = nullptr;
@@ -167,7 +162,8 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     }
     mg::pers::PJob& p = batch->job[batch->njobs++];
     p.share = share;
-    p.rec = c->d_prep;
+    p.rec = c->K == 2 ? j.mom_dev : c->d_prep;
+    p.norm = 1.0 / (256.0 * mg::factorial(c->ng));
     p.tab = c->d_tab;
     p.t64 = c->d_tab64;
     p.gslots = c->d_hslots;
@@ -175,15 +171,15 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     p.lin = c->d_lin;
     p.mask = c->d_mask;
     p.ctri = c->d_ctri;
-    p.part = c->d_part;
+    p.part = c->K == 2 ? j.me_dev : c->d_part;
     p.nevt = j.nevt;
     p.stride = stride;
     p.K = c->K;
-    const int tev = c->K == 2 ? mg::pers::kTileEv : mg::kPage;
-    p.ntile_ev = static_cast<int>((j.nevt + tev - 1) / tev);
+    p.ntile_ev = static_cast<int>((j.nevt + mg::kPage - 1) / mg::kPage);
     p.tile0 = batch->ntiles;
     p.cst = cst;
-    batch->ntiles += static_cast<int64_t>(p.ntile_ev) << (c->K - 1);   // every possible slot; absent ones exit at once
+    // 3 to 5 gluons: 2^(K-1) blocks of work per event tile (thread64); 2: one
+    batch->ntiles += static_cast<int64_t>(p.ntile_ev) << (c->K == 2 ? 0 : c->K - 1);
   }
   if (s == MG_OK && batch->njobs > 0) {
     // the tile counter of the costliest job's context (a context's work is ordered on one stream at a time)
@@ -204,7 +200,7 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     }
     for (int i = 0; i < njobs && s == MG_OK; ++i) {
       const mg_batch_job& j = jobs[i];
-      if (j.nevt == 0) continue;
+      if (j.nevt == 0 || j.ctx->K == 2) continue;
       const double norm = 1.0 / (256.0 * mg::factorial(j.ctx->ng));
       if (mg::fp64_hel_sum(j.ctx, j.nevt, pad_pg(j.nevt), norm, j.me_dev, st) != cudaSuccess)
         s = MG_ECUDA;
