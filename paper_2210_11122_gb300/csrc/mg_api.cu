@@ -217,7 +217,6 @@ mg_status ctx_reserve(mg_ctx* ctx, int64_t nevt, mg_precision precision) {
   const int64_t stride = pad32(nevt);
   const int64_t wstride = pad32(nevt < ctx->prm.hel_warmup ? nevt : ctx->prm.hel_warmup);
   mg_status s = grow(&ctx->d_part, &ctx->part_cap, (stride > wstride ? stride : wstride) * ctx->nhel);
-  if (s == MG_OK) s = grow(&ctx->d_tot, &ctx->tot_cap, wstride);
   const bool fp32 = precision == MG_FP32_AMP || precision == MG_MIXED;
   const bool tc = (precision == MG_FP64_TCCOLOR || precision == MG_MIXED) && !mixed_in_kernel(ctx, precision);
   int64_t chunk = stride;
@@ -399,7 +398,7 @@ void mg_destroy(mg_ctx* ctx) {
   mg::dev_free(ctx->d_nallg);
   mg::dev_free(ctx->d_nbad);
   mg::dev_free(ctx->d_part);
-  mg::dev_free(ctx->d_tot);
+  mg::dev_free(ctx->d_facc);
   mg::dev_free(ctx->d_prep);
   mg::dev_free(ctx->d_repair);
   mg::dev_free(ctx->d_nrepair);
@@ -475,6 +474,7 @@ mg_status mg_create(mg_process proc, const mg_params* params, mg_ctx** out) {
     for (int h = 0; h < c->nhel; ++h) all[h] = h;
     if (mg::dev_alloc(&c->d_mask, 4 * sizeof(uint32_t)) != cudaSuccess || mg::dev_alloc(&c->d_good, 128 * sizeof(int)) != cudaSuccess ||
         mg::dev_alloc(&c->d_maxr, 128 * sizeof(double)) != cudaSuccess ||
+        mg::dev_alloc(&c->d_facc, 129 * sizeof(unsigned long long)) != cudaSuccess ||
         mg::dev_alloc(&c->d_ngood, sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_allhel, c->nhel * sizeof(int)) != cudaSuccess ||
         mg::dev_alloc(&c->d_nhel, sizeof(int)) != cudaSuccess || mg::dev_alloc(&c->d_nbad, sizeof(unsigned long long)) != cudaSuccess) {
       st = MG_ENOMEM;
@@ -521,6 +521,7 @@ mg_status mg_create(mg_process proc, const mg_params* params, mg_ctx** out) {
         cudaMemcpy(c->d_nhel, &c->nhel, sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(c->d_nbad, 0, sizeof(unsigned long long)) != cudaSuccess ||
         cudaMemset(c->d_mask, 0, 4 * sizeof(uint32_t)) != cudaSuccess ||
+        cudaMemset(c->d_facc, 0, 129 * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMemset(c->d_ngood, 0, sizeof(int)) != cudaSuccess) {
       st = MG_ECUDA;
       break;
@@ -609,8 +610,6 @@ mg_status mg_hel_filter(mg_ctx* ctx, const double* mom_dev, int64_t nevt, void* 
   const int64_t stride = pad32(w);
   mg_status s = grow(&ctx->d_part, &ctx->part_cap, stride * ctx->nhel);
   if (s != MG_OK) return s;
-  s = grow(&ctx->d_tot, &ctx->tot_cap, stride);
-  if (s != MG_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ctx->last = st;
   const mg::MeConst cst = me_const(ctx);
@@ -624,11 +623,9 @@ mg_status mg_hel_filter(mg_ctx* ctx, const double* mom_dev, int64_t nevt, void* 
     MG_CUDA(mg::launch_me_helicity(ctx->K, false, mom_dev, w, ctx->d_tab, ctx->d_allhel, ctx->nhel, ctx->d_nhel,
                                    ctx->d_ctri, cst, ctx->d_part, stride, st));
   }
-  MG_CUDA(mg::launch_hel_sum(ctx->d_part, ctx->d_nhel, w, stride, 1.0, ctx->d_tot, st));
-  MG_CUDA(mg::launch_hel_mask(ctx->d_part, ctx->d_tot, ctx->nhel, w, stride, ctx->prm.hel_tau, ctx->d_maxr,
-                              ctx->d_mask, ctx->d_good, ctx->d_ngood, st));
-  MG_CUDA(mg::launch_gluon_slots(ctx->d_mask, ctx->K, ctx->d_gslots, ctx->d_ngslots, ctx->d_nrows, ctx->d_hslots,
-                                 ctx->d_nhslots, ctx->d_nhrows, ctx->d_lin, st));
+  MG_CUDA(mg::launch_hel_filter(ctx->K, ctx->d_part, w, stride, ctx->prm.hel_tau, ctx->d_facc, ctx->d_maxr, ctx->d_mask,
+                                ctx->d_good, ctx->d_ngood, ctx->d_gslots, ctx->d_ngslots, ctx->d_nrows, ctx->d_hslots,
+                                ctx->d_nhslots, ctx->d_nhrows, ctx->d_lin, st));
   ctx->mask_ready = true;
   return MG_OK;
 }

@@ -42,7 +42,7 @@ struct mg_ctx {
   unsigned long long* d_nbad = nullptr;
   double* d_part = nullptr;   // per-(helicity, event) colour sums
   int64_t part_cap = 0;
-  double* d_tot = nullptr;    // per-event helicity sums of the filter
+  unsigned long long* d_facc = nullptr;   // helicity filter: maxima in progress and block counter (zero between calls)
   double* d_prep = nullptr;   // per-event records (momenta sums, propagators, wavefunctions)
   int* d_repair = nullptr;    // FP32 modes: events recomputed in FP64, and their count
   int* d_nrepair = nullptr;
@@ -59,7 +59,6 @@ struct mg_ctx {
   cudaStream_t side = nullptr;         // FP32 modes: the FP64 recomputation runs here, beside the FP32 launches
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int64_t prep_cap = 0;       // in doubles
-  int64_t tot_cap = 0;
   double* d_mom_stage = nullptr;
   double* d_me_stage = nullptr;
   int64_t stage_cap = 0;

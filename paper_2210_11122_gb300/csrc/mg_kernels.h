@@ -14,7 +14,7 @@ struct MeConst {
   double mt, wt;        // top mass and width
   double colour_scale;  // g_s^2 / colour-matrix denominator
   double fp32_tau = 3e-4;  // FP32 modes: events with an internal invariant below fp32_tau * s are redone in FP64
-  // 1: the slots are one of each pair of flipped gluon-helicity combinations (launch_gluon_slots' hslots) and every
+  // 1: the slots are one of each pair of flipped gluon-helicity combinations (launch_hel_filter's hslots) and every
   // helicity h stands for itself and for ~h, |M_h|^2 = |M_~h|^2 (hel_weight); 0: every combination has its own slot
   int conj = 0;
 };
@@ -152,11 +152,13 @@ void colour_tc_pack(int ncol, const int64_t* num, uint16_t* out_halves);
 cudaError_t launch_colour_tc(int ncol, const float2* jamps, int64_t nevt, int rows_alloc, const int* nrows,
                              const void* cmat, double scale, double* out, int64_t stride, cudaStream_t st,
                              const uint8_t* skip = nullptr);
-// gslots: the gluon-helicity combinations with a good helicity (*n of them, *nrows = 4 *n); hslots: those with
-// gluon K-1 of helicity -1 for which the combination or its flip has a good helicity (*nh, *nhrows = 4 *nh); *lin = 1
-// if every helicity is good, else 0.
-cudaError_t launch_gluon_slots(const uint32_t* mask, int K, int* gslots, int* n, int* nrows, int* hslots, int* nh,
-                               int* nhrows, int* lin, cudaStream_t st);
+// The helicity filter from the per-helicity sums part[h * stride + e] of nevt events: maxr, mask, good list; gslots: the
+// gluon-helicity combinations with a good helicity (*n of them, *nrows = 4 *n); hslots: those with gluon K-1 of helicity -1
+// for which the combination or its flip has a good helicity (*nh, *nhrows = 4 *nh); *lin = 1 if every helicity is good,
+// else 0.  acc: 129 words, zero before the launch and after it.
+cudaError_t launch_hel_filter(int K, const double* part, int64_t nevt, int64_t stride, double tau, unsigned long long* acc,
+                              double* maxr, uint32_t* mask, int* good, int* ngood, int* gslots, int* n, int* nrows,
+                              int* hslots, int* nh, int* nhrows, int* lin, cudaStream_t st);
 // me[e] = norm * sum over launch_helicities' rows of hel_weight * part[row * stride + e]
 cudaError_t launch_hel_sum_top(int K, const double* part, const uint32_t* mask, int64_t nevt, int64_t stride, double norm,
                                double* me, cudaStream_t st);
@@ -166,7 +168,5 @@ cudaError_t launch_hel_sum_rows(int K, const double* part, const int* hslots, co
                                 int64_t nevt, int64_t stride, double norm, double* me, cudaStream_t st);
 cudaError_t launch_hel_sum(const double* part, const int* nslot, int64_t nevt, int64_t stride, double norm,
                            double* me, cudaStream_t st);
-cudaError_t launch_hel_mask(const double* part, const double* tot, int nhel, int64_t nevt, int64_t stride, double tau,
-                            double* maxr, uint32_t* mask, int* good, int* ngood, cudaStream_t st);
 
 }  // namespace mg

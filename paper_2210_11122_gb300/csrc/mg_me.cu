@@ -431,40 +431,97 @@ __global__ void k_hel_sum_top(int K, const double* __restrict__ part, const uint
   me[e] = s * norm;
 }
 
-// helicity filter, step 1: maxr[h] = max over the warm-up events of part[h][e] / tot[e]
-// (one block per helicity, fixed-shape tree reduction: order-independent maximum).
-__global__ void k_hel_ratio_max(const double* __restrict__ part, const double* __restrict__ tot, int64_t nevt,
-                                int64_t stride, double* __restrict__ maxr) {
-  __shared__ double red[256];
-  const int h = blockIdx.x;
-  double mx = 0.0;
-  for (int64_t e = threadIdx.x; e < nevt; e += blockDim.x) {
-    const double r = part[h * stride + e] / tot[e];
-    mx = r > mx ? r : mx;
-  }
-  red[threadIdx.x] = mx;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) red[threadIdx.x] = red[threadIdx.x + w] > red[threadIdx.x] ? red[threadIdx.x + w] : red[threadIdx.x];
+// Helicity filter: maxr[h] = max over the warm-up events of part[h][e] / sum_h' part[h'][e], good(h) <=> maxr[h] > tau;
+// the mask words, the ascending good list, and the gluon-helicity slot lists (launch_hel_filter).  A block of 8 warps takes
+// pages of 32 events and 16 helicities (2 per warp): the event sums in shared memory (an eighth per warp), the ratios'
+// maxima by atomics on the bit patterns of non-negative doubles (order-independent); the last block to finish makes the
+// lists.  One launch where there were four (hel_sum, ratio maxima, mask, slots: 23 us of gg -> t tbar's step with the gaps
+// between them).  acc: 128 maxima and a block counter, zero before and after.
+constexpr int kFilterHel = 16;
+__global__ void __launch_bounds__(256)
+k_hel_filter(const double* __restrict__ part, int K, int64_t nevt, int64_t stride, double tau,
+             unsigned long long* __restrict__ acc, double* __restrict__ maxr, uint32_t* __restrict__ mask,
+             int* __restrict__ good, int* __restrict__ ngood, int* __restrict__ gslots, int* __restrict__ n,
+             int* __restrict__ nrows, int* __restrict__ hslots, int* __restrict__ nh, int* __restrict__ nhrows,
+             int* __restrict__ lin) {
+  __shared__ double sum[8][kPage];
+  __shared__ bool last;
+  const int npar = K + 2, nhel = 1 << npar, lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+  const int h0 = blockIdx.y * kFilterHel + 2 * warp;   // (nhel is a multiple of 16)
+  double mx[2] = {0.0, 0.0};
+  for (int64_t page = blockIdx.x; page * kPage < nevt; page += gridDim.x) {
+    const int64_t e = page * kPage + lane;
+    double s = 0.0;
+    if (e < nevt)
+      for (int h = warp; h < nhel; h += 8) s += part[h * stride + e];
+    sum[warp][lane] = s;
+    __syncthreads();
+    if (e < nevt) {
+      double tot = 0.0;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) tot += sum[w][lane];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const double r = part[(h0 + k) * stride + e] / tot;
+        mx[k] = r > mx[k] ? r : mx[k];
+      }
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0) maxr[h] = red[0];
-}
-
-// step 2: good(h) <=> maxr[h] > tau; mask words, ascending good list and its length.
-__global__ void k_hel_mask(const double* __restrict__ maxr, int nhel, double tau, uint32_t* __restrict__ mask,
-                           int* __restrict__ good, int* __restrict__ ngood) {
-  const int h = threadIdx.x;
-  const bool g = h < nhel && maxr[h] > tau;
-  const unsigned bits = __ballot_sync(0xffffffffu, g);
-  if ((h & 31) == 0 && h < ((nhel + 31) & ~31)) mask[h >> 5] = bits;
-  __syncthreads();
-  if (h == 0) {
-    int n = 0;
-    for (int k = 0; k < nhel; ++k)
-      if ((mask[k >> 5] >> (k & 31)) & 1u) good[n++] = k;
-    *ngood = n;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double r = __shfl_xor_sync(0xffffffffu, mx[k], o);
+      mx[k] = r > mx[k] ? r : mx[k];
+    }
+    if (lane == 0) atomicMax(acc + h0 + k, static_cast<unsigned long long>(__double_as_longlong(mx[k])));
   }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(acc + 128, 1ull) == static_cast<unsigned long long>(gridDim.x) * gridDim.y - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x < 128) {   // (nhel <= 128)
+    const int h = threadIdx.x;
+    double m = 0.0;
+    if (h < nhel) {
+      m = __longlong_as_double(static_cast<long long>(atomicExch(acc + h, 0ull)));
+      maxr[h] = m;
+    }
+    const unsigned bits = __ballot_sync(0xffffffffu, h < nhel && m > tau);
+    if (lane == 0 && h < ((nhel + 31) & ~31)) mask[h >> 5] = bits;
+  }
+  __syncthreads();   // (the block's own mask words, through global memory)
+  if (threadIdx.x != 0) return;
+  acc[128] = 0;
+  int c = 0;
+  bool all = true;
+  for (int h = 0; h < nhel; ++h) {
+    if ((mask[h >> 5] >> (h & 31)) & 1u) good[c++] = h;
+    else all = false;
+  }
+  *ngood = c;
+  *lin = all ? 1 : 0;
+  int cnt = 0, hcnt = 0;
+  for (int gc = 0; gc < (1 << K); ++gc) {
+    int hb = 0;
+    for (int g = 0; g < K; ++g)
+      if ((gc >> g) & 1) hb |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
+    bool any = false, hany = false;
+    for (int t = 0; t < 4; ++t) {
+      const int h = hb | ((t & 1) << (npar - 3)) | ((t >> 1) << (npar - 4));
+      any = any || hel_weight(mask, h, npar, 0);
+      hany = hany || hel_weight(mask, h, npar, 1);
+    }
+    if (any) gslots[cnt++] = gc;
+    if (hany && gc < (1 << (K - 1))) hslots[hcnt++] = gc;
+  }
+  *n = cnt;
+  *nrows = 4 * cnt;
+  *nh = hcnt;
+  *nhrows = 4 * hcnt;
 }
 
 template <int K, class T>
@@ -521,10 +578,13 @@ cudaError_t launch_hel_sum_top(int K, const double* part, const uint32_t* mask, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_hel_mask(const double* part, const double* tot, int nhel, int64_t nevt, int64_t stride, double tau,
-                            double* maxr, uint32_t* mask, int* good, int* ngood, cudaStream_t st) {
-  { k_hel_ratio_max<<<nhel, 256, 0, st>>>(part, tot, nevt, stride, maxr); mg::note_launch(); }
-  { k_hel_mask<<<1, 128, 0, st>>>(maxr, nhel, tau, mask, good, ngood); mg::note_launch(); }
+cudaError_t launch_hel_filter(int K, const double* part, int64_t nevt, int64_t stride, double tau, unsigned long long* acc,
+                              double* maxr, uint32_t* mask, int* good, int* ngood, int* gslots, int* n, int* nrows,
+                              int* hslots, int* nh, int* nhrows, int* lin, cudaStream_t st) {
+  const int64_t pages = (nevt + kPage - 1) / kPage;
+  const dim3 grid(static_cast<unsigned>(pages < 256 ? pages : 256), (4 << K) / kFilterHel);
+  { k_hel_filter<<<grid, 256, 0, st>>>(part, K, nevt, stride, tau, acc, maxr, mask, good, ngood, gslots, n, nrows, hslots, nh,
+                                       nhrows, lin); mg::note_launch(); }
   return cudaGetLastError();
 }
 

@@ -78,43 +78,7 @@ __global__ void __launch_bounds__(128) k_event_flags(const double* __restrict__ 
   flag[e] = redo ? 1 : 0;
 }
 
-// Gluon-helicity combinations with at least one good helicity (fixed ascending order), and the half list of
-// one of each pair of flipped combinations (launch_gluon_slots).
-__global__ void k_gluon_slots(const uint32_t* __restrict__ mask, int K, int* __restrict__ gslots, int* __restrict__ n,
-                              int* __restrict__ nrows, int* __restrict__ hslots, int* __restrict__ nh,
-                              int* __restrict__ nhrows, int* __restrict__ lin) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const int npar = K + 2;
-  int cnt = 0, hcnt = 0;
-  bool all = true;
-  for (int h = 0; h < (1 << npar); ++h) all = all && ((mask[h >> 5] >> (h & 31)) & 1u);
-  *lin = all ? 1 : 0;
-  for (int gc = 0; gc < (1 << K); ++gc) {
-    int hb = 0;
-    for (int g = 0; g < K; ++g)
-      if ((gc >> g) & 1) hb |= 1 << (npar - 1 - (g < 2 ? g : g + 2));
-    bool any = false, hany = false;
-    for (int t = 0; t < 4; ++t) {
-      const int h = hb | ((t & 1) << (npar - 3)) | ((t >> 1) << (npar - 4));
-      any = any || hel_weight(mask, h, npar, 0);
-      hany = hany || hel_weight(mask, h, npar, 1);
-    }
-    if (any) gslots[cnt++] = gc;
-    if (hany && gc < (1 << (K - 1))) hslots[hcnt++] = gc;
-  }
-  *nh = hcnt;
-  *nhrows = 4 * hcnt;
-  *n = cnt;
-  *nrows = 4 * cnt;
-}
-
 }  // namespace v2
-
-cudaError_t launch_gluon_slots(const uint32_t* mask, int K, int* gslots, int* n, int* nrows, int* hslots, int* nh,
-                               int* nhrows, int* lin, cudaStream_t st) {
-  { v2::k_gluon_slots<<<1, 32, 0, st>>>(mask, K, gslots, n, nrows, hslots, nh, nhrows, lin); mg::note_launch(); }
-  return cudaGetLastError();
-}
 
 static int sm_count() {
   int dev = 0, n = 0;
