@@ -78,8 +78,9 @@ void build_tables(int K, Tables& t);
 // pext_bits order; entries are 8 doubles (4 complex) times what the comment says.
 // ----------------------------------------------------------------------------------------
 struct Tab64 {
-  enum Type { kJ1, kJq0, kChi, kPsi, kSeq, kZ, kY, kFull, kQQ };
-  static constexpr int kMaxTask = 2500, kMaxTaskL = 4200, kMaxLTask = 320, kMaxPass = 6;
+  enum Type { kJ1, kJq0, kChi, kPsi, kSeq, kZ, kY, kFull, kU, kDot, kQQ };
+  static constexpr int kMaxTask = 2500, kMaxTaskL = 5800, kMaxLTask = 480, kMaxPass = 6;
+  static constexpr int kMaxSeq3 = 45;      // canonical sequences of at most 3 gluons
   struct Off {
     int J[kMaxSeq];                        // current of a canonical sequence (1)
     int X[kMaxSeq];                        // (gamma.J) v, three or more gluons (antitop helicity: 2); -1: none
@@ -103,6 +104,9 @@ struct Tab64 {
     int z[kMaxGluons * kMaxGluons];        // (2)
     int y[kMaxSeq][kMaxGluons];            // 5 gluons (2)
     int full[kMaxNcol / 2];                // 2 complex numbers (4 doubles)
+    int u[kMaxSeq];                        // one and two gluons: ubar gamma^mu v joined to J by a three-gluon vertex (2)
+    int d[kMaxSeq];                        // up to K-2 gluons: ubar gamma^mu v . J, 2 complex numbers (4 doubles)
+    int dot[kMaxSeq3][kMaxSeq3];           // g J . J' of disjoint sequences of together at most K-1 gluons (1 double)
     int qq[kMaxGluons * kMaxGluons];       // 4 and 5 gluons (2)
   };
   int K, stride;                           // doubles per event of the shared buffer (either basis)

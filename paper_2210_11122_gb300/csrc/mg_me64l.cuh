@@ -3,7 +3,7 @@
 // The amplitude is linear in each gluon's polarisation vector, and the two helicity vectors are a unitary combination of
 // the two real transverse vectors e_theta, e_phi: summed over both, |M|^2 is the same.  With real polarisations every
 // gluon current is real (the vertices and propagators are), which makes the three-gluon vertex 30 FP64 instructions
-// instead of 80, the four-gluon vertex 27 instead of 102, and a quark current times a gluon current 8 instead of 16;
+// instead of 80, the four-gluon vertex 13 (products of currents tabulated) instead of 102, and a quark current times a gluon current 8 instead of 16;
 // and flipping both top helicities conjugates the amplitude, so top helicity -1 with both antitop helicities is enough.
 // So where every helicity is good (always, from 3 gluons on, at the default threshold) and only the sum is asked for,
 // mg_me64.cuh's scheme runs in this basis: 2^K polarisation combinations x 2 antitop helicities, as many as there are
@@ -15,7 +15,8 @@
 // 2^K undoes; the other factor 2 is the flip.
 //
 // Measured against the helicity basis: gg->ttg 9.47 vs 12.05 ms per 524,288 events, gg->ttgg 1.87 vs 2.64 ms per 10,007,
-// gg->ttggg 21.5 vs 31.7 ms per 8,192.
+// gg->ttggg 21.5 vs 31.7 ms per 8,192; with the all-gluon currents formed only in their contraction with the quark
+// current (ViewL::full) and the products of currents tabulated for the four-gluon vertices 8.98, 1.63 and 17.8 ms.
 #pragma once
 
 #include "mg_me64.cuh"
@@ -25,9 +26,9 @@ namespace m64 {
 
 // doubles of one combination's own items (LOCAL)
 template <int K> struct LocL;
-template <> struct LocL<3> { static constexpr int n = 268; };
-template <> struct LocL<4> { static constexpr int n = 856; };
-template <> struct LocL<5> { static constexpr int n = 3036; };
+template <> struct LocL<3> { static constexpr int n = 331; };
+template <> struct LocL<4> { static constexpr int n = 1100; };
+template <> struct LocL<5> { static constexpr int n = 3600; };
 
 __device__ __forceinline__ double rdot(const double* a, const double* b) {
   return fma(-a[3], b[3], fma(-a[2], b[2], fma(-a[1], b[1], a[0] * b[0])));
@@ -42,7 +43,7 @@ __device__ __forceinline__ cx<double> qdot(const cx<double>* q, const double* j)
   return r;
 }
 
-// v3_acc and v4_acc on real currents
+// v3_acc on real currents
 __device__ __forceinline__ void v3r_acc(double* acc, const double* JL, const double* JR, const double* PL, const double* PR,
                                         bool neg) {
   double jj = rdot(JL, JR);
@@ -50,12 +51,6 @@ __device__ __forceinline__ void v3r_acc(double* acc, const double* JL, const dou
   const double two = neg ? -2.0 : 2.0, cl = two * rdot(JL, PR), cr = two * rdot(JR, PL);
 #pragma unroll
   for (int m = 0; m < 4; ++m) acc[m] = fma(-cr, JL[m], fma(cl, JR[m], fma(PL[m] - PR[m], jj, acc[m])));
-}
-__device__ __forceinline__ void v4r_acc(double* acc, const double* JA, const double* JB, const double* JC, double g, bool neg) {
-  const double s = neg ? -g : g;
-  const double ab = s * rdot(JA, JB), bc = s * rdot(JB, JC), ac = (2.0 * s) * rdot(JA, JC);
-#pragma unroll
-  for (int m = 0; m < 4; ++m) acc[m] = fma(-ac, JB[m], fma(bc, JA[m], fma(ab, JC[m], acc[m])));
 }
 
 // gamma.J of a real current: a = J0 + J3, b = J0 - J3, and J1 -+ i J2
@@ -160,6 +155,21 @@ struct ViewL {
   }
   __device__ __forceinline__ int offFull(int f) const { return o->full[f] + h((1 << K) - 1) * 4; }
 
+  __device__ __forceinline__ double dot(int r, int s) const {   // g J_r . J_s
+    return buf[static_cast<int64_t>(o->dot[r][s] + h(tab->seq_mask[r] | tab->seq_mask[s])) * ST];
+  }
+  __device__ __forceinline__ cx<double> d(int s, int b) const {
+    const double* p = buf + static_cast<int64_t>(o->d[s] + h(tab->seq_mask[s]) * 4 + 2 * b) * ST;
+    return {p[0], p[ST]};
+  }
+  __device__ __forceinline__ void st_d(int s, int b, cx<double> x) const {
+    double* p = buf + static_cast<int64_t>(o->d[s] + h(tab->seq_mask[s]) * 4 + 2 * b) * ST;
+    p[0] = x.r;
+    p[ST] = x.i;
+  }
+  __device__ __forceinline__ int offU(int s, int b) const { return o->u[s] + (h(tab->seq_mask[s]) * 2 + b) * 8; }
+
+  // current of a canonical split list; the four-gluon vertices from the tabulated products: 13 instructions each
   __device__ __forceinline__ void vertices(double* acc, int n3, const int16_t (*v3)[2], int n4, const int16_t (*v4)[3]) const {
     for (int k = 0; k < n3; ++k) {
       const int16_t rl = v3[k][0], rr = v3[k][1];
@@ -171,12 +181,58 @@ struct ViewL {
       v3r_acc(acc, JL, JR, PL, PR, v2::rneg(rl) != v2::rneg(rr));
     }
     for (int k = 0; k < n4; ++k) {
-      const int16_t ra = v4[k][0], rb = v4[k][1], rc = v4[k][2];
+      const int a = v2::rslot(v4[k][0]), b = v2::rslot(v4[k][1]), c = v2::rslot(v4[k][2]);
+      const bool neg = v2::rneg(v4[k][0]) ^ v2::rneg(v4[k][1]) ^ v2::rneg(v4[k][2]);
       double JA[4], JB[4], JC[4];
-      J(v2::rslot(ra), JA);
-      J(v2::rslot(rb), JB);
-      J(v2::rslot(rc), JC);
-      v4r_acc(acc, JA, JB, JC, gs, v2::rneg(ra) ^ v2::rneg(rb) ^ v2::rneg(rc));
+      J(a, JA);
+      J(b, JB);
+      J(c, JC);
+      double ab = dot(a, b), bc = dot(b, c), ac = -2.0 * dot(a, c);
+      if (neg) { ab = -ab; bc = -bc; ac = -ac; }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) acc[m] = fma(ac, JB[m], fma(bc, JA[m], fma(ab, JC[m], acc[m])));
+    }
+  }
+  // all gluons on one current contracted with ubar gamma^mu v, without the propagator.  A three-gluon vertex of a
+  // split (L, R) is the shorter side's U times the longer side's current, antisymmetric in L and R; a four-gluon vertex
+  // combines tabulated products: 16 and 13 instructions for both antitop helicities, where the vector form takes 30
+  // and 13 and the contraction 16 more per current.
+  __device__ __forceinline__ void full(int f, cx<double>* x) const {
+    x[0] = x[1] = {0.0, 0.0};
+    for (int k = 0; k < tab->full_nv3[f]; ++k) {
+      const int16_t rl = tab->full_v3[f][k][0], rr = tab->full_v3[f][k][1];
+      const int l = v2::rslot(rl), r = v2::rslot(rr);
+      const bool left = tab->seq_len[l] <= tab->seq_len[r];
+      const bool neg = (v2::rneg(rl) != v2::rneg(rr)) != !left;
+      double Jl[4];
+      J(left ? r : l, Jl);
+      if (neg)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) Jl[m] = -Jl[m];
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        cx<double> U[4];
+        ld(offU(left ? l : r, b), U);
+        x[b].r = fma(U[0].r, Jl[0], x[b].r);
+        x[b].i = fma(U[0].i, Jl[0], x[b].i);
+#pragma unroll
+        for (int m = 1; m < 4; ++m) {
+          x[b].r = fma(-U[m].r, Jl[m], x[b].r);
+          x[b].i = fma(-U[m].i, Jl[m], x[b].i);
+        }
+      }
+    }
+    for (int k = 0; k < tab->full_nv4[f]; ++k) {
+      const int16_t* v = tab->full_v4[f][k];
+      const int a = v2::rslot(v[0]), b = v2::rslot(v[1]), c = v2::rslot(v[2]);
+      double ab = dot(a, b), bc = dot(b, c), ac = -2.0 * dot(a, c);
+      if (v2::rneg(v[0]) ^ v2::rneg(v[1]) ^ v2::rneg(v[2])) { ab = -ab; bc = -bc; ac = -ac; }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        v2::cmacr(x[q], ab, d(c, q));
+        v2::cmacr(x[q], bc, d(a, q));
+        v2::cmacr(x[q], ac, d(b, q));
+      }
     }
   }
 };
@@ -267,6 +323,13 @@ __device__ __forceinline__ void run_task_l(const ViewL<K, LOCAL>& V, uint32_t ta
 #pragma unroll
       for (int m = 0; m < 4; ++m) acc[m] *= f;
       V.stJ(a_, acc);
+      if (K == 5 && V.tab->seq_len[a_] == 3)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          cx<double> Jq[4];
+          V.ld(V.o->q0 + b * 8, Jq);
+          V.st_d(a_, b, qdot(Jq, acc));
+        }
       break;
     }
     case Tab64::kZ: {   // Z(g, h) and Z(h, g) of a canonical pair: J(h, g) = -J(g, h)
@@ -293,20 +356,52 @@ __device__ __forceinline__ void run_task_l(const ViewL<K, LOCAL>& V, uint32_t ta
       break;
     }
     case Tab64::kFull: {
-      double acc[4] = {};
-      V.vertices(acc, V.tab->full_nv3[a_], V.tab->full_v3[a_], V.tab->full_nv4[a_], V.tab->full_v4[a_]);
+      cx<double> x[2];
+      V.full(a_, x);
       const double f = V.rec(L::GP + (1 << K) - 1);
-#pragma unroll
-      for (int m = 0; m < 4; ++m) acc[m] *= f;
       double* p = V.buf + static_cast<int64_t>(V.offFull(a_)) * ViewL<K, LOCAL>::ST;
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
-        cx<double> Jq[4];
-        V.ld(V.o->q0 + b * 8, Jq);
-        const cx<double> x = qdot(Jq, acc);
-        p[(2 * b) * ViewL<K, LOCAL>::ST] = x.r;
-        p[(2 * b + 1) * ViewL<K, LOCAL>::ST] = x.i;
+        p[(2 * b) * ViewL<K, LOCAL>::ST] = f * x[b].r;
+        p[(2 * b + 1) * ViewL<K, LOCAL>::ST] = f * x[b].i;
       }
+      break;
+    }
+    case Tab64::kU: {
+      // D = Jq.J and U = 2 [(Jq.P) J + (J.P') Jq - (Jq.J) P] for Jq = ubar gamma^mu v, P the current's momentum and P'
+      // the other gluons': U.R = Jq . V3(J, R) for a conserved current R of the other gluons (P'.R = 0), Jq being
+      // conserved too (Jq.(P + P') = 0)
+      double J[4], P[4], PR[4];
+      V.J(a_, J);
+      V.mom(a_, P);
+      const int rest = ((1 << K) - 1) ^ V.tab->seq_mask[a_];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) PR[m] = V.rec(L::PT + 4 * rest + m);
+      const double jp = 2.0 * rdot(J, PR);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) P[m] *= 2.0;
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        cx<double> Jq[4], U[4];
+        V.ld(V.o->q0 + b * 8, Jq);
+        const cx<double> qp = qdot(Jq, P), qj = qdot(Jq, J);
+        V.st_d(a_, b, qj);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          U[m] = v2::cscale(J[m], qp);
+          v2::cmacr(U[m], jp, Jq[m]);
+          v2::cmacr(U[m], -P[m], qj);
+        }
+        V.st(V.offU(a_, b), U);
+      }
+      break;
+    }
+    case Tab64::kDot: {   // g J.J' of two sequences
+      double A[4], B[4];
+      V.J(a_, A);
+      V.J(b_, B);
+      V.buf[static_cast<int64_t>(V.o->dot[a_][b_] + V.h(V.tab->seq_mask[a_] | V.tab->seq_mask[b_])) * ViewL<K, LOCAL>::ST] =
+          V.gs * rdot(A, B);
       break;
     }
     case Tab64::kY: {   // (gamma.J_s) chi(g), 5 gluons

@@ -6,6 +6,7 @@
 #include <map>
 #include <mutex>
 #include <numeric>
+#include <utility>
 #include <vector>
 
 #include "mg_internal.h"
@@ -49,6 +50,8 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
     (own ? o.nloc : o.stride) = at;
   }
   // ---- linear polarisations ----
+  auto has_u = [&](int s) { return t.seq_len[s] <= (K == 3 ? 1 : 2); };
+  auto has_dot = [&](int r, int s) { return !(t.seq_mask[r] & t.seq_mask[s]) && t.seq_len[r] + t.seq_len[s] <= K - 1; };
   for (int own = 0; own < 2; ++own) {
     Tab64::OffL& f = own ? o.locl : o.shl;
     int at = 0;
@@ -77,6 +80,12 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
         if (K >= 4) f.qq[g * kMaxGluons + h] = take(1 << g | 1 << h, 16);
       }
     for (int i = 0; i < t.nfull; ++i) f.full[i] = take((1 << K) - 1, 4);
+    for (int s = 0; s < t.nseq; ++s) {
+      if (has_u(s)) f.u[s] = take(t.seq_mask[s], 16);
+      if (t.seq_len[s] <= K - 2) f.d[s] = take(t.seq_mask[s], 4);
+      for (int r = 0; r < s; ++r)
+        if (has_dot(r, s)) f.dot[r][s] = f.dot[s][r] = take(t.seq_mask[r] | t.seq_mask[s], 1);
+    }
     if (K == 5)
       for (int s = 0; s < t.nseq; ++s)
         for (int g = 0; g < K; ++g)
@@ -116,8 +125,21 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
   psis(1);
   if (K == 3) next_pass();   // (three gluons: four short passes instead of two)
   for (int g = 0; g < K; ++g) tasks(Tab64::kChi, g, 0, 1 << g);
+  // (linear polarisations) quark current and gluon, products of two currents of la and lb gluons
+  auto us = [&](int len) {
+    for (int s = 0; s < t.nseq; ++s)
+      if (t.seq_len[s] == len && has_u(s)) tasksl(Tab64::kU, s, 0, t.seq_mask[s]);
+  };
+  auto dots = [&](int la, int lb) {
+    for (int s = 0; s < t.nseq; ++s)
+      for (int r = 0; r < s; ++r)
+        if (t.seq_len[r] == la && t.seq_len[s] == lb && has_dot(r, s)) tasksl(Tab64::kDot, r, s, t.seq_mask[r] | t.seq_mask[s]);
+  };
+  if (K == 3) us(1);
   next_pass();
   seqs(Tab64::kSeq, 2);
+  dots(1, 1);
+  if (K >= 4) us(1);
   if (K >= 4)
     for (int g = 0; g < K; ++g)
       for (int h = 0; h < K; ++h)
@@ -132,6 +154,9 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
       for (int g = 0; g < K; ++g)
         if (o.sh.y[s][g] >= 0) tasks(Tab64::kY, s, g, t.seq_mask[s] | 1 << g);
     psis(2);
+    us(2);
+    dots(1, 2);
+    if (K == 5) dots(2, 2);
   }
   seqs(Tab64::kZ, 2);
   auto fulls = [&] {
@@ -145,6 +170,7 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
     if (K == 5) {
       seqs(Tab64::kSeq, 4);
       psis(3);
+      dots(1, 3);
       next_pass();
     }
     fulls();
@@ -214,7 +240,8 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
     return rank.at(q);
   };
   std::vector<bool> seen(t.ncol, false);
-  struct Vec { int at; std::vector<int> sign; int norm; };   // a basis combination: jamp index it replaces, signs
+  // a basis combination: the jamp index it replaces, its jamps with their signs
+  struct Vec { int at; std::vector<std::pair<int, int>> sign; int norm; };
   std::vector<Vec> blocks[8];
   for (int c = 0; c < t.ncol; ++c) {
     if (seen[c]) continue;
@@ -228,8 +255,8 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
       seen[orb[m]] = true;
     }
     for (int k = 0; k < n; ++k) {
-      Vec v{orb[k], std::vector<int>(t.ncol, 0), n};
-      for (int m = 0; m < n; ++m) v.sign[orb[m]] = __builtin_popcount(k & m) & 1 ? -1 : 1;
+      Vec v{orb[k], {}, n};
+      for (int m = 0; m < n; ++m) v.sign.push_back({orb[m], __builtin_popcount(k & m) & 1 ? -1 : 1});
       blocks[self ? k | (__builtin_popcount(k & self) & 1) << 2 : k].push_back(v);
     }
   }
@@ -241,9 +268,9 @@ void build_tab64(int K, const Tables& t, const std::vector<int64_t>& num, Tab64&
       o.blk[b][i] = static_cast<uint8_t>(blocks[b][i].at);
       for (size_t j = i; j < blocks[b].size(); ++j) {
         int64_t s = 0;
-        for (int x = 0; x < t.ncol; ++x)
-          for (int y = 0; y < t.ncol; ++y)
-            s += num[static_cast<size_t>(x) * t.ncol + y] * blocks[b][i].sign[x] * blocks[b][j].sign[y];
+        for (const auto& x : blocks[b][i].sign)
+          for (const auto& y : blocks[b][j].sign)
+            s += num[static_cast<size_t>(x.first) * t.ncol + y.first] * (x.second * y.second);
         // (exact: an integer over a power of two)
         o.blk_c[nc++] = (i == j ? 1.0 : 2.0) * static_cast<double>(s) / (blocks[b][i].norm * blocks[b][j].norm);
       }
