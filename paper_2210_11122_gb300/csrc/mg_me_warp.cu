@@ -241,8 +241,14 @@ k_me_warp(const void* __restrict__ rec_any, int64_t nevt, const Tables* __restri
     };
     auto getP = [&](int seq, T* P) {
       const int msk = tab->seq_mask[seq];
+      if constexpr (std::is_same<T, float>::value) {   // (PT is the record's first item: 16-byte aligned)
+        static_assert(L::PT == 0, "vector load of a momentum");
+        const float4 v = *reinterpret_cast<const float4*>(rs + 4 * msk);
+        P[0] = v.x; P[1] = v.y; P[2] = v.z; P[3] = v.w;
+      } else {
 #pragma unroll
-      for (int m = 0; m < 4; ++m) P[m] = ld(L::PT + 4 * msk + m);
+        for (int m = 0; m < 4; ++m) P[m] = ld(L::PT + 4 * msk + m);
+      }
     };
     // current of sequence s (splits from the tables) into acc
     auto current = [&](int nv3, const int16_t (*v3)[2], int nv4, const int16_t (*v4)[3], cx<T>* acc) {
@@ -301,6 +307,32 @@ k_me_warp(const void* __restrict__ rec_any, int64_t nevt, const Tables* __restri
       }
     }
     __syncwarp(gmask);
+    // ---- the quark line takes the currents as gamma.J: its four entries replace J in place (the same sums that every
+    // term formed for itself: 8 of a term's 57 instructions) ----
+    for (int s = lane; s < WSizes<K>::nseq; s += G) {
+      cx<T> j[4];
+      getJ(2 * s, j);
+      const v2::Slash<T> g = v2::slash_of(j, false);
+      S.J[0][s] = stw(g.a);
+      S.J[1][s] = stw(g.b);
+      S.J[2][s] = stw(g.jm);
+      S.J[3][s] = stw(g.jp);
+    }
+    __syncwarp(gmask);
+    // gamma.J of a signed sequence reference of len gluons: only sequences of even length change sign under reversal, so
+    // the odd lengths (known at compile time) need no select
+    auto getG = [&](int ref, int len) -> v2::Slash<T> {
+      cx<T> j[4];
+      getJ(ref, j);
+      v2::Slash<T> g = {j[0], j[1], j[2], j[3]};
+      if (len % 2 == 0 && (ref & 1)) {
+        g.a = v2::cneg(g.a);
+        g.b = v2::cneg(g.b);
+        g.jm = v2::cneg(g.jm);
+        g.jp = v2::cneg(g.jp);
+      }
+      return g;
+    };
 
     // ---- quark line: half-group per top helicity, a run of orderings per lane ----
     {
@@ -325,10 +357,7 @@ k_me_warp(const void* __restrict__ rec_any, int64_t nevt, const Tables* __restri
             cx<T> acc[4] = {};
 #pragma unroll
             for (int j = 0; j < m; ++j) {
-              const int r = tab->sub[c][j][m];
-              cx<T> Jr[4];
-              getJ(r, Jr);
-              v2::row_gamma_acc(acc, stk[j], Jr, (r & 1) != 0);
+              v2::row_slash_acc(acc, stk[j], getG(tab->sub[c][j][m], m - j));
             }
             const int pm = tab->prefix_mask[c][m];
             T q[5];
@@ -349,10 +378,8 @@ k_me_warp(const void* __restrict__ rec_any, int64_t nevt, const Tables* __restri
           }
 #pragma unroll
           for (int j = 1; j < K; ++j) {
-            const int r = tab->sub[c][j][K];
-            cx<T> Jr[4], t[4] = {};
-            getJ(r, Jr);
-            v2::row_gamma_acc(t, stk[j], Jr, (r & 1) != 0);
+            cx<T> t[4] = {};
+            v2::row_slash_acc(t, stk[j], getG(tab->sub[c][j][K], K - j));
             v2::sdot_acc(amp0, t, vv[0], false);
             v2::sdot_acc(amp1, t, vv[1], false);
           }
