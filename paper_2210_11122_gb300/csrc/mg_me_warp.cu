@@ -337,7 +337,7 @@ k_me_warp(const void* __restrict__ rec_any, int64_t nevt, const Tables* __restri
     // ---- quark line: half-group per top helicity, a run of orderings per lane ----
     {
       constexpr int H = G / 2;   // lanes per top helicity
-      const int a = lane / H, hl = lane % H;
+      const int a = lane & 1, hl = lane >> 1;   // (neighbouring lanes read the same currents: fewer bank conflicts)
       const int c0 = hl * NCOL / H, c1 = (hl + 1) * NCOL / H;
       if (good[2 * a] || good[2 * a + 1]) {
         cx<T> vv[2][4], stk[K][4], Jq[2][4];
