@@ -222,7 +222,8 @@ __device__ __forceinline__ void me_static_body(Ld&& ld, int64_t e, int slot, int
           sum = fma(A[b][x].r, wr, sum);
           sum = fma(A[b][x].i, wi, sum);
         }
-        total += static_cast<double>(sum) * cst.colour_scale;
+        if constexpr (std::is_same<T, float>::value) total += v2::f64_of(sum) * cst.colour_scale;
+        else total += static_cast<double>(sum) * cst.colour_scale;
       }
     }
   }

@@ -109,6 +109,45 @@ template <> struct Sizes<5> { static constexpr int ncol = 120, nseq = 105, nfull
 __device__ __forceinline__ int rslot(int16_t r) { return r >> 1; }
 __device__ __forceinline__ bool rneg(int16_t r) { return r & 1; }
 
+// ---- conversions between FP64 and FP32 on the integer pipe ----
+// The hardware's conversions issue on the FP64 pipe (64 cycles a warp and sub-partition), where they were 38 % of the
+// FP32 modes' FP64-pipe instructions; from the IEEE 754 fields they are about ten integer instructions.
+// x rounded to nearest even, as static_cast<float>: results in FP32's normal range (a carry out of the mantissa moves the
+// exponent, as it should) and zeros here, the rest (FP32 subnormals, overflow, infinities, NaN) by the conversion.
+__device__ __forceinline__ float f32_of_normal(int hi, unsigned lo) {
+  const unsigned a = static_cast<unsigned>(hi) & 0x7fffffffu;
+  unsigned u = __funnelshift_l(lo, a - (896u << 20), 3);   // exponent rebiased, 23 mantissa bits kept
+  u += ((lo & 0x1fffffffu) + 0x0fffffffu + (u & 1u)) >> 29;
+  return __uint_as_float(u | (static_cast<unsigned>(hi) & 0x80000000u));
+}
+__device__ __forceinline__ float f32_of(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned a = static_cast<unsigned>(hi) & 0x7fffffffu;
+  if (a - (897u << 20) < (254u << 20)) return f32_of_normal(hi, static_cast<unsigned>(__double2loint(x)));
+  if (a < (1u << 20)) return __uint_as_float(static_cast<unsigned>(hi) & 0x80000000u);   // zero or FP64 subnormal
+  return static_cast<float>(x);
+}
+// x exactly, as static_cast<double>
+__device__ __forceinline__ double f64_of_normal(float x) {
+  const unsigned u = __float_as_uint(x);
+  return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))),
+                          static_cast<int>(u << 29));
+}
+__device__ __forceinline__ double f64_of(float x) {
+  const unsigned e = (__float_as_uint(x) >> 23) & 0xffu;
+  return e - 1u < 254u ? f64_of_normal(x) : static_cast<double>(x);
+}
+// an FP64 value as T
+template <class T> __device__ __forceinline__ T rounded(double x) { return static_cast<T>(x); }
+template <> __device__ __forceinline__ float rounded<float>(double x) { return f32_of(x); }
+// FP32 by the hardware's conversion: for the few warps of a latency-bound kernel (the helicity filter), where the FP64
+// pipe idles and the integer form is the longer chain (filter of gg -> t tbar 18.6 vs 22.3 us)
+struct hwf {
+  float v;
+  hwf() = default;
+  __device__ explicit hwf(double x) : v(static_cast<float>(x)) {}
+};
+
 // ---- FP64 helpers of the per-event record ----
 // Reciprocal and reciprocal square root for the FP32-amplitude path's record: an FP32 seed refined by
 // one Newton-Raphson step in FP64 (r <- r (2 - x r) for 1/x, y <- y (3 - x y^2) / 2 for 1/sqrt(x); each
@@ -121,12 +160,12 @@ __device__ __forceinline__ bool in_f32_range(double x) {
 }
 __device__ __forceinline__ double rcp_nr(double x) {
   if (!in_f32_range(x)) return 1.0 / x;
-  const double r0 = static_cast<double>(__frcp_rn(static_cast<float>(x)));
+  const double r0 = f64_of_normal(__frcp_rn(f32_of_normal(__double2hiint(x), static_cast<unsigned>(__double2loint(x)))));
   return r0 * fma(-x, r0, 2.0);
 }
 __device__ __forceinline__ double rsqrt_nr(double x) {
   if (!(__double2hiint(x) > 0 && in_f32_range(x))) return rsqrt(x);
-  const double y0 = static_cast<double>(rsqrtf(static_cast<float>(x)));
+  const double y0 = f64_of_normal(rsqrtf(f32_of_normal(__double2hiint(x), static_cast<unsigned>(__double2loint(x)))));
   return y0 * fma(-0.5 * x * y0, y0, 1.5);
 }
 // NR = false: correctly rounded FP64 operations (FP64 path); true: the Newton-refined forms above
@@ -182,8 +221,8 @@ __device__ __forceinline__ void top_ubar(const double* p, double m, int lam, cx<
   cx<double> c[2];
   chi2<NR>(p, pa, lam, c);
   const double fl = lam > 0 ? sm : sp, fr = lam > 0 ? sp : sm;
-  w[0] = {T(fr * c[0].r), T(-fr * c[0].i)}; w[1] = {T(fr * c[1].r), T(-fr * c[1].i)};
-  w[2] = {T(fl * c[0].r), T(-fl * c[0].i)}; w[3] = {T(fl * c[1].r), T(-fl * c[1].i)};
+  w[0] = {rounded<T>(fr * c[0].r), rounded<T>(-fr * c[0].i)}; w[1] = {rounded<T>(fr * c[1].r), rounded<T>(-fr * c[1].i)};
+  w[2] = {rounded<T>(fl * c[0].r), rounded<T>(-fl * c[0].i)}; w[3] = {rounded<T>(fl * c[1].r), rounded<T>(-fl * c[1].i)};
 }
 
 template <class T>
@@ -194,8 +233,8 @@ __device__ __forceinline__ void top_v(const double* p, double m, int lam, cx<T>*
   cx<double> c[2];
   chi2<NR>(p, pa, -lam, c);
   const double fl = lam > 0 ? -sp : sm, fr = lam > 0 ? sm : -sp;
-  w[0] = {T(fl * c[0].r), T(fl * c[0].i)}; w[1] = {T(fl * c[1].r), T(fl * c[1].i)};
-  w[2] = {T(fr * c[0].r), T(fr * c[0].i)}; w[3] = {T(fr * c[1].r), T(fr * c[1].i)};
+  w[0] = {rounded<T>(fl * c[0].r), rounded<T>(fl * c[0].i)}; w[1] = {rounded<T>(fl * c[1].r), rounded<T>(fl * c[1].i)};
+  w[2] = {rounded<T>(fr * c[0].r), rounded<T>(fr * c[0].i)}; w[3] = {rounded<T>(fr * c[1].r), rounded<T>(fr * c[1].i)};
 }
 
 // Transverse polarisation basis of a gluon of momentum k, pre-scaled by 1/sqrt(2):
@@ -224,9 +263,9 @@ __device__ __forceinline__ void gluon_pol(const double* k, T* pol) {
     ep[0] = 0.0; ep[1] = 1.0;
   }
 #pragma unroll
-  for (int i = 0; i < 3; ++i) pol[i] = T(r * et[i]);
-  pol[3] = T(r * ep[0]);
-  pol[4] = T(r * ep[1]);
+  for (int i = 0; i < 3; ++i) pol[i] = rounded<T>(r * et[i]);
+  pol[3] = rounded<T>(r * ep[0]);
+  pol[4] = rounded<T>(r * ep[1]);
 }
 
 // External gluon current of helicity lam: eps = (-lam e_theta + i s e_phi) / sqrt2, s = +1 for an
@@ -438,12 +477,12 @@ __device__ __forceinline__ void record_subsets(const double (*p)[4], const MeCon
       // sum or quark propagator; of the two, only the all-gluon propagator factor is read
       if (S != 0) {
         const double p2 = P[0] * P[0] - P[1] * P[1] - P[2] * P[2] - P[3] * P[3];
-        put(L::GP + S, static_cast<T>(sizeof(T) == 8 ? -cst.gs / p2 : -cst.gs * rcp_nr(p2)));
+        put(L::GP + S, rounded<T>(sizeof(T) == 8 ? -cst.gs / p2 : -cst.gs * rcp_nr(p2)));
       }
       continue;
     }
 #pragma unroll
-    for (int m = 0; m < 4; ++m) put(L::PT + 4 * S + m, static_cast<T>(P[m]));
+    for (int m = 0; m < 4; ++m) put(L::PT + 4 * S + m, rounded<T>(P[m]));
     const double p2 = P[0] * P[0] - P[1] * P[1] - P[2] * P[2] - P[3] * P[3];
     const double Q0 = p[2][0] - P[0], Q1 = p[2][1] - P[1], Q2 = p[2][2] - P[2], Q3 = p[2][3] - P[3];
     const double dq = Q0 * Q0 - Q1 * Q1 - Q2 * Q2 - Q3 * Q3 - cst.mt * cst.mt;
@@ -457,12 +496,12 @@ __device__ __forceinline__ void record_subsets(const double (*p)[4], const MeCon
       gp = (S & (S - 1)) ? -cst.gs * rcp_nr(p2) : 0.0;
       f = -cst.gs * rcp_nr(dq);
     }
-    put(L::GP + S, static_cast<T>(gp));
-    put(L::QC + 5 * S + 0, static_cast<T>((Q0 + Q3) * f));
-    put(L::QC + 5 * S + 1, static_cast<T>((Q0 - Q3) * f));
-    put(L::QC + 5 * S + 2, static_cast<T>(Q1 * f));
-    put(L::QC + 5 * S + 3, static_cast<T>(Q2 * f));
-    put(L::QC + 5 * S + 4, static_cast<T>(cst.mt * f));
+    put(L::GP + S, rounded<T>(gp));
+    put(L::QC + 5 * S + 0, rounded<T>((Q0 + Q3) * f));
+    put(L::QC + 5 * S + 1, rounded<T>((Q0 - Q3) * f));
+    put(L::QC + 5 * S + 2, rounded<T>(Q1 * f));
+    put(L::QC + 5 * S + 3, rounded<T>(Q2 * f));
+    put(L::QC + 5 * S + 4, rounded<T>(cst.mt * f));
   }
 }
 
@@ -534,8 +573,8 @@ __device__ __forceinline__ void record_j2(const double (*p)[4], const MeConst& c
         const int base = L::J2 + (pair_index(K, a, b) * 4 + h) * 8;
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-          put(base + 2 * m, static_cast<T>(gp * acc[m].r));
-          put(base + 2 * m + 1, static_cast<T>(gp * acc[m].i));
+          put(base + 2 * m, rounded<T>(gp * acc[m].r));
+          put(base + 2 * m + 1, rounded<T>(gp * acc[m].i));
         }
       }
     }
@@ -554,7 +593,8 @@ __device__ __forceinline__ void event_data(const double (*p)[4], const MeConst& 
                                            T (*pol)[5], cx<T> (*ub)[4], cx<T> (*vv)[4]) {
   using L = EvLayout<K>;
   T r[L::NBASE] = {};   // (the items no kernel reads stay zero)
-  record_all<K, T>(p, cst, [&](int i, T v) { r[i] = v; });
+  if constexpr (sizeof(T) == 4) record_all<K, hwf>(p, cst, [&](int i, hwf v) { r[i] = v.v; });
+  else record_all<K, T>(p, cst, [&](int i, T v) { r[i] = v; });
   constexpr int NSUB = 1 << K;
 #pragma unroll
   for (int S = 0; S < NSUB; ++S) {
@@ -587,7 +627,7 @@ __device__ __forceinline__ float min_invariant_ratio(const double (*p)[4], float
 #pragma unroll
   for (int i = 0; i < K + 2; ++i)
 #pragma unroll
-    for (int m = 0; m < 4; ++m) q[i][m] = static_cast<float>(p[i][m]);
+    for (int m = 0; m < 4; ++m) q[i][m] = f32_of(p[i][m]);
   float Pst[NSUB][4];
   float xmin = 3.0e38f;
 #pragma unroll
