@@ -845,11 +845,14 @@ mg_status mg_sigmakin_host(mg_ctx* ctx, const double* mom_host, int64_t nevt, mg
       }
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // up to kHostChunks chunks of whole 32-event pages, each of at least 16,384 events: the copies in run
+  // up to kHostChunks chunks of whole 32-event pages, each of at least 262,144 events: the copies in run
   // on cp_in, the matrix elements of chunk c on st once its momenta are in, its results go out on cp_out.
   // Per-event results do not depend on the chunking (the helicity filter of a first call sees the same
-  // first events, a chunk holding at least 16,384 of them).
-  int64_t nch = nevt / 16384;
+  // first events).  Host memory is copied at 190 GB/s (0.11 ms for 131,072 gg -> t tbar g events), so a chunk's
+  // own launches and partial waves cost more than its copy hides below that size: gg -> t tbar g, 65,536 events in one
+  // chunk 1.24 (MIXED 0.46) ms, in four 1.34 (0.78); 131,073: 2.40 (0.79) vs 2.46 (1.01); 524,288 in two 9.24 (2.75), in
+  // four 9.24 (2.81), in one 9.42 (2.88).
+  int64_t nch = nevt / 262144;
   if (nch < 1) nch = 1;
   if (nch > mg_ctx::kHostChunks) nch = mg_ctx::kHostChunks;
   const int64_t chunk = pad32((nevt + nch - 1) / nch);
