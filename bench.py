@@ -91,7 +91,7 @@ def parse():
 
 
 # sources of the FP64 slot kernels (body, algebra, dispatch): a committed traffic figure holds while their hash does
-ME_SOURCES = ("mg_me_kernel.cuh", "mg_me_algebra.cuh", "mg_me2.cu")
+ME_SOURCES = ("mg_me64.cuh", "mg_me64l.cuh", "mg_me64_k2.cuh", "mg_me64.cu", "mg_tables64.cpp", "mg_me_algebra.cuh")
 
 
 def profiled_traffic(kernel_files, profile_md, nevt):
@@ -307,10 +307,10 @@ def time_roofline(parts, me_ms):
 
 
 def fp64_roofline(model_flops, oracle_flops, nevt, me_ms, peak, traffic, kernel):
-    """ALU roofline of the FP64 path on the FP64 pipe.  achieved counts the flops of the engine's own
-    algorithm (its flop model, pinned to the hardware's FP64 instruction counts); the oracle-count
+    """ALU roofline of the FP64 path on the FP64 pipe.  achieved counts the flops the kernels execute
+    (model_flops: ncu's counts of one call, from the committed profile); the oracle-count
     figures count the FP64 oracle's instrumented operations (plain recursion per helicity) for the same
-    events in the same time, and count_ratio = oracle / engine flops per event."""
+    events in the same time, and count_ratio = oracle / executed flops per event."""
     ach = model_flops * nevt / (me_ms * 1e-3)
     r = {"bound": "alu", "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s", "frac": ach / peak,
          "traffic": traffic, "kernel": kernel, "flops_per_event": model_flops,
@@ -323,10 +323,19 @@ def fp64_roofline(model_flops, oracle_flops, nevt, me_ms, peak, traffic, kernel)
 
 
 def profile_for(process):
-    """The committed ncu summary of the FP64 matrix-element kernel of a process, if any."""
-    import glob
-    c = sorted(glob.glob(os.path.join(ROOT, "profiles", "k_me_gluonhel_fp64_%s_*.md" % process)))
-    return c[0] if c else None
+    """The committed ncu summary of one FP64 call of a process, if any."""
+    p = os.path.join(ROOT, "profiles", "fp64_call_%s_8192.md" % process)
+    return p if os.path.exists(p) else None
+
+
+def executed_fp64_flops(process):
+    """FP64 flops per event that one call executes, from the committed ncu summary (None without one)."""
+    p = profile_for(process)
+    if p:
+        for line in open(p):
+            if line.startswith("fp64_flops_per_event:"):
+                return float(line.split()[1])
+    return None
 
 
 # ------------------------------------------------------------------------------------------
@@ -423,12 +432,12 @@ class Leg:
             traffic = profiled_traffic([os.path.join(csrc, f) for f in ME_SOURCES], prof, nev) if prof else None
             shared = self.shapes[name]["shared"]
             K = self.ng + 2
-            slot_kernel = "k_me_gluonhel2" if K == 2 else "k_me64<%d>" % K
-            kernel = ("k_event_prep + %s%s + k_hel_sum (one mg_sigmakin call)"
-                      % ("k_pass64 (per pass) + " if shared and K >= 3 else "", slot_kernel))
-            return fp64_roofline(amp + col, oracle_flops, nev, me_ms, p64, traffic, kernel)
+            kernel = ("k_me64_k2" if K == 2 else "k_event_prep + %sk_me64<%d> + k_hel_sum_rows"
+                      % ("k_pass64 (per pass) + " if shared else "", K)) + " (one mg_sigmakin call)"
+            return fp64_roofline(executed_fp64_flops(self.process) or amp + col, oracle_flops, nev, me_ms, p64, traffic, kernel)
         if precision == mg.MG_FP64_TCCOLOR:
-            return time_roofline([("fp64", amp * nev, p64, src64),
+            # (the amplitudes of the FP64 call; its colour sums, here on the tensor cores, are a few per cent of its flops)
+            return time_roofline([("fp64", (executed_fp64_flops(self.process) or amp) * nev, p64, src64),
                                   ("tensor_f16", colour_tc_flops(ncol, ngood) * nev, ptc, tc_src)], me_ms)
         # FP32 amplitudes: the per-event FP64 record is the amplitude count with no good helicity
         rec64, _ = mg.flops_per_event(self.ng, [0] * len(mask), precision, flags)
