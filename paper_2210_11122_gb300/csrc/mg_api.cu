@@ -239,10 +239,11 @@ mg_status ctx_reserve(mg_ctx* ctx, int64_t nevt, mg_precision precision) {
   }
   if (s == MG_OK) s = grow(&ctx->d_prep, &ctx->prep_cap, chunk * event_record_bytes(ctx->K, fp32) / 8 + 1);
   if (s == MG_OK) s = grow_repair(ctx, chunk);
-  if (s == MG_OK && (precision == MG_FP64 || precision == MG_FP64_TCCOLOR) && ctx->shape[precision].shared &&
-      ctx->prm.wt == 0.0) {
-    const int64_t sc = share_chunk(ctx->K, stride);
-    s = grow(&ctx->d_share, &ctx->share_cap, (sc < chunk ? sc : chunk) * share_doubles(ctx->K));
+  if (s == MG_OK && (precision == MG_FP64 || precision == MG_FP64_TCCOLOR) && ctx->prm.wt == 0.0) {
+    // (the largest chunk of any batch up to nevt, as the FP64 branches of mg_sigmakin need it)
+    const int64_t need = (ctx->shape[precision].shared ? share_doubles(ctx->K) : 0) + (tc ? amp_doubles(ctx->K) : 0);
+    const int64_t sc = share_chunk(need, stride);
+    if (need > 0) s = grow(&ctx->d_share, &ctx->share_cap, (sc < chunk ? sc : chunk) * need);
   }
   return s;
 }

@@ -79,3 +79,30 @@ def test_channel_weights_of_both_paths(env, ng):
         for e in (0, 31, 32):
             ref = sde.weights(ng, evs[e], mask, dias=dias)[order]
             assert np.max(np.abs(got[:, e] - ref)) <= 1e-12 * ref.max()
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+def test_graph_of_fresh_contexts(env, precision):
+    """mg_graph_create reserves every scratch buffer of the FP64 modes before it captures: contexts that have run nothing
+    capture and replay, and give the bits of the same steps called one by one."""
+    torch, mg, orc = env
+    sizes = {0: 300, 1: 200, 2: 97, 3: 40}
+    ctxs = {p: mg.Context(p) for p in sizes}
+    bufs = {p: (torch.zeros(ctxs[p].mom_count(n), dtype=torch.float64, device="cuda"),
+                torch.zeros(n, dtype=torch.float64, device="cuda")) for p, n in sizes.items()}
+    g = mg.GraphBatch([(ctxs[p], 11 + p, 0, n, 1500.0, bufs[p][0], bufs[p][1], precision) for p, n in sizes.items()])
+    live = mg.live_allocs()
+    g.launch()
+    torch.cuda.synchronize()
+    assert mg.live_allocs() == live
+    for p, n in sizes.items():
+        with mg.Context(p) as c:
+            mom = torch.zeros(c.mom_count(n), dtype=torch.float64, device="cuda")
+            me = torch.zeros(n, dtype=torch.float64, device="cuda")
+            c.rambo(11 + p, n, 1500.0, mom)
+            c.hel_filter(mom, n)
+            c.sigmakin(mom, n, me, precision)
+            assert torch.equal(me, bufs[p][1]), p
+    g.close()
+    for c in ctxs.values():
+        c.close()
