@@ -82,6 +82,7 @@ namespace mg {
 int64_t share_doubles(int K);
 int64_t amp_doubles(int K);
 int64_t share_chunk(int64_t per_event, int64_t stride);
+int64_t share_chunk_max(int64_t per_event, int64_t stride);   // the bound that share_chunk evens out
 // FP64 colour sums of n events (from a page boundary: FP64 records rec; zero top width; 3 to 5 gluons) in rows of out, for
 // fp64_hel_sum.  shared: through the items buffer (d_share, share_doubles(K) * pad(n) doubles), else every combination on
 // its own.
