@@ -176,8 +176,10 @@ mg_status mg_check(mg_ctx* ctx, void* stream, int64_t* nbad);
  * an FMA as 2.  The FP64-amplitude modes tabulate (gamma.J) v per current, the FP32-amplitude modes
  * form it per jamp term; from gg -> t tbar g on, the FP64-amplitude count is that of the
  * default MG_LAUNCH_SHARED algorithm (the currents of fewer than all gluons, with their (gamma.J) v, once
- * per helicity assignment of their own gluons per event).  mask (ceil(nhel/32) words, as returned by
- * mg_hel_mask) selects the good helicities; NULL = all.  Host only. */
+ * per helicity assignment of their own gluons per event).  It counts every good helicity, whereas the
+ * FP64 kernels evaluate one of each pair of helicities related by flipping all of them, over linear
+ * polarisations: they execute 0.33 / 0.21 / 0.14 of it for 3 / 4 / 5 gluons.  mask (ceil(nhel/32) words, as
+ * returned by mg_hel_mask) selects the good helicities; NULL = all.  Host only. */
 mg_status mg_flops_per_event(mg_process proc, mg_precision precision, const uint32_t* mask, double* amp_flops,
                              double* colour_flops);
 
@@ -188,7 +190,8 @@ mg_status mg_flops_per_event(mg_process proc, mg_precision precision, const uint
 mg_status mg_flops_per_event_shape(mg_process proc, mg_precision precision, const uint32_t* mask, int flags,
                                    double* amp_flops, double* colour_flops);
 
-/* FP64 matrix elements exactly as mg_sigmakin(..., MG_FP64, ...), for callers that must not have
+/* FP64 matrix elements as mg_sigmakin(..., MG_FP64, ...) (up to rounding: one thread per event and gluon
+ * helicities, without the items that mg_sigmakin shares), for callers that must not have
  * the library allocate device memory during the call (an application that hands the engine a
  * fixed memory budget, or whose own pooling allocator must remain the only one): this entry point
  * calls no cudaMalloc/cudaFree and no allocating routine.  The paper has no counterpart; it is an
@@ -236,10 +239,10 @@ mg_status mg_sigmakin_noalloc(mg_ctx* ctx, const double* mom_dev, int64_t nevt, 
  * needed when the matching output is requested, else MG_EINVAL).  hel_dev / col_dev: int32 per event.
  * Every buffer holds nevt entries.  Zero top width only (MG_ENOTSUP otherwise).  The matrix elements come
  * from the FP64 algorithm that the context's MG_FP64 launch shape selects (with MG_LAUNCH_SHARED: the
- * shared currents and quark-line prefixes); at fixed coupling they equal mg_sigmakin(MG_FP64)'s up to the
- * order of the helicity sum.
- * Scratch: per-slot sums of |J_sigma|^2 (events processed in chunks that keep it within 1 GiB, and the
- * shared currents within 2 GiB), owned by the context.  If no helicity mask exists yet, the call first
+ * shared items); at fixed coupling they equal mg_sigmakin(MG_FP64)'s up to rounding (the sums run over
+ * helicities, there over linear gluon polarisations).
+ * Scratch: the amplitudes, the items shared by them and the sums of |J_sigma|^2 (events processed in chunks
+ * that keep it within 2 GiB), owned by the context.  If no helicity mask exists yet, the call first
  * runs mg_hel_filter on its own first events. */
 mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, const double* rnd_hel_dev,
                           const double* rnd_col_dev, int running_alphas, double* me_dev, int* hel_dev, int* col_dev,
@@ -260,7 +263,7 @@ mg_status mg_alphas_running(mg_ctx* ctx, const double* mom_dev, int64_t nevt, do
  * A_d the diagram's amplitude with its colour factor stripped (Feynman-gauge vertices and propagators; the
  * couplings and phases, common to all channels, cancel).  w_dev holds nchannels * nevt doubles.  Zero top
  * width (MG_ENOTSUP otherwise); if no helicity mask exists yet, the call first runs mg_hel_filter on its
- * own first events.  Scratch (events in chunks of at most 2 GiB of per-channel sums) is owned by the context. */
+ * own first events.  Scratch (events in chunks of at most 2 GiB) is owned by the context. */
 mg_status mg_sde_weights(mg_ctx* ctx, const double* mom_dev, int64_t nevt, double* w_dev, void* stream);
 
 /* Number of channels of a process.  Host only. */
@@ -334,7 +337,8 @@ mg_status mg_autotune(mg_ctx* ctx, mg_precision precision, int64_t nevt, const c
 mg_status mg_get_launch_shape(mg_ctx* ctx, mg_precision precision, int* tile_ev, int* slot_major, int* flags);
 
 /* Set the launch shape of mg_sigmakin(precision) by hand: tile_ev in {32, 64, 128}, slot_major 0 or 1,
- * flags a combination of the MG_LAUNCH_ bits.  MG_EINVAL otherwise. */
+ * flags a combination of the MG_LAUNCH_ bits.  MG_EINVAL otherwise.  (With zero top width the FP64-amplitude
+ * kernels read slot_major, MG_LAUNCH_SHARED and, for the colour pass, MG_LAUNCH_TC_SYNC only.) */
 mg_status mg_set_launch_shape(mg_ctx* ctx, mg_precision precision, int tile_ev, int slot_major, int flags);
 
 /* FP32 modes (MG_FP32_AMP, MG_MIXED): the events whose smallest internal invariant -- |P^2| of a gluon
@@ -369,11 +373,11 @@ typedef struct {
 
 /* FP64 matrix elements of njobs jobs (1..64, any mix of processes, one context each, zero top width) with
  * ONE persistent kernel launch for all their matrix elements: its thread blocks drain a queue of (job,
- * gluon-helicity slot, 128-event tile) work items (the jobs with more gluons first) from an atomic counter,
+ * block of amplitude rows, 32-event tile) work items (the jobs with more gluons first) from an atomic counter,
  * so many small jobs fill the GPU together (the paper's Sec. 4: throughput keeps growing up to batches of
  * ~16k events).  Per job, as mg_sigmakin(MG_FP64): the helicity filter on its own first events if its
  * context has no mask yet, the per-event records, and the helicity sums after the shared launch.  Results
- * are bit-identical to mg_sigmakin(MG_FP64) with a launch shape without MG_LAUNCH_SHARED.  Stream-ordered,
+ * are bit-identical to mg_sigmakin(MG_FP64).  Stream-ordered,
  * graph-capturable once each context's scratch is large enough (mg_graph_create reserves it). */
 mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void* stream);
 

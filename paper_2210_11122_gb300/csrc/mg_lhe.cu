@@ -3,8 +3,9 @@
 //
 // The paper (Sec. 4) names event-by-event helicities and leading colours as the two pieces missing from
 // the LHE files written with its GPU matrix elements, and the running of alpha_s (Sec. 2) as a feature
-// the engine gained; both are cheap per-event epilogues on quantities the matrix-element kernel already
-// has: the colour-summed |M_h|^2 of every helicity and the colour-ordered amplitudes (jamps).
+// the engine gained; both are cheap per-event epilogues on the colour-summed |M_h|^2 of every helicity
+// and the colour-ordered amplitudes (jamps), which from three gluons on the FP64
+// kernels of mg_me64.cu write over linear gluon polarisations and k_helicities turns into helicities'.
 //   * helicity choice: the smallest good helicity h (ascending index) whose running sum of |M_h|^2
 //     exceeds r_hel times the sum over all good helicities;
 //   * colour choice: the smallest colour flow sigma (lexicographic permutation rank) whose running sum

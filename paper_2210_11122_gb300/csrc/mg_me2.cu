@@ -1,9 +1,11 @@
-// mg_me2.cu -- matrix-element kernel, one thread per (event, gluon-helicity combination).
+// mg_me2.cu -- matrix-element kernel, one thread per (event, gluon-helicity combination): FP32 and double-float
+// amplitudes, the helicity filter, events recomputed in FP64, mg_sigmakin_noalloc and the FP64 jamps of two gluons (mg_me64.cu
+// has the other FP64 kernels).
 //
 // Same physics as the per-helicity kernel of mg_me.cu (HELAS wavefunctions, every tree diagram of
 // g g -> t tbar + (K-2) g summed into colour-ordered amplitudes by the Berends-Giele recursion of
 // mg_tables.cpp, exact colour matrix, helicity sum; the hot path of the paper's Sec. 2), organised
-// for GB300's FP64 pipe (2 DFMA/clk/SM, 1/64 of FP32), where the instruction count is the cost:
+// so that few instructions are executed:
 //   * the gluon currents J(seq) and the all-gluon currents J(sigma) depend only on the gluon
 //     helicities: one thread computes them once and reuses them for the 4 top-helicity pairs;
 //   * quark-line prefixes depend on the top helicity only: one depth-first walk per top helicity,
