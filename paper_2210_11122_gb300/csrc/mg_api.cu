@@ -707,28 +707,30 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
     chunk = chunk / mg::kPage * mg::kPage;
     if (chunk < mg::kPage) chunk = mg::kPage;
     if (chunk > stride) chunk = stride;
+    int64_t room = chunk;   // events the scratch holds (share_chunk)
     // FP64 amplitudes: optionally through the shared items (as MG_FP64)
     const bool shared = !fp32 && ctx->shape[precision].shared && ctx->K >= 3;
     const bool amps = !fp32 && ctx->K >= 3;
     if (amps) {
       const int64_t need = (shared ? mg::share_doubles(ctx->K) : 0) + mg::amp_doubles(ctx->K);
-      const int64_t sc = mg::share_chunk(need, stride);
+      const int64_t sc = mg::share_chunk(need, stride), most = mg::share_chunk_max(need, stride);
       if (sc < chunk) chunk = sc;
-      s = grow(&ctx->d_share, &ctx->share_cap, chunk * need);
+      if (most < room) room = most;
+      s = grow(&ctx->d_share, &ctx->share_cap, room * need);
       if (s != MG_OK) return s;
     }
-    if (ctx->jamp_cap < chunk * per_event) {
+    if (ctx->jamp_cap < room * per_event) {
       if (ctx->d_jamps) mg::dev_free(ctx->d_jamps);
       ctx->d_jamps = nullptr;
       ctx->jamp_cap = 0;
-      if (mg::dev_alloc(&ctx->d_jamps, static_cast<size_t>(chunk * per_event) * sizeof(float2)) != cudaSuccess) {
+      if (mg::dev_alloc(&ctx->d_jamps, static_cast<size_t>(room * per_event) * sizeof(float2)) != cudaSuccess) {
         cudaGetLastError();
         return MG_ENOMEM;
       }
-      ctx->jamp_cap = chunk * per_event;
+      ctx->jamp_cap = room * per_event;
     }
-    s = grow(&ctx->d_prep, &ctx->prep_cap, chunk * mg::event_record_bytes(ctx->K, fp32) / 8 + 1);
-    if (s == MG_OK && fp32) s = grow_repair(ctx, chunk);
+    s = grow(&ctx->d_prep, &ctx->prep_cap, room * mg::event_record_bytes(ctx->K, fp32) / 8 + 1);
+    if (s == MG_OK && fp32) s = grow_repair(ctx, room);
     if (s != MG_OK) return s;
     for (int64_t e0 = 0; e0 < nevt; e0 += chunk) {
       const int64_t n = nevt - e0 < chunk ? nevt - e0 : chunk;
@@ -794,8 +796,8 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
     const bool shared = !fp32 && ctx->shape[precision].shared && ctx->K >= 3;
     if (!fp32) {
       // with shared items, in chunks of events that bound their buffer
-      const int64_t chunk = shared ? mg::share_chunk(mg::share_doubles(ctx->K), stride) : stride;
-      if (shared) s = grow(&ctx->d_share, &ctx->share_cap, chunk * mg::share_doubles(ctx->K));
+      const int64_t items = mg::share_doubles(ctx->K), chunk = shared ? mg::share_chunk(items, stride) : stride;
+      if (shared) s = grow(&ctx->d_share, &ctx->share_cap, mg::share_chunk_max(items, stride) * items);
       if (s != MG_OK) return s;
       const int64_t nitem = mg::event_record_bytes(ctx->K, false) / 8;
       for (int64_t e0 = 0; e0 < nevt; e0 += chunk) {

@@ -228,11 +228,12 @@ mg_status mg_sigmakin_lhe(mg_ctx* ctx, const double* mom_dev, int64_t nevt, cons
   const int64_t stride_all = pad_page(nevt);
   const bool shared = ctx->shape[MG_FP64].shared && K >= 3;
   const int64_t need = (shared ? mg::share_doubles(K) : 0) + mg::amp_doubles(K);
-  int64_t chunk = K >= 3 ? mg::share_chunk(need, stride_all) : mg::share_chunk(2 * j2rows, stride_all);
-  mg_status s = grow_buf(&ctx->d_part, &ctx->part_cap, chunk * ctx->nhel);
-  if (s == MG_OK) s = grow_buf(&ctx->d_prep, &ctx->prep_cap, chunk * mg::event_record_bytes(K, false) / 8 + 1);
-  if (s == MG_OK) s = grow_buf(&ctx->d_j2, &ctx->j2_cap, chunk * j2rows);
-  if (s == MG_OK && need > 0) s = grow_buf(&ctx->d_share, &ctx->share_cap, chunk * need);
+  const int64_t per_event = K >= 3 ? need : 2 * j2rows;
+  const int64_t chunk = mg::share_chunk(per_event, stride_all), room = mg::share_chunk_max(per_event, stride_all);
+  mg_status s = grow_buf(&ctx->d_part, &ctx->part_cap, room * ctx->nhel);
+  if (s == MG_OK) s = grow_buf(&ctx->d_prep, &ctx->prep_cap, room * mg::event_record_bytes(K, false) / 8 + 1);
+  if (s == MG_OK) s = grow_buf(&ctx->d_j2, &ctx->j2_cap, room * j2rows);
+  if (s == MG_OK && need > 0) s = grow_buf(&ctx->d_share, &ctx->share_cap, room * need);
   if (s != MG_OK) return s;
   mg::MeConst cst;
   cst.gs = std::sqrt(4.0 * 3.14159265358979323846 * ctx->prm.alphas);
