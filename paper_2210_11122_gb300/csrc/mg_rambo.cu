@@ -70,11 +70,8 @@ __global__ void __launch_bounds__(128) k_rambo(uint64_t seed, int64_t e0, int64_
     Q0 += q[j][0]; Q1 += q[j][1]; Q2 += q[j][2]; Q3 += q[j][3];
   }
   const double M = sqrt(Q0 * Q0 - Q1 * Q1 - Q2 * Q2 - Q3 * Q3);
-  // (one reciprocal of M: an FP64 division is about twenty instructions, and at 16,384 events a warp's chain of them is
-  // the kernel's time)
-  const double r = 1.0 / M;
-  const double b1 = -Q1 * r, b2 = -Q2 * r, b3 = -Q3 * r;
-  const double gam = Q0 * r, a = 1.0 / (1.0 + gam), x = sqrts * r;
+  const double b1 = -Q1 / M, b2 = -Q2 / M, b3 = -Q3 / M;
+  const double gam = Q0 / M, a = 1.0 / (1.0 + gam), x = sqrts / M;
   double p[NF][4];
 #pragma unroll
   for (int j = 0; j < NF; ++j) {
@@ -110,9 +107,8 @@ __global__ void __launch_bounds__(128) k_rambo(uint64_t seed, int64_t e0, int64_
       const double v = xi * p[j][0];
       p[j][1] *= xi; p[j][2] *= xi; p[j][3] *= xi;
       p[j][0] = ej;
-      const double beta = v / ej;
-      prod *= beta;
-      sumv += v * beta;
+      prod *= v / ej;
+      sumv += v * v / ej;
     }
     double xp = 1.0;
 #pragma unroll
