@@ -858,14 +858,18 @@ mg_status mg_sigmakin_host(mg_ctx* ctx, const double* mom_host, int64_t nevt, mg
       }
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // up to kHostChunks chunks of whole 32-event pages, each of at least 262,144 events: the copies in run
+  // up to kHostChunks chunks of whole 32-event pages, each of at least 131,072 events: the copies in run
   // on cp_in, the matrix elements of chunk c on st once its momenta are in, its results go out on cp_out.
   // Per-event results do not depend on the chunking (the helicity filter of a first call sees the same
-  // first events).  Host memory is copied at 190 GB/s (0.11 ms for 131,072 gg -> t tbar g events), so a chunk's
-  // own launches and partial waves cost more than its copy hides below that size: gg -> t tbar g, 65,536 events in one
-  // chunk 1.24 (MIXED 0.46) ms, in four 1.34 (0.78); 131,073: 2.40 (0.79) vs 2.46 (1.01); 524,288 in two 9.24 (2.75), in
-  // four 9.24 (2.81), in one 9.42 (2.88).
-  int64_t nch = nevt / 262144;
+  // first events).  Pinned memory is copied at about 190 GB/s, so with the cheapest kernels (gg -> t tbar in FP32:
+  // 0.8 ns per event) the copies are half as long as the matrix elements and worth hiding, but a chunk's own launches
+  // and partial waves cost 20 to 70 us.  Smallest chunk 16,384 / 131,072 / 262,144 events, us per call:
+  //   pinned    gg -> t tbar FP32      65,536 events 161 / 141 / 142, 262,144 372 / 356 / 409, 524,287 598 / 605 / 775
+  //             gg -> t tbar g FP32    65,536 events 730 / 298 / 302, 262,144 995 / 912 / 951, 524,287 1,684 / 1,666 / 1,860
+  //             gg -> t tbar g FP64    131,073 events 2,473 / 2,415 / 2,415, 524,287 9,255 / 9,235 / 9,440
+  //   pageable  gg -> t tbar FP32      262,144 events 560 / 459 / 420
+  // from 2 final-state gluons on the three are within 2 %.
+  int64_t nch = nevt / 131072;
   if (nch < 1) nch = 1;
   if (nch > mg_ctx::kHostChunks) nch = mg_ctx::kHostChunks;
   const int64_t chunk = pad32((nevt + nch - 1) / nch);
