@@ -189,6 +189,16 @@ int64_t share_chunk(int64_t per_event, int64_t stride) {
   return pad32((stride + nch - 1) / nch);
 }
 
+int64_t item_chunk_max(const mg_ctx* ctx, int64_t stride) {
+  const int64_t most = share_chunk_max(share_doubles(ctx->K), stride);
+  return ctx->item_events > 0 && ctx->item_events < most ? ctx->item_events : most;
+}
+
+int64_t item_chunk(const mg_ctx* ctx, int64_t stride) {
+  const int64_t chunk = share_chunk(share_doubles(ctx->K), stride);
+  return ctx->item_events > 0 && ctx->item_events < chunk ? ctx->item_events : chunk;
+}
+
 cudaError_t fp64_slots(mg_ctx* ctx, const double* rec, int64_t n, bool shared, const MeConst& cst,
                        double* out, int64_t stride, MeShape shape, cudaStream_t st) {
   if (shared) {
@@ -251,7 +261,7 @@ mg_status ctx_reserve(mg_ctx* ctx, int64_t nevt, mg_precision precision) {
   if (s == MG_OK && (precision == MG_FP64 || precision == MG_FP64_TCCOLOR) && ctx->prm.wt == 0.0) {
     // (the largest chunk of any batch up to nevt, as the FP64 branches of mg_sigmakin need it)
     const int64_t need = (ctx->shape[precision].shared ? share_doubles(ctx->K) : 0) + (tc ? amp_doubles(ctx->K) : 0);
-    const int64_t sc = share_chunk_max(need, stride);
+    const int64_t sc = tc ? share_chunk_max(need, stride) : item_chunk_max(ctx, stride);
     if (need > 0) s = grow(&ctx->d_share, &ctx->share_cap, (sc < chunk ? sc : chunk) * need);
   }
   return s;
@@ -796,8 +806,8 @@ mg_status mg_sigmakin(mg_ctx* ctx, const double* mom_dev, int64_t nevt, mg_preci
     const bool shared = !fp32 && ctx->shape[precision].shared && ctx->K >= 3;
     if (!fp32) {
       // with shared items, in chunks of events that bound their buffer
-      const int64_t items = mg::share_doubles(ctx->K), chunk = shared ? mg::share_chunk(items, stride) : stride;
-      if (shared) s = grow(&ctx->d_share, &ctx->share_cap, mg::share_chunk_max(items, stride) * items);
+      const int64_t chunk = shared ? mg::item_chunk(ctx, stride) : stride;
+      if (shared) s = grow(&ctx->d_share, &ctx->share_cap, mg::item_chunk_max(ctx, stride) * mg::share_doubles(ctx->K));
       if (s != MG_OK) return s;
       const int64_t nitem = mg::event_record_bytes(ctx->K, false) / 8;
       for (int64_t e0 = 0; e0 < nevt; e0 += chunk) {

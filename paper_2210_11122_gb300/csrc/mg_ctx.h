@@ -56,6 +56,7 @@ struct mg_ctx {
   mg::Tab64* d_tab64 = nullptr;   // FP64 matrix elements of 3 to 5 gluons: items, tasks and terms
   double* d_share = nullptr;   // FP64: items shared between gluon-helicity combinations (one chunk of events)
   int64_t share_cap = 0;      // in doubles
+  int64_t item_events = 0;    // > 0: MG_FP64 holds the items of at most this many events at a time
   cudaStream_t side = nullptr;         // FP32 modes: the FP64 recomputation runs here, beside the FP32 launches
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int64_t prep_cap = 0;       // in doubles
@@ -85,6 +86,9 @@ int64_t share_doubles(int K);
 int64_t amp_doubles(int K);
 int64_t share_chunk(int64_t per_event, int64_t stride);
 int64_t share_chunk_max(int64_t per_event, int64_t stride);   // the bound that share_chunk evens out
+// the same for the items of MG_FP64, within the context's item_events
+int64_t item_chunk(const mg_ctx* ctx, int64_t stride);
+int64_t item_chunk_max(const mg_ctx* ctx, int64_t stride);
 // FP64 colour sums of n events (from a page boundary: FP64 records rec; zero top width; 3 to 5 gluons) in rows of out, for
 // fp64_hel_sum.  shared: through the items buffer (d_share, share_doubles(K) * pad(n) doubles), else every combination on
 // its own.

@@ -42,6 +42,15 @@ namespace {
 
 using Clock = std::chrono::steady_clock;
 
+// A server of small chunks (at most 1,024 events) is one of bounded memory, not of throughput.  The shared items of
+// gg -> t tbar g g g in FP64 are 309 KB per event, 316 MB for every slot's context and 45 times the rest of its scratch,
+// so there they are held for two pages of events at a time (20 MB; the same bits).  Without the items, which this replaces,
+// the kernel's 50 KB of local memory per thread made the driver reserve 12 GB on the first request: a one-slot server
+// 2.7 instead of 14.8 GB after a request, an eight-slot one 3.3 instead of 15.2.  1,024 events take 8.6 ms in one slot
+// (7.8 without the items, 2.6 with the items of all of them), and 3.2 ms with eight slots at work (6.4 without), the
+// slots' launches of two pages running side by side.
+constexpr int64_t kSmallChunk = 1024, kSmallChunkItems = 64;
+
 struct Request {
   bool small = true;
   uint64_t ticket;
@@ -259,11 +268,7 @@ mg_status mg_serve_create(const mg_serve_cfg* cfg_in, mg_server** out) {
     }
     for (int p = 0; p < 4 && st == MG_OK; ++p) {
       st = mg_create(static_cast<mg_process>(p), &cfg.params, &s.ctx[p]);
-      // A server of small chunks (at most 1,024 events: bounded memory and prompt cancellation, not throughput) runs
-      // gg -> t tbar g g g in FP64 without the shared items, the same bits: they are 309 KB per event, up to 316 MB
-      // for every slot and outside the admission footprint (7 KB per event).  It takes 8.6 instead of 2.7 ms per
-      // 1,024 events, so servers of larger chunks keep them.
-      if (st == MG_OK && p == MG_GG_TTGGG && nmax <= 1024) s.ctx[p]->shape[MG_FP64].shared = false;
+      if (st == MG_OK && p == MG_GG_TTGGG && nmax <= kSmallChunk) s.ctx[p]->item_events = kSmallChunkItems;
       if (st == MG_OK) st = mg::ctx_reserve(s.ctx[p], nmax, cfg.precision);
     }
     if (st != MG_OK) break;

@@ -1,0 +1,37 @@
+"""Device memory of calls whose kernels could make the driver reserve local memory for every thread the GPU can hold:
+measured in a process of its own, the context and the library's buffers included."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+HEAD = """
+import torch
+import paper_2210_11122_gb300 as mg
+torch.zeros(1, device="cuda")
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+"""
+TAIL = """
+torch.cuda.synchronize()
+print("used_mib", (free - torch.cuda.mem_get_info()[0]) >> 20)
+"""
+SERVE = """
+srv = mg.Server(slots=1, max_nevt=1024)
+srv.wait(srv.submit("ggttggg", 5, 1024))
+"""
+
+
+# 2.7 GB measured, 14.8 GB with a kernel of 50 KB of local memory per thread; the bound is twice the former
+@pytest.mark.parametrize("code,bound_mib", [(SERVE, 5500)], ids=["server"])
+def test_device_memory(code, bound_mib):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    r = subprocess.run([sys.executable, "-c", HEAD + code + TAIL], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert int(r.stdout.split("used_mib")[1]) <= bound_mib, r.stdout
