@@ -377,8 +377,9 @@ typedef struct {
  * so many small jobs fill the GPU together (the paper's Sec. 4: throughput keeps growing up to batches of
  * ~16k events).  Per job, as mg_sigmakin(MG_FP64): the helicity filter on its own first events if its
  * context has no mask yet, the per-event records, and the helicity sums after the shared launch.  Results
- * are bit-identical to mg_sigmakin(MG_FP64).  Stream-ordered,
- * graph-capturable once each context's scratch is large enough (mg_graph_create reserves it). */
+ * are bit-identical to mg_sigmakin(MG_FP64).  A job whose shared items exceed 2 GiB (more than 6,944
+ * gg -> t tbar g g g or 53,664 gg -> t tbar g g events) runs in chunks and launches of its own, as mg_sigmakin's.
+ * Stream-ordered, graph-capturable once each context's scratch is large enough (mg_graph_create reserves it). */
 mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void* stream);
 
 /* Flags of mg_graph_create_ex. */

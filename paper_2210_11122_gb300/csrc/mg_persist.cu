@@ -7,10 +7,10 @@
 // (job, block of helicities, tile of 32 events) triples, the jobs ordered by falling cost per tile (more
 // gluons first, so the longest tiles start first); each 128-thread block takes the next tile from an
 // atomic counter until the queue is empty, and runs the same per-thread FP64 work as the
-// single-job kernels (the
-// per-event record from k_event_prep; the items shared between a job's gluon-helicity combinations from its
-// launch_pass64 where its context's FP64 shape shares them and the job's buffer fits 2 GiB, else built in
-// the thread).  The results are
+// single-job kernels (the per-event record
+// from k_event_prep; the items shared between a job's gluon-helicity combinations from its
+// launch_pass64 where its context's FP64 shape shares them, else built in the thread; a job whose items exceed
+// 2 GiB runs in launches of its own).  The results are
 // bit-identical to mg_sigmakin(MG_FP64), with or without the shared currents.
 #include <cuda_runtime.h>
 
@@ -53,16 +53,20 @@ struct PBatch {
   PJob job[kMaxJobs];
 };
 
-template <int K>
+template <int K, bool OWN>
 __device__ __forceinline__ void run64(const PJob& J, int64_t tile, int blk) {
-  if (J.share)
+  if (!OWN || J.share)
     m64::thread64<K, false, false>(J.rec, J.nevt, tile, blk, J.tab, J.t64, J.gslots, J.nslot, J.lin, J.mask, J.ctri, J.cst,
                                    J.part, J.stride, J.share);
-  else
+  else if constexpr (OWN)
     m64::thread64<K, false, true>(J.rec, J.nevt, tile, blk, J.tab, J.t64, J.gslots, J.nslot, J.lin, J.mask, J.ctri, J.cst,
                                   J.part, J.stride, nullptr);
 }
 
+// OWN: some job of 3 to 5 gluons runs without shared items.  Its threads keep their items in 50 KB of local memory, which
+// the driver reserves for every thread the GPU can hold (14.7 GB of device memory in all, against 2.7), so batches whose jobs all
+// share have a kernel without that code.
+template <bool OWN>
 __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_constant__ PBatch b,
                                                               unsigned long long* __restrict__ next) {
   __shared__ long long s_tile;
@@ -85,9 +89,9 @@ __global__ void __launch_bounds__(kMeThreads, 3) k_me_persistent(const __grid_co
     const int64_t etile = t - static_cast<int64_t>(slot) * J.ntile_ev;
     switch (J.K) {
       case 2: m64::k2_page(s_k2, J.rec, J.nevt, etile, J.mask, J.ctri, J.cst, J.norm, J.part); break;
-      case 3: run64<3>(J, etile, slot); break;
-      case 4: run64<4>(J, etile, slot); break;
-      default: run64<5>(J, etile, slot); break;
+      case 3: run64<3, OWN>(J, etile, slot); break;
+      case 4: run64<4, OWN>(J, etile, slot); break;
+      default: run64<5, OWN>(J, etile, slot); break;
     }
   }
 }
@@ -133,6 +137,7 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
   batch->njobs = 0;
   batch->ntiles = 0;
   mg_status s = MG_OK;
+  bool own = false;
   for (int oi = 0; oi < njobs && s == MG_OK; ++oi) {
     const mg_batch_job& j = jobs[order[oi]];
     mg_ctx* c = j.ctx;
@@ -151,15 +156,27 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     cst.colour_scale = cst.gs * cst.gs / static_cast<double>(c->colour_den);
     if (c->K >= 3 && mg::launch_event_prep(c->K, false, j.mom_dev, j.nevt, cst, c->d_prep, st) != cudaSuccess) { s = MG_ECUDA; break; }
     // the job's items shared between its gluon-helicity combinations, where its
-    // context's FP64 shape asks for them and the whole job's buffer stays within 2 GiB
+    // context's FP64 shape asks for them
     const double* share = nullptr;
-    const int64_t sdoubles = stride * mg::share_doubles(c->K);
-    if (c->shape[MG_FP64].shared && c->K >= 3 && sdoubles <= (int64_t(1) << 28)) {
-      s = grow_d(&c->d_share, &c->share_cap, sdoubles);
+    if (c->shape[MG_FP64].shared && c->K >= 3) {
+      const int64_t chunk = mg::item_chunk(c, stride);
+      s = grow_d(&c->d_share, &c->share_cap, mg::item_chunk_max(c, stride) * mg::share_doubles(c->K));
       if (s != MG_OK) break;
+      if (chunk < stride) {
+        // items over 2 GiB: the job's matrix elements in chunks and launches of its own, as mg_sigmakin's.  In the
+        // persistent launch without items 7,008 gg -> t tbar g g g events took 43.3 ms, now 15.3, 60,000
+        // gg -> t tbar g g events 33.3, now 9.4
+        const int64_t nitem = mg::event_record_bytes(c->K, false) / 8;
+        for (int64_t e0 = 0; e0 < j.nevt && s == MG_OK; e0 += chunk)
+          if (mg::fp64_slots(c, c->d_prep + (e0 / mg::kPage) * nitem * mg::kPage, j.nevt - e0 < chunk ? j.nevt - e0 : chunk,
+                             true, cst, c->d_part + e0, stride, c->shape[MG_FP64], st) != cudaSuccess)
+            s = MG_ECUDA;
+        continue;
+      }
       if (mg::launch_pass64(c->K, c->d_prep, j.nevt, c->d_tab, c->d_tab64, cst, c->d_lin, c->d_share, st) != cudaSuccess) { s = MG_ECUDA; break; }
       share = c->d_share;
     }
+    own = own || (c->K >= 3 && !share);
     mg::pers::PJob& p = batch->job[batch->njobs++];
     p.share = share;
     p.rec = c->K == 2 ? j.mom_dev : c->d_prep;
@@ -187,24 +204,25 @@ extern "C" mg_status mg_sigmakin_batch(const mg_batch_job* jobs, int njobs, void
     int dev = 0, nsm = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mg::pers::k_me_persistent, mg::kMeThreads, 0) != cudaSuccess ||
+    const auto kernel = own ? mg::pers::k_me_persistent<true> : mg::pers::k_me_persistent<false>;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, mg::kMeThreads, 0) != cudaSuccess ||
         per_sm < 1)
       per_sm = 1;
     int64_t blocks = static_cast<int64_t>(nsm) * per_sm;
     if (blocks > batch->ntiles) blocks = batch->ntiles;
     if (cudaMemsetAsync(counter_dev, 0, sizeof(unsigned long long), st) != cudaSuccess) s = MG_ECUDA;
     if (s == MG_OK) {
-      mg::pers::k_me_persistent<<<static_cast<unsigned>(blocks), mg::kMeThreads, 0, st>>>(*batch, counter_dev);
+      kernel<<<static_cast<unsigned>(blocks), mg::kMeThreads, 0, st>>>(*batch, counter_dev);
       mg::note_launch();
       if (cudaGetLastError() != cudaSuccess) s = MG_ECUDA;
     }
-    for (int i = 0; i < njobs && s == MG_OK; ++i) {
-      const mg_batch_job& j = jobs[i];
-      if (j.nevt == 0 || j.ctx->K == 2) continue;
-      const double norm = 1.0 / (256.0 * mg::factorial(j.ctx->ng));
-      if (mg::fp64_hel_sum(j.ctx, j.nevt, pad_pg(j.nevt), norm, j.me_dev, st) != cudaSuccess)
-        s = MG_ECUDA;
-    }
+  }
+  for (int i = 0; i < njobs && s == MG_OK; ++i) {
+    const mg_batch_job& j = jobs[i];
+    if (j.nevt == 0 || j.ctx->K == 2) continue;
+    const double norm = 1.0 / (256.0 * mg::factorial(j.ctx->ng));
+    if (mg::fp64_hel_sum(j.ctx, j.nevt, pad_pg(j.nevt), norm, j.me_dev, st) != cudaSuccess)
+      s = MG_ECUDA;
   }
   delete batch;
   return s;

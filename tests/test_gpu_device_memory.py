@@ -24,10 +24,18 @@ SERVE = """
 srv = mg.Server(slots=1, max_nevt=1024)
 srv.wait(srv.submit("ggttggg", 5, 1024))
 """
+BATCH = """
+jobs = [(mg.Context(p), n) for p, n in ((3, 64), (2, 100), (1, 33), (0, 5))]
+jobs = [(c, torch.zeros(c.mom_count(n), dtype=torch.float64, device="cuda"), n,
+         torch.zeros(n, dtype=torch.float64, device="cuda")) for c, n in jobs]
+for c, mom, n, me in jobs:
+    c.rambo(3, n, 1500.0, mom)
+mg.sigmakin_batch(jobs)
+"""
 
 
-# 2.7 GB measured, 14.8 GB with a kernel of 50 KB of local memory per thread; the bound is twice the former
-@pytest.mark.parametrize("code,bound_mib", [(SERVE, 5500)], ids=["server"])
+# 2.7 GB measured, 14.7 GB with a kernel of 50 KB of local memory per thread; the bound is twice the former
+@pytest.mark.parametrize("code,bound_mib", [(SERVE, 5500), (BATCH, 5500)], ids=["server", "batch"])
 def test_device_memory(code, bound_mib):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
