@@ -319,13 +319,14 @@ mg_status mg_colour_flow(mg_process proc, int flow, int* order);
 #define MG_LAUNCH_TC_SYNC 64
 
 /* Time mg_sigmakin(precision) of nevt probe events (this context's process, fixed seed) for each
- * launch shape of the matrix-element kernel -- 32, 64 or 128 events per 128-thread block (the other
+ * launch shape that its kernels read and keep the fastest for this context and precision.  FP32 amplitudes
+ * (and MG_FP64_TCCOLOR of gg -> t tbar): 32, 64 or 128 events per 128-thread block (the other
  * threads of a block take further helicity combinations of the same events), grid dispatched
  * event-tile-major or helicity-tile-major, with and without MG_LAUNCH_UNROLLED where that kernel
  * exists, MG_LAUNCH_UNROLLED | MG_LAUNCH_FUSED, MG_LAUNCH_WARP and (MG_MIXED) MG_LAUNCH_WARP | MG_LAUNCH_TC_APART
- * -- then the fastest with MG_LAUNCH_DF_REDO (FP32 modes) or MG_LAUNCH_SHARED (MG_FP64) toggled, and for the
- * tensor-core colour modes with MG_LAUNCH_TC_SYNC toggled, and keep the fastest
- * for this context and precision.  cache_path (may be NULL): text file of
+ * -- then the fastest with MG_LAUNCH_DF_REDO toggled (FP32 modes).  FP64 amplitudes from gg -> t tbar g on: both grid
+ * orders, with MG_LAUNCH_SHARED.  The tensor-core colour modes: the fastest with MG_LAUNCH_TC_SYNC toggled.  MG_FP64
+ * of gg -> t tbar, and any mode with a top width, has one shape, which is timed and kept.  cache_path (may be NULL): text file of
  * "gpu|process|precision tile_ev slot_major flags ms" lines; an existing entry is used without timing,
  * a new result is appended.  *best_ms may be NULL.  Synchronous; allocates probe buffers; nevt >= 32. */
 mg_status mg_autotune(mg_ctx* ctx, mg_precision precision, int64_t nevt, const char* cache_path, double* best_ms);

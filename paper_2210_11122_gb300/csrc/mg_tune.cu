@@ -1,8 +1,8 @@
 // mg_tune.cu -- autotuner for the matrix-element launch shape, and CUDA-graph batches.
 //
 // Autotuner: for one context and precision, time mg_sigmakin on probe events for every launch
-// shape of the matrix-element kernel (events per block 32 / 64 / 128, the remaining threads of the
-// 128-thread block taking further gluon-helicity slots of the same events; grid dispatched event-
+// shape that the context's kernels read (FP32 amplitudes: events per block 32 / 64 / 128, the remaining threads of the
+// 128-thread block taking further gluon-helicity slots of the same events, and the kernel variants; grid dispatched event-
 // tile-major or slot-tile-major) and keep the fastest.  Results can be cached in a text file, one
 // line per (GPU, process, precision).
 //
@@ -125,17 +125,29 @@ extern "C" mg_status mg_autotune(mg_ctx* ctx, mg_precision precision, int64_t ne
     *out_ms = t;
     return r;
   };
-  const int tiles[3] = {32, 64, 128};
+  const int tiles[3] = {128, 64, 32};
   const bool fp32 = precision == MG_FP32_AMP || precision == MG_MIXED;
+  // Only shapes that differ are timed, or the file would keep the winner of noise: with a top width and for FP64
+  // gg -> t tbar there is one kernel, FP64 amplitudes of 3 to 5 gluons read the grid order only.  (Their shared items are
+  // kept: without them a call is slower at every size, 1.6 to 4.2 times, and the kernel makes the driver reserve 12 GB.)
+  const bool one = ctx->prm.wt != 0.0 || (precision == MG_FP64 && ctx->K == 2), order = !fp32 && ctx->K >= 3;
   const int nun = mg::me_static_available(ctx->K, fp32) && ctx->prm.wt == 0.0 ? 2 : 1;
   for (int un = 0; un < nun && rc == MG_OK; ++un)
-    for (int ti = 0; ti < 3 && rc == MG_OK; ++ti)
-      for (int sm = 0; sm < 2 && rc == MG_OK; ++sm) {
+    for (int ti = 0; ti < (one || order ? 1 : 3) && rc == MG_OK; ++ti)
+      for (int sm = 0; sm < (one ? 1 : 2) && rc == MG_OK; ++sm) {
         mg::MeShape s;
-        s.tile_ev = tiles[ti];
-        s.slot_major = sm != 0;
-        s.unrolled = nun == 2 ? un == 0 : true;
-        s.fused = false;
+        if (one || order) {
+          s = saved;
+          if (order && !one) {
+            s.slot_major = sm != 0;
+            s.shared = true;
+          }
+        } else {
+          s.tile_ev = tiles[ti];
+          s.slot_major = sm != 0;
+          s.unrolled = nun == 2 ? un == 0 : true;
+          s.fused = false;
+        }
         float t = 1e30f;
         rc = time_shape(s, &t);
         if (rc == MG_OK && t < best_t) { best_t = t; best = s; }
@@ -157,10 +169,9 @@ extern "C" mg_status mg_autotune(mg_ctx* ctx, mg_precision precision, int64_t ne
       if (rc == MG_OK && t < best_t) { best_t = t; best = s; }
     }
   }
-  if ((fp32 || precision == MG_FP64) && rc == MG_OK) {   // recomputation arithmetic / shared currents
+  if (fp32 && !one && rc == MG_OK) {   // recomputation arithmetic
     mg::MeShape s = best;
-    if (fp32) s.df_redo = !s.df_redo;
-    else s.shared = !s.shared;
+    s.df_redo = !s.df_redo;
     float t = 1e30f;
     rc = time_shape(s, &t);
     if (rc == MG_OK && t < best_t) { best_t = t; best = s; }

@@ -32,10 +32,13 @@ for c, mom, n, me in jobs:
     c.rambo(3, n, 1500.0, mom)
 mg.sigmakin_batch(jobs)
 """
+TUNE = """
+mg.Context(3).autotune(mg.MG_FP64, nevt=64)
+"""
 
 
 # 2.7 GB measured, 14.7 GB with a kernel of 50 KB of local memory per thread; the bound is twice the former
-@pytest.mark.parametrize("code,bound_mib", [(SERVE, 5500), (BATCH, 5500)], ids=["server", "batch"])
+@pytest.mark.parametrize("code,bound_mib", [(SERVE, 5500), (BATCH, 5500), (TUNE, 5500)], ids=["server", "batch", "autotune"])
 def test_device_memory(code, bound_mib):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
