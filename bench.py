@@ -94,9 +94,9 @@ def parse():
 ME_SOURCES = ("mg_me64.cuh", "mg_me64l.cuh", "mg_me64_k2.cuh", "mg_me64.cu", "mg_tables64.cpp", "mg_me_algebra.cuh")
 
 
-def profiled_traffic(kernel_files, profile_md, nevt):
-    """DRAM bytes of one launch scaled from a committed ncu summary, or None when the kernel sources
-    (hashed in the order given) have changed since the counters were taken."""
+def profiled_field(kernel_files, profile_md, field):
+    """A figure of a committed ncu summary, or None when the kernel sources (hashed in the order given) have
+    changed since the counters were taken."""
     import hashlib
     try:
         h = hashlib.sha256()
@@ -105,14 +105,20 @@ def profiled_traffic(kernel_files, profile_md, nevt):
         sha = h.hexdigest()[:16]
         fields = {}
         for line in open(profile_md):
-            if ":" in line and line.split(":")[0].strip() in ("source_sha256_16", "traffic_bytes_per_event"):
+            if ":" in line and line.split(":")[0].strip() in ("source_sha256_16", field):
                 k, v = line.split(":", 1)
                 fields[k.strip()] = v.split()[0]
         if fields.get("source_sha256_16") != sha:
             return None
-        return float(fields["traffic_bytes_per_event"]) * nevt
-    except (OSError, KeyError, ValueError):
+        return float(fields[field])
+    except (OSError, KeyError, ValueError, IndexError):
         return None
+
+
+def profiled_traffic(kernel_files, profile_md, nevt):
+    """DRAM bytes of one call scaled from a committed ncu summary (profiled_field)."""
+    per_event = profiled_field(kernel_files, profile_md, "traffic_bytes_per_event")
+    return None if per_event is None else per_event * nevt
 
 
 def config_of(args, nevt, extra=None):
@@ -308,17 +314,19 @@ def time_roofline(parts, me_ms):
 
 def fp64_roofline(model_flops, oracle_flops, nevt, me_ms, peak, traffic, kernel):
     """ALU roofline of the FP64 path on the FP64 pipe.  achieved counts the flops the kernels execute
-    (model_flops: ncu's counts of one call, from the committed profile); the oracle-count
+    (model_flops: ncu's counts of one call, from the committed profile; without them there is no achieved rate, the
+    flop model counting several times what runs); the oracle-count
     figures count the FP64 oracle's instrumented operations (plain recursion per helicity) for the same
     events in the same time, and count_ratio = oracle / executed flops per event."""
-    ach = model_flops * nevt / (me_ms * 1e-3)
-    r = {"bound": "alu", "achieved": ach / 1e12, "peak": peak / 1e12, "unit": "TFLOP/s", "frac": ach / peak,
-         "traffic": traffic, "kernel": kernel, "flops_per_event": model_flops,
+    ach = model_flops * nevt / (me_ms * 1e-3) if model_flops else None
+    r = {"bound": "alu", "achieved": ach / 1e12 if ach else None, "peak": peak / 1e12, "unit": "TFLOP/s",
+         "frac": ach / peak if ach else None, "traffic": traffic, "kernel": kernel, "flops_per_event": model_flops,
          "peak_source": "measured FP64 DFMA-chain microbenchmark (mg_measure_fma_peak) on this GPU"}
     if oracle_flops:
         ach_o = oracle_flops * nevt / (me_ms * 1e-3)
         r.update({"oracle_flops_per_event": oracle_flops, "oracle_count_achieved": ach_o / 1e12,
-                  "oracle_count_frac": ach_o / peak, "count_ratio": oracle_flops / model_flops})
+                  "oracle_count_frac": ach_o / peak,
+                  "count_ratio": oracle_flops / model_flops if model_flops else None})
     return r
 
 
@@ -328,14 +336,15 @@ def profile_for(process):
     return p if os.path.exists(p) else None
 
 
-def executed_fp64_flops(process):
-    """FP64 flops per event that one call executes, from the committed ncu summary (None without one)."""
-    p = profile_for(process)
-    if p:
-        for line in open(p):
-            if line.startswith("fp64_flops_per_event:"):
-                return float(line.split()[1])
-    return None
+def executed_fp64_flops(process, ngood, shared):
+    """FP64 flops per event that one call executes, from the committed ncu summary: None without one, after a
+    change of the kernel sources, and where the call is not the one captured (its good helicities, all but the
+    four vanishing ones of gg -> t tbar, and the shared items)."""
+    ng = WORKLOADS[process]["ng"]
+    if ngood != (12 if ng == 0 else 1 << (ng + 4)) or not (shared or ng == 0):
+        return None
+    csrc = os.path.join(ROOT, "paper_2210_11122_gb300", "csrc")
+    return profiled_field([os.path.join(csrc, f) for f in ME_SOURCES], profile_for(process) or "", "fp64_flops_per_event")
 
 
 # ------------------------------------------------------------------------------------------
@@ -434,11 +443,13 @@ class Leg:
             K = self.ng + 2
             kernel = ("k_me64_k2" if K == 2 else "k_event_prep + %sk_me64<%d> + k_hel_sum_rows"
                       % ("k_pass64 (per pass) + " if shared else "", K)) + " (one mg_sigmakin call)"
-            return fp64_roofline(executed_fp64_flops(self.process) or amp + col, oracle_flops, nev, me_ms, p64, traffic, kernel)
+            return fp64_roofline(executed_fp64_flops(self.process, ngood, shared), oracle_flops, nev, me_ms, p64, traffic,
+                                 kernel)
         if precision == mg.MG_FP64_TCCOLOR:
             # (the amplitudes of the FP64 call; its colour sums, here on the tensor cores, are a few per cent of its flops)
-            return time_roofline([("fp64", (executed_fp64_flops(self.process) or amp) * nev, p64, src64),
-                                  ("tensor_f16", colour_tc_flops(ncol, ngood) * nev, ptc, tc_src)], me_ms)
+            ex = executed_fp64_flops(self.process, ngood, self.shapes[name]["shared"])
+            return time_roofline(([("fp64", ex * nev, p64, src64)] if ex else []) +
+                                 [("tensor_f16", colour_tc_flops(ncol, ngood) * nev, ptc, tc_src)], me_ms)
         # FP32 amplitudes: the per-event FP64 record is the amplitude count with no good helicity
         rec64, _ = mg.flops_per_event(self.ng, [0] * len(mask), precision, flags)
         if precision == mg.MG_FP32_AMP:
