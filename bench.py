@@ -87,7 +87,55 @@ def parse():
                     help="jobs of the default run's graph-batch leg (the first requests of the serving trace)")
     ap.add_argument("--serve-requests", type=int, default=500,
                     help="requests of the default run's serving leg (the first ones of the 20,000-request trace)")
+    ap.add_argument("--details", default=None, metavar="FILE",
+                    help="write every measured figure of the default run to FILE (the printed line holds a summary)")
     return ap.parse_args()
+
+
+LINE_BYTES = 8192   # a reader that keeps a bounded tail of the output must still find the whole line
+
+
+def rounded(x):
+    """Numbers to six significant digits, in nested lists and dicts."""
+    if isinstance(x, float):
+        return float("%.6g" % x)
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    return [rounded(v) for v in x] if isinstance(x, list) else x
+
+
+def summary_line(full):
+    """The printed line of a full record: the headline's keys whole, of the other modes, processes and legs the rates,
+    times, roofline fractions and largest errors."""
+    def mode(m):
+        r = {"value": m["value"], "ms_per_step": m["ms_per_step"], "me_kernel_ms": m["me_kernel_ms"],
+             "frac": m["roofline"]["frac"]}
+        if "rel_err_vs_fp64" in m:
+            r["max_rel_err"] = m["rel_err_vs_fp64"]["max"]
+        return r
+
+    whole = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "clocks", "gpu_launches")
+    line = {k: full[k] for k in whole}
+    line["e2e"] = {k: v for k, v in full["e2e"].items() if k != "api"}
+    rest = {k: full[k] for k in ("me_kernel_ms", "wall_s", "nonconverged_events", "good_helicities", "roofline")}
+    rest["modes"] = {k: mode(v) for k, v in full["modes"].items()}
+    rest["processes"] = {p: dict({k: mode(v) for k, v in r["modes"].items()}, events_per_gpu=r["events_per_gpu"],
+                                 lhe_ms=r["epilogues"]["lhe_ms"], sde_ms=r["epilogues"]["sde_ms"])
+                         for p, r in full["processes"].items() if p != full["config"]["process"]}
+    rest["graph"] = {k: v for k, v in full["graph"].items() if k != "what"}
+    rest["cpu_baseline"] = full["cpu_baseline"]
+    rest["peaks"] = {k: v for k, v in full["peaks"].items() if k != "what"}
+    if full["graph_batch"]:
+        rest["graph_batch_ms"] = {k: v["ms"] for k, v in full["graph_batch"].items() if isinstance(v, dict)}
+    if full["serving"]:
+        rest["serving"] = {k: {f: v[f] for f in ("closed_loop_MEs_per_s", "p50_ms", "p99_ms")}
+                           for k, v in full["serving"].items() if isinstance(v, dict)}
+    line.update(rounded(rest))
+    for k in ("serving", "graph_batch_ms", "peaks", "processes"):   # (never reached by the default run)
+        if len(json.dumps(line)) > LINE_BYTES:
+            line.pop(k, None)
+    return line
 
 
 # sources of the FP64 slot kernels (body, algebra, dispatch): a committed traffic figure holds while their hash does
@@ -678,7 +726,10 @@ def run_ours(args):
                               "mg_measure_mma_peak: tcgen05.mma kind::f16 M128 N256 K16, exact integer result checked); "
                               "the tensor rooflines divide by the pool's measured bf16 peak (tensor_denominator_tflops)"},
             "gpu_launches": launches}
-    print(json.dumps(line))
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(line, f)
+    print(json.dumps(summary_line(line)))
     if world > 1:
         dist.destroy_process_group()
     return 0
