@@ -209,7 +209,7 @@ mg_status mg_flops_per_event_shape(mg_process proc, mg_precision precision, cons
  *     that device current); make that first call before any stream capture.
  *   - The library allocates nothing, but the CUDA driver itself may enlarge the context's
  *     per-thread local-memory reservation the first time a kernel with a large stack runs in the
- *     process (the five-gluon kernel keeps ~28 KB of local arrays per thread), which is a device
+ *     process (the five-gluon kernel keeps ~33 KB of local arrays per thread), which is a device
  *     allocation and a device-wide synchronisation made by the driver.  To keep that out of the
  *     caller's steady state, make one warm-up call per device and process at set-up. */
 mg_status mg_sigmakin_noalloc(mg_ctx* ctx, const double* mom_dev, int64_t nevt, double* me_dev, void* stream);
@@ -240,7 +240,9 @@ mg_status mg_sigmakin_noalloc(mg_ctx* ctx, const double* mom_dev, int64_t nevt, 
  * Every buffer holds nevt entries.  Zero top width only (MG_ENOTSUP otherwise).  The matrix elements come
  * from the FP64 algorithm that the context's MG_FP64 launch shape selects (with MG_LAUNCH_SHARED: the
  * shared items); at fixed coupling they equal mg_sigmakin(MG_FP64)'s up to rounding (the sums run over
- * helicities, there over linear gluon polarisations).
+ * helicities, there over linear gluon polarisations).  From gg -> t tbar g on a helicity's amplitude is a sum of
+ * those of the linear polarisations, so its rounding is relative to the event's largest amplitude: a strongly
+ * suppressed |M_h|^2 has the absolute accuracy of the event's sum, not the relative one.
  * Scratch: the amplitudes, the items shared by them and the sums of |J_sigma|^2 (events processed in chunks
  * that keep it within 2 GiB), owned by the context.  If no helicity mask exists yet, the call first
  * runs mg_hel_filter on its own first events. */
@@ -306,7 +308,9 @@ mg_status mg_colour_flow(mg_process proc, int flow, int* order);
  *                       (their currents, the quark line's row and column spinors and their products) is
  *                       computed once per helicity assignment of those gluons, by a few passes before the
  *                       matrix-element kernel, instead of once per gluon-helicity combination (the same
- *                       bits);
+ *                       bits).  Without it the kernel keeps a combination's items in local memory, with five
+ *                       gluons 50 KB per thread, for which the driver reserves 12 GB of device memory when the
+ *                       kernel first runs;
  *   MG_LAUNCH_TC_SYNC   the separate tensor-core colour pass (MG_FP64_TCCOLOR, and MG_MIXED where the jamps
  *                       are written out) on warp-level mma.sync instead of the default fifth-generation
  *                       tensor-core kernel (tcgen05.mma with the accumulators in tensor memory). */
@@ -437,7 +441,9 @@ typedef struct mg_server mg_server;
 
 void mg_serve_default_cfg(mg_serve_cfg* cfg);
 
-/* Device bytes a request of nevt events holds while in flight (momenta, MEs, scratch); host only. */
+/* Device bytes a request of nevt events holds while in flight (momenta, MEs, per-helicity sums, records, FP32
+ * jamps); host only.  The shared items and FP64 amplitudes of the FP64 modes are not counted: every slot's contexts
+ * hold them from creation (at most 2 GiB each; gg -> t tbar g g g in MG_FP64 on servers of at most 1,024 events: 20 MB). */
 int64_t mg_serve_footprint(mg_process proc, int64_t nevt, mg_precision precision);
 
 /* Create a server on the current device (allocates every slot up front).  cfg may be NULL. */

@@ -44,13 +44,14 @@ mg_status grow(double** buf, int64_t* cap, int64_t need) {
   return MG_OK;
 }
 
-// Flop model of the matrix-element kernel of mg_me2.cu for one event (FMA counted as 2 flops, a
-// complex multiply-add as 8): mirrors the kernel operation by operation.  One thread per gluon-
+// Flop model of the matrix elements by helicity for one event (FMA counted as 2 flops, a
+// complex multiply-add as 8): operation by operation the FP32 kernels and, without shared, the table kernel of mg_me2.cu;
+// with shared the same recursion with currents and prefixes formed once.  One thread per gluon-
 // helicity combination with a good helicity; per thread the gluon currents once, (gamma.J) v per
 // antitop helicity, a depth-first walk of the quark-line prefixes per top helicity, the jamps and
 // the colour sum per good helicity.  mask == NULL means every helicity is good.  This counts the
-// algorithm with every good helicity evaluated; the FP64 kernels evaluate one of each pair of flipped
-// helicities (hel_weight) and execute about half of it.
+// algorithm with every good helicity evaluated; the FP64 kernels of 3 to 5 gluons (mg_me64.cuh, mg_me64l.cuh) do less:
+// 0.33 / 0.21 / 0.14 of it by executed instructions.
 // warp_simt: the FP32 lane-group kernel's SIMT colour epilogue, which multiplies the full ncol x ncol matrix
 // into the jamps of all four helicities of a slot (4 ncol^2 + 4 ncol each, good or not) instead of the
 // packed triangle per good helicity.  warp: the FP32 lane-group kernel (any epilogue), which for 5 gluons

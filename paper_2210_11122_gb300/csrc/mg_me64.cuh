@@ -18,12 +18,14 @@
 // A flipped combination's |M|^2 equals the combination's (hel_weight), so gluon K-1 has helicity -1 throughout and
 // an item's helicity index leaves its bit out.
 //
-// Measured against carrying the prefixes of up to K-1 gluons (both on half of the combinations): gg->ttg FP64 12.13 vs
-// 14.48 ms per 524,288 events, LHE choices of gg->ttgg 9.35 vs 11.63 ms per 32,768, gg->ttggg + TC colour 8.60 vs
-// 12.37 ms per 2,049.
+// The helicity basis of this file is the path of partial helicity masks; with every helicity good the same scheme runs
+// over linear polarisations (mg_me64l.cuh).  Measured in this basis against carrying the prefixes of up to K-1 gluons, both
+// on half of the combinations: gg->ttg 12.13 vs 14.48 ms per 524,288 events, amplitudes of gg->ttggg 8.60 vs 12.37 ms
+// per 2,049; with 20 of 32 / 50 of 64 / 112 of 128 helicities good now 0.17 / 1.14 / 15.5 ms per 4,099 events of
+// gg->ttg / ttgg / ttggg (0.28 / 2.95 / 57.3 before).
 //
 // The combination may also build its own items in local memory (LOCAL, no buffer): the same functions, so the same
-// bits, at about three times the FP64 work.
+// bits, at about three times the FP64 work and, with 5 gluons, 50 KB of local memory per thread.
 #pragma once
 
 #include "mg_me_algebra.cuh"
@@ -332,8 +334,8 @@ __device__ __forceinline__ void signed_sums(cx<double>* a) {
 
 // Colour sum of the jamps A (overwritten) of one helicity.  4 and 5 gluons: in the basis of Tab64::blk, whose blocks of
 // at most 4 / 16 replace the full triangle of 24 / 120: 280 instead of 648 and 2,872 instead of 14,760 FP64
-// instructions, most of the slot kernel's work with 5 gluons before.  Measured: gg->ttggg FP64 31.7 vs 41.9 ms per
-// 8,192 events, gg->ttgg 2.64 vs 2.81 ms per 10,007.  With 3 gluons the blocks save nothing.
+// instructions, most of the slot kernel's work with 5 gluons before.  Measured in the helicity basis: gg->ttggg FP64
+// 31.7 vs 41.9 ms per 8,192 events, gg->ttgg 2.64 vs 2.81 ms per 10,007.  With 3 gluons the blocks save nothing.
 template <int K>
 __device__ __forceinline__ double colour_sum64(cx<double>* A, const Tab64* __restrict__ t, const double* __restrict__ ctri) {
   if constexpr (K < 4) {

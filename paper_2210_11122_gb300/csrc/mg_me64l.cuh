@@ -543,7 +543,7 @@ __device__ __forceinline__ double* amp_at(double* amp, int64_t e, int row, int c
 
 // A warp takes one top helicity pair of one combination (the all-gluon currents, which the pairs share, are items
 // of the last pass): a thread doing all four pairs made 4 times longer warps, of which gg->ttgg's 10,007 events are
-// 4.1 per sub-partition, so the busiest had 5; measured 2.81 vs 3.19 ms there, gg->ttggg + TC colour 7.60 vs 8.60 ms
+// 4.1 per sub-partition, so the busiest had 5; measured in the helicity basis 2.81 vs 3.19 ms there, gg->ttggg + TC colour 7.60 vs 8.60 ms
 // per 2,049 events, gg->ttg 12.05 vs 12.13 ms per 524,288.
 //
 // One thread of a block (32 events x 4 warps) on event tile `tile`, block `blk` < 2^(K-1) of the tile.

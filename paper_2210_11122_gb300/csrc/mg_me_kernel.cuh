@@ -19,7 +19,7 @@ namespace v2 {
 // weight 0), and the slot's weighted sum over its helicities of every |jamp|^2,
 // j2[(slot * ncol + sigma) * stride + e].
 // The work of one thread: event e, gluon-helicity slot `slot` with gluon helicities gc (bit g = helicity +1
-// of gluon g).  Called by k_me_gluonhel below and by the persistent multi-process kernel (mg_persist.cu).
+// of gluon g).
 template <int K, class T, bool PER_HEL, bool PREP, bool JOUT, bool LHE = false>
 __device__ __forceinline__ void me_slot(const double* __restrict__ mom, const T* __restrict__ rec, int64_t e, int slot,
                                         int gc, const Tables* __restrict__ tab, const uint32_t* __restrict__ mask,
