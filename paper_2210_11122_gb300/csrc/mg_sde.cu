@@ -85,6 +85,7 @@ struct TabL {
 struct Built {
   Tab tab;
   TabL lin;
+  bool ok;   // lin's capacities hold
   std::vector<std::string> keys;
 };
 
@@ -142,8 +143,9 @@ void build(int K, Built& out) {
   walk((1 << K) - 1, 0, 0);
 }
 
-// the linear polarisations' tables from the walk
-void build_lin(const Tab& t, TabL& o) {
+// the linear polarisations' tables from the walk; false if they do not fit (185 of 190 prefixes and 2,961 of 3,400 tasks with
+// five gluons)
+bool build_lin(const Tab& t, TabL& o) {
   const int K = t.K, full = (1 << K) - 1;
   std::memset(&o, 0xff, sizeof(o));   // -1: none
   auto size = [](int m) { return __builtin_popcount(m); };
@@ -160,15 +162,15 @@ void build_lin(const Tab& t, TabL& o) {
   o.q0 = take(0, 16);
   // prefixes of up to K-2 gluons and channels, replaying the walk; stack[d]: the prefix before the tree at depth d
   o.npre = 0;
-  int stack[6], tree[6], masks[6];
+  int stack[6], tree[6];
   stack[0] = -1;
   for (int i = 0; i < t.nop; ++i) {
     const int d = t.op_depth[i], n = t.op_node[i], c = t.op_ch[i];
     tree[d] = n;
-    masks[d] = t.op_mask[i];
     if (c < 0) {
       stack[d + 1] = -2;   // (K-1 gluons: not kept)
       if (size(t.op_mask[i]) <= K - 2) {
+        if (o.npre == TabL::kMaxPre) return false;
         const int p = o.npre++;
         o.pre_parent[p] = static_cast<int16_t>(stack[d]);
         o.pre_node[p] = static_cast<int16_t>(n);
@@ -200,7 +202,7 @@ void build_lin(const Tab& t, TabL& o) {
   o.pass0[0] = 0;
   auto tasks = [&](TabL::Task type, int i, int mask) {
     for (int gc = 0; gc <= full; ++gc)
-      if (!(gc & ~mask)) o.task[nt++] = static_cast<uint32_t>(type) | static_cast<uint32_t>(i) << 4 | static_cast<uint32_t>(gc) << 16;
+      if (!(gc & ~mask) && nt++ < TabL::kMaxTask) o.task[nt - 1] = static_cast<uint32_t>(type) | static_cast<uint32_t>(i) << 4 | static_cast<uint32_t>(gc) << 16;
   };
   // pass k: the trees of k+1 gluons; the prefixes of k gluons (their trees and parents come from earlier passes) and the
   // quark currents of those of k-1
@@ -216,6 +218,7 @@ void build_lin(const Tab& t, TabL& o) {
     }
     o.pass0[++o.npass] = nt;
   }
+  return nt <= TabL::kMaxTask;
 }
 
 const Built& built(int K) {
@@ -223,7 +226,7 @@ const Built& built(int K) {
   static std::once_flag once[6];
   std::call_once(once[K], [K] {
     build(K, b[K]);
-    build_lin(b[K].tab, b[K].lin);
+    b[K].ok = build_lin(b[K].tab, b[K].lin);
   });
   return b[K];
 }
@@ -710,8 +713,9 @@ extern "C" {
 
 mg_status mg_sde_channels(mg_process proc, int* nchannels) {
   if (proc < MG_GG_TT || proc > MG_GG_TTGGG || !nchannels) return MG_EINVAL;
-  *nchannels = mg::sde::built(mg::gluons_of(proc)).tab.nch;
-  return MG_OK;
+  const mg::sde::Built& b = mg::sde::built(mg::gluons_of(proc));
+  *nchannels = b.tab.nch;
+  return b.ok ? MG_OK : MG_ENOTSUP;
 }
 
 mg_status mg_sde_channel_key(mg_process proc, int channel, char* key, int keylen) {
@@ -735,6 +739,7 @@ mg_status mg_sde_weights(mg_ctx* ctx, const double* mom_dev, int64_t nevt, doubl
   }
   const int K = ctx->K;
   const mg::sde::Built& b = mg::sde::built(K);
+  if (!b.ok) return MG_ENOTSUP;
   if (!ctx->d_sdetab) {
     if (mg::dev_alloc(&ctx->d_sdetab, kLinOffset + sizeof(mg::sde::TabL)) != cudaSuccess) {
       cudaGetLastError();
