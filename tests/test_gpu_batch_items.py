@@ -99,3 +99,34 @@ def test_jobs_over_the_items_bound(env, jobs):
         mg.diag_fail_alloc(0)
         for c in ctxs:
             c.close()
+
+
+def test_persistent_graph_with_a_job_over_the_bound(env):
+    """The chunks of such a job are captured with the rest; contexts that have run nothing capture and replay."""
+    torch, mg, orc = env
+    sizes = [(3, 7008), (1, 65), (0, 33)]
+    ctxs = []
+    try:
+        def graph(persistent):
+            jobs = []
+            for i, (p, n) in enumerate(sizes):
+                c = mg.Context(p)
+                ctxs.append(c)
+                mom = torch.zeros(c.mom_count(n), dtype=torch.float64, device="cuda")
+                me = torch.full((n,), -1.0, dtype=torch.float64, device="cuda")
+                jobs.append((c, 60 + i, 0, n, SQRTS, mom, me, mg.MG_FP64))
+            return mg.GraphBatch(jobs, persistent=persistent), jobs
+        (ga, ja), (gb, jb) = graph(True), graph(False)
+        for _ in range(2):
+            ga.launch()
+            gb.launch()
+            torch.cuda.synchronize()
+            for a, b in zip(ja, jb):
+                assert torch.equal(a[6], b[6]) and bool((a[6] > 0).all())
+                a[6].zero_()
+                b[6].zero_()
+        ga.close()
+        gb.close()
+    finally:
+        for c in ctxs:
+            c.close()
