@@ -396,7 +396,9 @@ mg_status mg_graph_create(const mg_job* jobs, int njobs, mg_graph** out);
 
 /* As mg_graph_create; flags = MG_GRAPH_PERSISTENT (every job MG_FP64 with zero top width, at most 64 jobs,
  * else MG_ENOTSUP / MG_EINVAL): each job's mg_rambo_range and mg_hel_filter on its own branch, then the
- * matrix elements of all jobs in one persistent launch (mg_sigmakin_batch) and the helicity sums.
+ * matrix elements of all jobs in one persistent launch (mg_sigmakin_batch) and the helicity sums.  The default
+ * graph is usually the faster: its branches overlap the jobs' passes and run each process's own kernels (48 jobs,
+ * 354,144 events: 18.2 ms against 20.3); the persistent launch pays without a graph, for many small jobs.
  * mg_graph_update, _launch, _nodes and _destroy apply unchanged. */
 mg_status mg_graph_create_ex(const mg_job* jobs, int njobs, int flags, mg_graph** out);
 
